@@ -519,7 +519,7 @@ int scalp_init(scalp_ctx **out, const scalp_image *image, const scalp_contour *c
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) dev = 0;
     a.map_cap = (params->global_walk & 1) ? 0 : assign_map_capacity(dev);
-    a.prune = (params->global_walk & 2) ? 0 : 1;
+    a.prune = (params->global_walk & 2) || !bound_valid(H, W, a.lam, a.ms2) ? 0 : 1;
     c->smem = assign_smem_bytes(a.map_cap);
     int rc = cuda_check(c, assign_configure(params->storage), "configure kernel");
     if (rc == SCALP_OK) rc = cuda_check(c, srgb_table(&a.lut, c->st), "transfer-function table");
@@ -1451,7 +1451,7 @@ int scalp_batch_iterate(scalp_batch *b, int32_t n)
         const unsigned flags = capturing ? cudaEventRecordExternal : cudaEventRecordDefault;
         for (int i = 0; i < iters; ++i) {
             if (b->profiling) cudaEventRecordWithFlags(b->ev[2 * i], b->st, flags);
-            launch_assign_batch(b->bargs, b->storage, b->total_tiles, b->smem, b->st, pdl);
+            launch_assign_batch(b->bargs, b->storage, b->ctx[0]->a.count_samples != 0, b->total_tiles, b->smem, b->st, pdl);
             if (b->profiling) cudaEventRecordWithFlags(b->ev[2 * i + 1], b->st, flags);
             launch_batch_update(b->bargs, b->total_clusters, b->total_fill, b->st, pdl,
                                 capturing ? b->it_side : nullptr, b->it_fork, b->it_join);

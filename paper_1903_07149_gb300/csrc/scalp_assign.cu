@@ -73,18 +73,18 @@ int assign_map_capacity(int device)
     return cap > 0 ? (int)cap : 0;
 }
 
-template <typename T>
+template <typename T, bool COUNT>
 __global__ void __launch_bounds__(ASSIGN_THREADS, ASSIGN_CTAS_PER_SM) k_assign(SolveArgs a)
 {
     pdl_wait();
     pdl_release();
     extern __shared__ __align__(16) unsigned char smem[];
-    assign_tile<T>(a, blockIdx.x, smem);
+    assign_tile<T, false, COUNT>(a, blockIdx.x, smem);
 }
 
 // All tiles of all images of a batch in one launch: block g is tile
 // g - tile_base[i] of image i, tile_base being the prefix of tile counts.
-template <typename T>
+template <typename T, bool COUNT>
 __global__ void __launch_bounds__(ASSIGN_THREADS, ASSIGN_CTAS_PER_SM) k_assign_batch(BatchArgs b)
 {
     pdl_wait();
@@ -92,23 +92,51 @@ __global__ void __launch_bounds__(ASSIGN_THREADS, ASSIGN_CTAS_PER_SM) k_assign_b
     extern __shared__ __align__(16) unsigned char smem[];
     const int g = blockIdx.x;
     const int i = batch_find(b.tile_base, b.count, g);
-    assign_tile<T, true>(b.args[i], g - b.tile_base[i], smem);
+    assign_tile<T, true, COUNT>(b.args[i], g - b.tile_base[i], smem);
+}
+
+template <typename T, bool COUNT>
+static void launch_assign_as(const SolveArgs &a, size_t smem_bytes, cudaStream_t st, bool pdl)
+{
+    pdl_launch(pdl, k_assign<T, COUNT>, dim3(a.n_tx * a.n_ty), dim3(ASSIGN_THREADS), smem_bytes, st, a);
 }
 
 void launch_assign(const SolveArgs &a, int storage, size_t smem_bytes, cudaStream_t st, bool pdl)
 {
-    const dim3 grid(a.n_tx * a.n_ty), block(ASSIGN_THREADS);
-    if (storage == 0) pdl_launch(pdl, k_assign<float4>, grid, block, smem_bytes, st, a);
-    else pdl_launch(pdl, k_assign<uint2>, grid, block, smem_bytes, st, a);
+    if (storage == 0) {
+        if (a.count_samples) launch_assign_as<float4, true>(a, smem_bytes, st, pdl);
+        else launch_assign_as<float4, false>(a, smem_bytes, st, pdl);
+    } else {
+        if (a.count_samples) launch_assign_as<uint2, true>(a, smem_bytes, st, pdl);
+        else launch_assign_as<uint2, false>(a, smem_bytes, st, pdl);
+    }
 }
 
-void launch_assign_batch(const BatchArgs &b, int storage, int total_tiles, size_t smem_bytes,
+template <typename T, bool COUNT>
+static void launch_assign_batch_as(const BatchArgs &b, int total_tiles, size_t smem_bytes, cudaStream_t st, bool pdl)
+{
+    pdl_launch(pdl, k_assign_batch<T, COUNT>, dim3(total_tiles), dim3(ASSIGN_THREADS), smem_bytes, st, b);
+}
+
+void launch_assign_batch(const BatchArgs &b, int storage, bool count, int total_tiles, size_t smem_bytes,
                          cudaStream_t st, bool pdl)
 {
     if (total_tiles <= 0) return;
-    const dim3 grid(total_tiles), block(ASSIGN_THREADS);
-    if (storage == 0) pdl_launch(pdl, k_assign_batch<float4>, grid, block, smem_bytes, st, b);
-    else pdl_launch(pdl, k_assign_batch<uint2>, grid, block, smem_bytes, st, b);
+    if (storage == 0) {
+        if (count) launch_assign_batch_as<float4, true>(b, total_tiles, smem_bytes, st, pdl);
+        else launch_assign_batch_as<float4, false>(b, total_tiles, smem_bytes, st, pdl);
+    } else {
+        if (count) launch_assign_batch_as<uint2, true>(b, total_tiles, smem_bytes, st, pdl);
+        else launch_assign_batch_as<uint2, false>(b, total_tiles, smem_bytes, st, pdl);
+    }
+}
+
+// Whether the pruning bound's error estimate holds (scalp_assign_tile.cuh):
+// coordinates exact in FP32, and lam and m^2/r^2 far enough from both ends of
+// the FP32 range that no product under- or overflows where D would not.
+bool bound_valid(int H, int W, float lam, float ms2)
+{
+    return std::max(H, W) <= (1 << 24) && ms2 >= 1e-12f && ms2 <= 1e12f && (lam == 0.0f || lam >= 1e-12f);
 }
 
 // The limit is a property of the kernel, shared by every context on the
@@ -122,14 +150,23 @@ static cudaError_t configure(const void *f)
                                 (int)assign_smem_bytes(assign_map_capacity(dev)));
 }
 
+// (the kernels with and without counting)
+template <typename T>
+static cudaError_t configure_pair(bool batch)
+{
+    const cudaError_t e = configure(batch ? (const void *)k_assign_batch<T, false> : (const void *)k_assign<T, false>);
+    if (e != cudaSuccess) return e;
+    return configure(batch ? (const void *)k_assign_batch<T, true> : (const void *)k_assign<T, true>);
+}
+
 cudaError_t assign_batch_configure(int storage)
 {
-    return configure(storage == 0 ? (const void *)k_assign_batch<float4> : (const void *)k_assign_batch<uint2>);
+    return storage == 0 ? configure_pair<float4>(true) : configure_pair<uint2>(true);
 }
 
 cudaError_t assign_configure(int storage)
 {
-    return configure(storage == 0 ? (const void *)k_assign<float4> : (const void *)k_assign<uint2>);
+    return storage == 0 ? configure_pair<float4>(false) : configure_pair<uint2>(false);
 }
 
 }  // namespace scalp

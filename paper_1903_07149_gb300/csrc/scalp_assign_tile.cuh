@@ -64,22 +64,22 @@ __device__ __forceinline__ int path_sums_map(uint32_t map, int bw, int bx0, int 
 // per-candidate records follow, sized for the tile's own candidate count, and
 // the distance maps fill the rest (a tile with few candidates has more room).
 __host__ __device__ constexpr size_t align16(size_t x) { return (x + 15) & ~(size_t)15; }
+constexpr int ASSIGN_QUEUE = 160;  // pairs a warp's queue holds (pass 2)
 struct AssignSmem {
     static constexpr size_t best = 0;
-    static constexpr size_t prev = align16(best + TILE_PIXELS * sizeof(unsigned long long));
-    static constexpr size_t queue = align16(prev + TILE_PIXELS);
-    static constexpr size_t misc = align16(queue + (ASSIGN_THREADS / 32) * 64 * sizeof(uint32_t));
+    static constexpr size_t queue = align16(best + TILE_PIXELS * sizeof(unsigned long long));
+    static constexpr size_t misc = align16(queue + (ASSIGN_THREADS / 32) * ASSIGN_QUEUE * sizeof(uint16_t));
     static constexpr size_t records = align16(misc + 64);
 };
-static_assert(AssignSmem::prev % 16 == 0 && AssignSmem::queue % 16 == 0 &&
-                  AssignSmem::misc % 16 == 0 && AssignSmem::records % 16 == 0,
+static_assert(AssignSmem::queue % 16 == 0 && AssignSmem::misc % 16 == 0 && AssignSmem::records % 16 == 0,
               "shared-memory sections aligned");
 // Per candidate (rank c): three 16-byte records the walk reads,
-//   rec0 = (xa, ya, w | h << 8, 0)                   its rectangle
+//   rec0 = (columns, rows, K bits, g_y bits)         its rectangle as a mask of
+//          the tile's columns and one of its rows; terms of the bound
 //   rec1 = (ex, ey, xk bits, yk bits)                endpoint, X_k
 //   rec2 = (bx0, by0, pitch, map byte offset, or -1: walk the plane)
 // the map box for the build, box = (bx0, by0, pitch, 32-bit reciprocal of
-// the pitch), the colour C_k, col = (l_k, a_k, b_k, 0), the cluster index
+// the pitch), the colour C_k, col = (l_k, a_k, b_k, g_x), the cluster index
 // cid, the box area and the prefixes mfirst and cfirst of the map layout.
 struct TileLayout {
     uint32_t rec0, rec1, rec2, box, col, cid, area, mfirst, cfirst, maps;
@@ -105,7 +105,6 @@ __host__ __device__ constexpr int extra_map_pairs(int n)
 {
     return (int)((tile_layout(MAX_TILE_CANDIDATES).maps - tile_layout(n).maps) / 8u);
 }
-static_assert(MAX_TILE_CANDIDATES < 255, "slots are bytes; 0xff is none");
 static_assert(TILE_PIXELS <= 1024 && MAX_TILE_CANDIDATES < (1 << 21), "queued pairs pack into 32 bits");
 static_assert(MAX_TILE_CANDIDATES % 32 == 0, "the scans give each lane whole candidates");
 
@@ -121,15 +120,31 @@ __device__ __forceinline__ int find_slot(const int *cid, int cnt, int k)
     return lo < cnt && cid[lo] == k ? lo : -1;
 }
 
-// A lower bound of D (Eq. 3) from the pixel's own colour distance and the
-// spatial term, in FP32 such that it never exceeds the D scalp_distance()
-// computes from the same dcp and ds: there dcol = lam*dcp + (1-lam)*avg is a
-// rounded sum of non-negative terms, so dcol >= fl(lam*dcp); dcon =
-// 1 + gamma*avg_w >= 1; D = fl(dcol*dcon + fl(ms2*ds)) >= fl(fl(lam*dcp) +
-// fl(ms2*ds)), rounding being monotone.  (lam in [0, 1], gamma >= 0.)
-__device__ __forceinline__ float distance_lower_bound(float dcp, float lam, float ms2, float ds)
+// The pruning bound.  With q = lam |v - c|^2 + m^2/r^2 |X - X_k|^2 (v, X the
+// pixel's own sample and place), the D that scalp_distance() computes is at
+// least q up to rounding: the path term of Eq. 1 and the contour term of
+// Eq. 2 are non-negative and every factor is at least one.  Expanded,
+//   q = P(pixel) + K(cluster) + f . g,
+//   P = lam |v|^2 + m^2/r^2 |X|^2,  f = (-2 lam v, X),
+//   K = lam |c|^2 + m^2/r^2 |X_k|^2,  g = (c, -2 m^2/r^2 X_k)
+// with X and X_k from the tile's corner: five multiply-adds per pair, against
+// fourteen operations for the two squared distances.  P and K are scaled by
+// 1 - 2^-17 here.  With u = 2^-24, the rounding of K (8 u K), of f and g (3 u
+// |f . g|) and of the chain (10 u (P + K)) adds up to less than 30 u (P + K)
+// as |f . g| <= P + K, so P' + K' + f . g stays below q - 98 u (P + K); the
+// computed D is above q - 20 u (P + K) (at most ten roundings).  A pair whose
+// bound exceeds the pixel's pass-1 D raised by 2^-20 (bound_threshold()
+// subtracts P') therefore has a larger D: it can neither win nor tie.  The
+// host turns the pruning off where these estimates do not hold (bound_valid()
+// in scalp_assign.cu: products that could leave the FP32 range, coordinates
+// above 2^24).
+constexpr float BOUND_SCALE = 1.0f - 1.0f / 131072.0f;
+
+// What f . g + K' must exceed for the pair to lose; NaN (no pair loses) for a
+// pixel without a pass-1 D, or with one near the end of the FP32 range.
+__device__ __forceinline__ float bound_threshold(float D, float P)
 {
-    return __fadd_rn(__fmul_rn(lam, dcp), __fmul_rn(ms2, ds));
+    return D < 1e30f ? fmaf(D, 1.0f + 1.0f / 1048576.0f, -BOUND_SCALE * P) : __int_as_float(0x7fffffff);
 }
 
 __device__ __forceinline__ unsigned long long pack_best(float D, int slot)
@@ -193,7 +208,9 @@ __device__ __forceinline__ int warp_scan_maps(const int *area, int *mfirst, int 
 // rectangle; each warp owns 64 pixels of the tile (two blocks of 8 x 4).
 // PREFETCH_TILE: the tile's plane rows are first asked into L2 (for batches,
 // whose planes outgrow L2; an image whose plane stays in L2 only pays for it).
-template <typename T, bool PREFETCH_TILE = false>
+// COUNT: the work is counted when a.count_samples asks for it (the counting
+// code costs the walks and the bound even when it is off).
+template <typename T, bool PREFETCH_TILE = false, bool COUNT = true>
 __device__ __forceinline__ void assign_tile(const SolveArgs &a, int tile, unsigned char *smem)
 {
     constexpr int THREADS = ASSIGN_THREADS;
@@ -208,7 +225,6 @@ __device__ __forceinline__ void assign_tile(const SolveArgs &a, int tile, unsign
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
     unsigned long long *best = reinterpret_cast<unsigned long long *>(smem + AssignSmem::best);
-    unsigned char *prev_slot = smem + AssignSmem::prev;
     int *misc = reinterpret_cast<int *>(smem + AssignSmem::misc);
 
     // this thread's pixels: block (warp * PIX_PER_THREAD + j) of the tile
@@ -267,6 +283,15 @@ __device__ __forceinline__ void assign_tile(const SolveArgs &a, int tile, unsign
         my_pixel(j, px, py);
         prev_lab[j] = fast && px < a.W && py < a.H ? a.labels[(long long)py * a.W + px] : -1;
     }
+    // the samples of this thread's pixels
+    const auto load_own = [&](T (&own)[PIX_PER_THREAD]) {
+#pragma unroll
+        for (int j = 0; j < PIX_PER_THREAD; ++j) {
+            int px, py;
+            my_pixel(j, px, py);
+            own[j] = px < a.W && py < a.H ? __ldg(plane + (long long)py * a.pitch + px) : T{};
+        }
+    };
     if (tid == 0) {
         misc[4] = 0;  // path samples and pairs (counting on)
         misc[5] = 0;
@@ -278,16 +303,23 @@ __device__ __forceinline__ void assign_tile(const SolveArgs &a, int tile, unsign
         const int xa = max(cd.xlo, x0), xb = min(min(cd.xhi, x0 + TILE_X - 1), a.W - 1);
         const int ya = max(cd.ylo, y0), yb = min(min(cd.yhi, y0 + TILE_Y - 1), a.H - 1);
         const int w = max(xb - xa + 1, 0), h = max(yb - ya + 1, 0);
-        rec0[rank] = make_int4(xa, ya, w | (h << 8), 0);
+        static_assert(TILE_X == 32 && TILE_Y == 32, "a rectangle is two 32-bit masks");
+        const bool some = w > 0 && h > 0;
+        const float kx = cd.xk - (float)x0, ky = cd.yk - (float)y0;
+        const float K = BOUND_SCALE * fmaf(a.lam, fmaf(cd.L, cd.L, fmaf(cd.a, cd.a, cd.b * cd.b)),
+                                           a.ms2 * fmaf(kx, kx, ky * ky));
+        rec0[rank] = make_int4(some ? (int)((0xffffffffu >> (32 - w)) << (xa - x0)) : 0,
+                               some ? (int)((0xffffffffu >> (32 - h)) << (ya - y0)) : 0, __float_as_int(K),
+                               __float_as_int(-2.0f * a.ms2 * ky));
         rec1[rank] = make_int4(cd.ex, cd.ey, __float_as_int(cd.xk), __float_as_int(cd.yk));
-        col[rank] = make_float4(cd.L, cd.a, cd.b, 0.f);
+        col[rank] = make_float4(cd.L, cd.a, cd.b, -2.0f * a.ms2 * kx);
         // map box: the rectangle and the endpoint (both inside the image).
         // Rows are padded to a pitch = 4 (mod 8) pairs: the walks of a warp
         // then spread over the shared-memory banks (neighbouring rows start
         // 8 banks apart); 32-bit reciprocal of the pitch for the build.
         int bx0 = 0, by0 = 0, pitch = 1;
         long long n = 0;
-        if (w > 0 && h > 0) {
+        if (some) {
             bx0 = min(xa, cd.ex);
             by0 = min(ya, cd.ey);
             const int bw = max(xb, cd.ex) - bx0 + 1;
@@ -352,26 +384,24 @@ __device__ __forceinline__ void assign_tile(const SolveArgs &a, int tile, unsign
     __syncthreads();
 
     // each pixel's previous label, as a candidate slot when the pixel lies in
-    // that candidate's rectangle (0xff otherwise): pass 1 below evaluates it
+    // that candidate's rectangle (-1 otherwise): pass 1 below evaluates it
     // first, pass 2 skips it
-    if (fast) {
+    int slot[PIX_PER_THREAD];
 #pragma unroll
-        for (int j = 0; j < PIX_PER_THREAD; ++j) {
-            int px, py;
-            my_pixel(j, px, py);
-            int c = prev_lab[j] >= 0 ? find_slot(cid, cnt, prev_lab[j]) : -1;
-            if (c >= 0) {
-                const int4 r0 = rec0[c];
-                if (px < r0.x || px >= r0.x + (r0.z & 0xff) || py < r0.y || py >= r0.y + ((r0.z >> 8) & 0xff))
-                    c = -1;
-            }
-            prev_slot[(py - y0) * TILE_X + (px - x0)] = (unsigned char)(c >= 0 ? c : 0xff);
+    for (int j = 0; j < PIX_PER_THREAD; ++j) {
+        int px, py;
+        my_pixel(j, px, py);
+        int c = prev_lab[j] >= 0 ? find_slot(cid, cnt, prev_lab[j]) : -1;
+        if (c >= 0) {
+            const int4 r0 = rec0[c];
+            if (!(((unsigned)r0.x >> (px - x0)) & ((unsigned)r0.y >> (py - y0)) & 1u)) c = -1;
         }
+        slot[j] = c;
     }
 
     // the distance maps of the candidates whose boxes fit: entries [0, used)
-    // hold the leading candidates' boxes back to back, row-major; the
-    // padding columns of a row are left unwritten (no walk reads them)
+    // hold the leading candidates' boxes back to back, row-major (no walk reads
+    // the padding columns of a row)
     const int used = fast ? misc[2] : 0;
     if (fast) {
         if (tid < cnt) {
@@ -380,15 +410,17 @@ __device__ __forceinline__ void assign_tile(const SolveArgs &a, int tile, unsign
             rec2[tid] = make_int4(b.x, b.y, b.z, mapped ? mfirst[tid] * (int)sizeof(float2) : -1);
         }
         // warps take the chunks in turn; within one the candidate is uniform
-        // and the lanes read consecutive entries (coalesced plane rows)
+        // and the lanes read consecutive entries (coalesced plane rows).  No
+        // branch per entry: a padding column reads its row's last sample and
+        // an entry past the box the last one, and only the latter's store is
+        // left out (the padding is inside the box's own part of the buffer).
         const int n_chunks = cfirst[cnt];
         int c = 0;
         for (int g = warp; g < n_chunks; g += WARPS) {
             while (g >= cfirst[c + 1]) ++c;
             const int4 b = box[c];
-            // unpadded width: from the rectangle's right edge and e_k
-            const int4 r0 = rec0[c];
-            const int bw = max(r0.x + (r0.z & 0xff) - 1, rec1[c].x) - b.x + 1;
+            // last unpadded column: the rectangle's right edge or e_k
+            const int last = max(x0 + 31 - __clz(rec0[c].x), rec1[c].x) - b.x;
             const float4 ck = col[c];
             const int m0 = mfirst[c];
             const int n_le = mfirst[c + 1] - m0;
@@ -399,23 +431,19 @@ __device__ __forceinline__ void assign_tile(const SolveArgs &a, int tile, unsign
             const T *__restrict__ pbox = plane + (long long)b.y * a.pitch + b.x;
             float2 *mrow = maps + (m0 + le0);
             T v[BUILD_UNROLL];  // raw samples: all loads issue before any use
-            bool ok[BUILD_UNROLL];
 #pragma unroll
             for (int u = 0; u < BUILD_UNROLL; ++u) {
-                const int le = le0 + u * 32;
+                const int le = min(le0 + u * 32, n_le - 1);
                 // a mapped box has pitch >= 4 and le * pitch < 2^32, so the
                 // 32-bit reciprocal gives the exact row
                 const int row = (int)__umulhi((unsigned)le, (unsigned)b.w);
-                const int cx = le - row * b.z;
-                ok[u] = le < n_le && cx < bw;
-                if (ok[u]) v[u] = __ldg(pbox + (row * a.pitch + cx));
+                v[u] = __ldg(pbox + (row * a.pitch + min(le - row * b.z, last)));
             }
 #pragma unroll
             for (int u = 0; u < BUILD_UNROLL; ++u) {
-                if (ok[u]) {
-                    const float4 q = sample_value(v[u]);
-                    mrow[u * 32] = make_float2(colour_dist(q, ck.x, ck.y, ck.z), q.w);
-                }
+                const float4 q = sample_value(v[u]);
+                const float2 pair = make_float2(colour_dist(q, ck.x, ck.y, ck.z), q.w);
+                if (le0 + u * 32 < n_le) mrow[u * 32] = pair;
             }
         }
     }
@@ -453,7 +481,7 @@ __device__ __forceinline__ void assign_tile(const SolveArgs &a, int tile, unsign
         return fmaf(ddx, ddx, ddy * ddy);
     };
     auto count_pair = [&](int len) {
-        if (a.count_samples) {
+        if (COUNT && a.count_samples) {
             atomicAdd(tile_samples, (unsigned)len);
             atomicAdd(tile_samples + 1, 1u);
         }
@@ -472,83 +500,125 @@ __device__ __forceinline__ void assign_tile(const SolveArgs &a, int tile, unsign
         for (int j = 0; j < PIX_PER_THREAD; ++j) {
             int px, py;
             my_pixel(j, px, py);
-            const int pix = (py - y0) * TILE_X + (px - x0);
-            const int c = prev_slot[pix];
-            if (c != 0xff) {
+            int c = slot[0];
+#pragma unroll
+            for (int i = 1; i < PIX_PER_THREAD; ++i)  // (registers: constant indices)
+                if (i == j) c = slot[i];
+            if (c >= 0) {
                 const int4 r1 = rec1[c], r2 = rec2[c];
                 int len;
                 const float D = pair_distance(px, py, c, r1, r2, own_distance(px, py, c, r2), spatial(px, py, r1),
                                               &len);
-                atomicMin(&best[pix], pack_best(D, c));
+                best[(py - y0) * TILE_X + (px - x0)] = pack_best(D, c);  // (the pixel's first D)
 #pragma unroll
-                for (int i = 0; i < PIX_PER_THREAD; ++i)  // (registers: constant indices)
+                for (int i = 0; i < PIX_PER_THREAD; ++i)
                     if (i == j) dprev[i] = D;
                 count_pair(len);
             }
         }
+        __syncwarp();  // the D's before the warp's other lanes lower them
 
         // Pass 2: each warp checks its own pixels against every other
-        // candidate whose rectangle holds them.  A surviving pair goes to the
-        // warp's queue (slot << 10 | tile pixel); each time 32 are queued the
-        // warp walks them, one per lane, and the last few at the end.  (A
-        // barrier before the walks, to share them among the warps, cost more
-        // than the uneven loads it evens out.)
-        const auto walk_queued = [&](uint32_t e) {
-            const int pix = (int)(e & 1023u), c = (int)(e >> 10);
-            const int qx = x0 + (pix & (TILE_X - 1)), qy = y0 + (pix / TILE_X);
-            const int4 r1 = rec1[c], r2 = rec2[c];
-            int len;
-            const float D = pair_distance(qx, qy, c, r1, r2, own_distance(qx, qy, c, r2), spatial(qx, qy, r1), &len);
-            atomicMin(&best[pix], pack_best(D, c));
-            count_pair(len);
-        };
-        uint32_t *wq = reinterpret_cast<uint32_t *>(smem + AssignSmem::queue) + warp * 64;
-        const unsigned lanes_below = (1u << lane) - 1u;
-        int queued = 0;  // warp-uniform
-        for (int c = 0; c < cnt; ++c) {
-            const int4 r0 = rec0[c];
-            const unsigned rw = (unsigned)(r0.z & 0xff), rh = (unsigned)((r0.z >> 8) & 0xff);
-            bool in[PIX_PER_THREAD];
-            bool any = false;
+        // candidate whose rectangle holds them, and queues the surviving
+        // pairs (slot << 6 | block << 5 | lane); then it walks the queue 32
+        // pairs at a time, one per lane.  (A barrier before the walks, to
+        // share them among the warps, cost more than the uneven loads it
+        // evens out.)  The pixels' samples are at hand only while the queue
+        // fills: held across the walks as well they spill registers (FP32, HD
+        // 140.0 us a launch against 134.7).
+        static_assert(WARPS % (TILE_X / WARP_BLOCK_X) == 0, "the warp's blocks lie in one column of blocks");
+        static_assert(PIX_PER_THREAD == 2 && MAX_TILE_CANDIDATES <= 1024, "queued pairs pack into 16 bits");
+        constexpr int ROW_STEP = WARPS / (TILE_X / WARP_BLOCK_X) * WARP_BLOCK_Y;  // block 1 lies this far below block 0
+        int px, py;
+        my_pixel(0, px, py);
+        const int bx = px - lane % WARP_BLOCK_X, by = py - lane / WARP_BLOCK_X;
+        uint16_t *wq = reinterpret_cast<uint16_t *>(smem + AssignSmem::queue) + warp * ASSIGN_QUEUE;
+        int queued = 0, c0 = -32;                    // warp-uniform, as all that follows
+        unsigned meets[PIX_PER_THREAD] = {}, any = 0;  // candidates c0 + bit left, per block and over both
+        for (bool more = true; more;) {
+            // the pixels' side of the bound
+            float fL[PIX_PER_THREAD], fa[PIX_PER_THREAD], fb[PIX_PER_THREAD], thr[PIX_PER_THREAD];
+            const float X = (float)(px - x0), Y = (float)(py - y0);
+            {
+                T own[PIX_PER_THREAD];
+                load_own(own);
 #pragma unroll
-            for (int j = 0; j < PIX_PER_THREAD; ++j) {
-                int px, py;
-                my_pixel(j, px, py);
-                // (a pixel of the rectangle lies in the image)
-                in[j] = (unsigned)(px - r0.x) < rw && (unsigned)(py - r0.y) < rh &&
-                        prev_slot[(py - y0) * TILE_X + (px - x0)] != c;
-                any = any || in[j];
+                for (int j = 0; j < PIX_PER_THREAD; ++j) {
+                    const float4 v = sample_value(own[j]);
+                    const float Yj = Y + (float)(j * ROW_STEP);
+                    thr[j] = a.prune ? bound_threshold(dprev[j], fmaf(a.lam, fmaf(v.x, v.x, fmaf(v.y, v.y, v.z * v.z)),
+                                                                      a.ms2 * fmaf(X, X, Yj * Yj)))
+                                     : __int_as_float(0x7fffffff);
+                    fL[j] = -2.0f * a.lam * v.x;
+                    fa[j] = -2.0f * a.lam * v.y;
+                    fb[j] = -2.0f * a.lam * v.z;
+                }
             }
-            if (!__any_sync(0xffffffffu, any)) continue;
-            const int4 r1 = rec1[c], r2 = rec2[c];
+            const unsigned lanes_below = (1u << lane) - 1u;
+            while (queued <= ASSIGN_QUEUE - 64) {
+                if (!any) {
+                    // the next 32 candidates: which of their rectangles meet
+                    // each of the warp's blocks, one candidate per lane
+                    c0 += 32;
+                    more = c0 < cnt;
+                    if (!more) break;
+                    const int4 r0 = c0 + lane < cnt ? rec0[c0 + lane] : make_int4(0, 0, 0, 0);
+                    const bool mx = ((unsigned)r0.x >> (bx - x0)) & ((1u << WARP_BLOCK_X) - 1u);
 #pragma unroll
-            for (int j = 0; j < PIX_PER_THREAD; ++j) {
-                int px, py;
-                my_pixel(j, px, py);
-                bool keep = false;
-                if (in[j]) {
-                    const float dcp = own_distance(px, py, c, r2);
-                    keep = !a.prune || !(distance_lower_bound(dcp, a.lam, a.ms2, spatial(px, py, r1)) > dprev[j]);
-                    // a pair that cannot win is not walked (counted as the method's work)
-                    if (!keep) count_pair(max(abs(px - r1.x), abs(py - r1.y)) + 1);
+                    for (int j = 0; j < PIX_PER_THREAD; ++j) {
+                        const bool my = ((unsigned)r0.y >> (by - y0 + j * ROW_STEP)) & ((1u << WARP_BLOCK_Y) - 1u);
+                        meets[j] = __ballot_sync(0xffffffffu, mx && my);
+                        any |= meets[j];
+                    }
+                    continue;
                 }
-                const unsigned kept = __ballot_sync(0xffffffffu, keep);
-                if (keep)
-                    wq[queued + __popc(kept & lanes_below)] =
-                        ((uint32_t)c << 10) | (uint32_t)((py - y0) * TILE_X + (px - x0));
-                queued += __popc(kept);
+                const int b = __ffs(any) - 1, c = c0 + b;
+                any &= any - 1;
+                const int4 r0 = rec0[c];
+                const float4 ck = col[c];
+                const float base = fmaf(X, ck.w, __int_as_float(r0.z));
+                const bool inx = (unsigned)r0.x & (1u << (px - x0));
+#pragma unroll
+                for (int j = 0; j < PIX_PER_THREAD; ++j) {
+                    if (!((meets[j] >> b) & 1u)) continue;
+                    // (a pixel of the rectangle lies in the image)
+                    const bool in = inx && ((unsigned)r0.y & (1u << (py - y0 + j * ROW_STEP))) && slot[j] != c;
+                    const float bound = fmaf(fL[j], ck.x, fmaf(fa[j], ck.y, fmaf(fb[j], ck.z,
+                                             fmaf(Y + (float)(j * ROW_STEP), __int_as_float(r0.w), base))));
+                    const bool loses = bound > thr[j];
+                    if (COUNT && in && loses) {
+                        // a pair that cannot win is not walked (counted as the method's work)
+                        const int4 r1 = rec1[c];
+                        count_pair(max(abs(px - r1.x), abs(py + j * ROW_STEP - r1.y)) + 1);
+                    }
+                    const bool keep = in && !loses;
+                    const unsigned kept = __ballot_sync(0xffffffffu, keep);
+                    if (keep) wq[queued + __popc(kept & lanes_below)] = (uint16_t)((c << 6) | (j << 5) | lane);
+                    queued += __popc(kept);
+                }
+            }
+            __syncwarp();  // the queued pairs
+            int from = 0;
+#pragma unroll 1
+            for (; more ? from + 32 <= queued : from < queued; from += 32) {
+                if (from + lane >= queued) continue;
+                const int e = wq[from + lane], c = e >> 6;
+                const int qx = bx + (e & 31) % WARP_BLOCK_X;
+                const int qy = by + (e & 31) / WARP_BLOCK_X + ((e >> 5) & 1) * ROW_STEP;
+                const int4 r1 = rec1[c], r2 = rec2[c];
+                int len;
+                const float D = pair_distance(qx, qy, c, r1, r2, own_distance(qx, qy, c, r2), spatial(qx, qy, r1), &len);
+                atomicMin(&best[(qy - y0) * TILE_X + (qx - x0)], pack_best(D, c));
+                count_pair(len);
+            }
+            if (more) {  // the pairs left over start the next queue
+                queued -= from;
+                const uint16_t e = lane < queued ? wq[from + lane] : (uint16_t)0;
                 __syncwarp();
-                if (queued >= 32) {
-                    const uint32_t e = wq[lane];
-                    __syncwarp();
-                    if (lane < queued - 32) wq[lane] = wq[32 + lane];
-                    queued -= 32;
-                    __syncwarp();
-                    walk_queued(e);
-                }
+                if (lane < queued) wq[lane] = e;
+                __syncwarp();
             }
         }
-        if (lane < queued) walk_queued(wq[lane]);
     } else {
         // per-pixel path: every candidate straight from the global list
 #pragma unroll 1
@@ -573,7 +643,7 @@ __device__ __forceinline__ void assign_tile(const SolveArgs &a, int tile, unsign
                     bestD = D;
                     bestk[j] = k;
                 }
-                if (a.count_samples) {
+                if (COUNT && a.count_samples) {
                     atomicAdd(tile_samples, (unsigned)len);
                     atomicAdd(tile_samples + 1, 1u);
                 }
@@ -586,21 +656,14 @@ __device__ __forceinline__ void assign_tile(const SolveArgs &a, int tile, unsign
 
     // labels and the warp-aggregated integer sums of the update; the
     // pixels' own samples are all requested first
-    float4 owns[PIX_PER_THREAD];
-#pragma unroll
-    for (int j = 0; j < PIX_PER_THREAD; ++j) {
-        int px, py;
-        my_pixel(j, px, py);
-        owns[j] = px < a.W && py < a.H ? fetch_sample<T>(plane + (long long)py * a.pitch + px)
-                                       : make_float4(0.f, 0.f, 0.f, 0.f);
-    }
+    T own[PIX_PER_THREAD];
+    load_own(own);
 #pragma unroll
     for (int j = 0; j < PIX_PER_THREAD; ++j) {
         int px, py;
         my_pixel(j, px, py);
         const bool valid = px < a.W && py < a.H;
         const long long p = (long long)py * a.W + px;
-        const float4 own = owns[j];
         int lab = -1;
         if (valid) {
             if (fast) {
@@ -618,9 +681,9 @@ __device__ __forceinline__ void assign_tile(const SolveArgs &a, int tile, unsign
         }
         // fire-and-forget reductions into the global cluster sums, one set
         // per label group of the warp (offsets within the tile)
-        warp_aggregate_global(valid, lab, x0, y0, px - x0, py - y0, own, a.acc);
+        warp_aggregate_global(valid, lab, x0, y0, px - x0, py - y0, sample_value(own[j]), a.acc);
     }
-    if (a.count_samples) {
+    if (COUNT && a.count_samples) {
         __syncthreads();  // every warp's counts are in (a CTA-uniform branch)
         if (tid == 0) {
             atomicAdd(&a.ctr->samples, (unsigned long long)tile_samples[0]);
@@ -630,7 +693,7 @@ __device__ __forceinline__ void assign_tile(const SolveArgs &a, int tile, unsign
         if (tid == 0) {
             unsigned long long on_map = 0, on_plane = 0;
             for (int c = 0; c < cnt; ++c) {
-                if (fast && (rec0[c].z & 0xff) * ((rec0[c].z >> 8) & 0xff) == 0) continue;  // no pixel
+                if (fast && rec0[c].x == 0) continue;  // no pixel
                 if (fast && rec2[c].w >= 0) ++on_map;
                 else ++on_plane;
             }

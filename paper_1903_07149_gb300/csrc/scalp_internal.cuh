@@ -488,18 +488,51 @@ __device__ __forceinline__ float colour_dist(float4 v, float cL, float ca, float
 }
 
 // Sums along the path of d_c(q, C_k) (Eq. 1) and of the contour factor w(q)
-// (Eq. 2), in walk order.  Returns |P|.
+// (Eq. 2), in walk order.  Returns |P|.  The walk waits on its loads, so paths
+// the fixed-point rule covers take it in groups of four independent samples
+// (the offset of any of their samples from the path's start fits 32 bits: at
+// most 512 rows of a plane of at most 2^30 pixels).
 template <typename T>
 __device__ __forceinline__ int path_sums(const T *__restrict__ base, int pitch, int ox, int oy,
                                          const PathSetup &s, float cL, float ca, float cb,
                                          float &sum_dc, float &sum_w)
 {
     float dc = 0.f, w = 0.f;
-    int len = walk_path(base, pitch, ox, oy, s, [&](const T *q) {
-        const float4 v = fetch_sample<T>(q);
+    const auto add = [&](float4 v) {
         dc += colour_dist(v, cL, ca, cb);
         w += v.w;
-    });
+    };
+    int len;
+    if (s.ns <= FIXED_STEP_MAX_NS) {
+        int smaj, smin;
+        path_strides(s, pitch, smaj, smin);
+        const T *__restrict__ q0 = base + (long long)(s.ay - oy) * pitch + (s.ax - ox);
+        const uint32_t S = fixed_step_slope(s.dmin, s.ns);
+        uint32_t acc = 0x80000000u;
+        len = s.ns + 1;
+        int q = 0;
+        const auto at = [&](int k) {
+            const uint32_t m = k == 0 ? 0u : (uint32_t)(((unsigned long long)S * (unsigned)k + acc) >> 32);
+            return q + k * smaj + (int)m * smin;
+        };
+        int i = 0;
+#pragma unroll 1
+        for (; i + 4 <= len; i += 4) {
+            T v[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) v[k] = __ldg(q0 + at(k));
+#pragma unroll
+            for (int k = 0; k < 4; ++k) add(sample_value(v[k]));
+            const unsigned long long t = (unsigned long long)S * 4u + acc;
+            acc = (uint32_t)t;
+            q += 4 * smaj + (int)(t >> 32) * smin;
+        }
+#pragma unroll
+        for (int k = 0; k < 3; ++k)
+            if (i + k < len) add(sample_value(__ldg(q0 + at(k))));
+    } else {
+        len = walk_path(base, pitch, ox, oy, s, [&](const T *q) { add(fetch_sample<T>(q)); });
+    }
     sum_dc = dc;
     sum_w = w;
     return len;

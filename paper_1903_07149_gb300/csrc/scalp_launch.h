@@ -63,7 +63,7 @@ bool project_lists_fused(const SolveArgs &a);
 void launch_project_lists(const SolveArgs &a, cudaStream_t st, bool pdl = false);
 // Batch: the assignment of every tile of every image in one launch, and one
 // iteration's update, projection and candidate lists for every image.
-void launch_assign_batch(const BatchArgs &b, int storage, int total_tiles, size_t smem_bytes,
+void launch_assign_batch(const BatchArgs &b, int storage, bool count, int total_tiles, size_t smem_bytes,
                          cudaStream_t st, bool pdl = false);
 cudaError_t assign_batch_configure(int storage);
 // The persistent batched iterations (scalp_persistent.cu): the cooperative
@@ -77,6 +77,8 @@ void launch_batch_update(const BatchArgs &b, int total_clusters, int total_fill,
 // pairs per CTA; smem_bytes = assign_smem_bytes(a.map_cap).
 void launch_assign(const SolveArgs &a, int storage, size_t smem_bytes, cudaStream_t st, bool pdl = false);
 size_t assign_smem_bytes(int map_cap);
+// Whether the assignment may prune with these sizes and weights.
+bool bound_valid(int H, int W, float lam, float ms2);
 // Distance-map pairs that fit when ASSIGN_CTAS_PER_SM assignment CTAs share an SM.
 int assign_map_capacity(int device);
 cudaError_t assign_configure(int storage);

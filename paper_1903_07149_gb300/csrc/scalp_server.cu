@@ -375,7 +375,7 @@ int scalp_server_step(scalp_server *s, int32_t *n_running)
             if (w != cudaSuccess) return server_fail(SCALP_E_CUDA, "join: %s", cudaGetErrorString(w));
             v->joined = true;
         }
-        launch_assign_batch(s->bargs, s->params.storage, s->total_tiles, s->smem, s->st, true);
+        launch_assign_batch(s->bargs, s->params.storage, false, s->total_tiles, s->smem, s->st, true);
         launch_batch_update(s->bargs, s->total_clusters, s->total_fill, s->st, true);
         cudaError_t e = cudaGetLastError();
         // the argument slot stays live until this step has run
