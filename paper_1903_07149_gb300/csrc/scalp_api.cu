@@ -507,6 +507,8 @@ int scalp_init(scalp_ctx **out, const scalp_image *image, const scalp_contour *c
     a.tpw_x = tiles_per_window(c->r, TILE_X);
     a.tpw_y = tiles_per_window(c->r, TILE_Y);
     a.prev_win = reinterpret_cast<int4 *>(c->ws + L.prev_win);
+    // (the connectivity's buffer: the enforcement never runs beside an iteration)
+    a.orphan_list = reinterpret_cast<int *>(c->ws + L.parent);
     a.ctr = reinterpret_cast<DevCounters *>(c->ws + L.ctr);
     c->ccl.parent = reinterpret_cast<int *>(c->ws + L.parent);
     c->ccl.size = reinterpret_cast<int *>(c->ws + L.size);

@@ -676,7 +676,7 @@ __device__ __forceinline__ void assign_tile(const SolveArgs &a, int tile, unsign
                 a.labels[p] = lab;
             } else {
                 lab = a.labels[p];  // no window reaches p: keep its label
-                atomicAdd(&a.ctr->orphans, 1);
+                a.orphan_list[atomicAdd(&a.ctr->orphans, 1)] = (int)p;
             }
         }
         // fire-and-forget reductions into the global cluster sums, one set

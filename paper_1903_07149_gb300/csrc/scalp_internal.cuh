@@ -200,7 +200,7 @@ struct DevCounters {
     unsigned long long map_rects;    // optional: (tile, cluster) rectangles walked on a map
     unsigned long long plane_rects;  // optional: ... walked on the plane in global memory
     unsigned prior_max;  // scratch: maximum of the gradient prior (float bits)
-    int proj_all;        // the update saw orphans: the projection searches the image
+    int proj_orphans;    // orphans of the assignment the update finished: their list is searched as well
     int n_labels;        // labels after the last connectivity enforcement
 };
 constexpr int ERR_TILE_LIST_OVERFLOW = 1;
@@ -232,6 +232,7 @@ struct SolveArgs {
     int4 *prev_win;    // window (xlo, xhi, ylo, yhi) the last assignment used
     const float *lut;  // 256-entry inverse sRGB transfer function
     int *proj_list;
+    int *orphan_list;  // raster indices of the last assignment's orphans (room for N)
     int *tile_count, *tile_off, *tile_cursor, *tile_list;
     long long tile_cap;
     int tpw_x, tpw_y;  // bound on the tiles one window spans, per axis

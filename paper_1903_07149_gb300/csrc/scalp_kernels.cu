@@ -417,8 +417,8 @@ __global__ void __launch_bounds__(PROJ_THREADS) k_project_batch_images(BatchArgs
 // CTAs several times (more than four per CTA): then one
 // warp per cluster for the images whose windows have at most
 // PROJ_WARP_MAX_AREA pixels, and one CTA per cluster for those with larger
-// windows and for those whose projection searches the whole image (at
-// set-up, or after orphans); with fewer clusters, one CTA per cluster for
+// windows, for those with many orphans and, at set-up, for all (the whole
+// image is searched then); with fewer clusters, one CTA per cluster for
 // all.  Dynamic shared memory: 4 * count + 2 ints.
 constexpr float PROJ_WARP_MAX_AREA = 4096.0f;
 
@@ -443,7 +443,7 @@ __global__ void __launch_bounds__(PROJ_THREADS) k_project_batch(BatchArgs b, int
         for (int i = threadIdx.x; i < count; i += blockDim.x) {
             const SolveArgs &a = b.args[i];
             const float side = 2.0f * (float)a.r + 1.0f;  // window side
-            const bool cta = whole_image || a.ctr->proj_all || side * side > PROJ_WARP_MAX_AREA;
+            const bool cta = whole_image || a.ctr->proj_orphans > PROJ_WARP_ORPHANS || side * side > PROJ_WARP_MAX_AREA;
             s_nw[i] = cta ? 0 : s_nc[i];
             s_nc[i] = cta ? s_nc[i] : 0;
         }
@@ -456,8 +456,7 @@ __global__ void __launch_bounds__(PROJ_THREADS) k_project_batch(BatchArgs b, int
         const int i = batch_find(s_pw, count, t);
         project_warp(b.args[i], t - s_pw[i]);
     }
-    // (t is CTA-uniform: the barriers inside project_cta are safe; it searches
-    // the whole image only at set-up or after orphans)
+    // (t is CTA-uniform: the barriers inside project_cta are safe)
     for (int t = blockIdx.x; t < total_c; t += G) {
         const int i = batch_find(s_pc, count, t);
         project_cta(b.args[i], whole_image, t - s_pc[i], INT_MAX);

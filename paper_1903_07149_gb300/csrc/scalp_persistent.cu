@@ -116,10 +116,10 @@ __device__ __noinline__ void phase_update(const BatchArgs &b, int total_clusters
 }
 
 
-// The whole-image searches (an image whose last assignment left pixels with
-// no candidate), one CTA per queued cluster: out of line, so that their
-// registers stay out of the other phases' allocation.
-__device__ __noinline__ void project_whole_image(const SolveArgs &a, int j)
+// The searches of an image whose last assignment left many pixels with no
+// candidate, one CTA per queued cluster: out of line, so that their registers
+// stay out of the other phases' allocation.
+__device__ __noinline__ void project_by_cta(const SolveArgs &a, int j)
 {
     project_cta(a, 0, j, INT_MAX);
 }
@@ -128,18 +128,18 @@ __device__ __noinline__ void project_whole_image(const SolveArgs &a, int j)
 // lays out the same list of all queued clusters of all images (a prefix over
 // the images' queue lengths, in the dynamic shared memory the assignment
 // phase has finished with) and its warps take entries in turn, a warp per
-// cluster; the clusters of images that need a whole-image search are taken
-// by whole CTAs afterwards.  Needs 2 * count + 1 ints of shared memory
+// cluster; the clusters of images with many orphans are taken by whole CTAs
+// afterwards.  Needs 2 * count + 1 ints of shared memory
 // (checked on the host).
 __device__ __noinline__ void phase_project(const BatchArgs &b, unsigned char *smem)
 {
     __shared__ int s_warp[32];
     const int G = gridDim.x, count = b.count;
     for (int i = blockIdx.x; i < count; i += G) scan_tiles_cta<ASSIGN_THREADS>(b.args[i]);
-    int *s_cnt = reinterpret_cast<int *>(smem);  // per image: queue length, 0 for whole-image
+    int *s_cnt = reinterpret_cast<int *>(smem);  // per image: queue length, 0 with many orphans
     int *s_pref = s_cnt + count;                 // count + 1: its prefix
     for (int i = threadIdx.x; i < count; i += blockDim.x)
-        s_cnt[i] = b.args[i].ctr->proj_all ? 0 : b.args[i].ctr->nproj;
+        s_cnt[i] = b.args[i].ctr->proj_orphans > PROJ_WARP_ORPHANS ? 0 : b.args[i].ctr->nproj;
     __syncthreads();
     cta_scan(s_cnt, s_pref, count, ASSIGN_THREADS, s_warp);
     const int total = s_pref[count];
@@ -148,11 +148,11 @@ __device__ __noinline__ void phase_project(const BatchArgs &b, unsigned char *sm
         const int i = batch_find(s_pref, count, t);
         project_warp(b.args[i], t - s_pref[i]);
     }
-    // whole-image searches: image by image, entry j on CTA (j mod G)
+    // images with many orphans: image by image, entry j on CTA (j mod G)
     for (int i = 0; i < count; ++i) {
-        if (s_cnt[i] != 0 || !b.args[i].ctr->proj_all) continue;
+        if (s_cnt[i] != 0 || b.args[i].ctr->proj_orphans <= PROJ_WARP_ORPHANS) continue;
         const int nproj = b.args[i].ctr->nproj;
-        for (int j = blockIdx.x; j < nproj; j += G) project_whole_image(b.args[i], j);
+        for (int j = blockIdx.x; j < nproj; j += G) project_by_cta(b.args[i], j);
     }
 }
 

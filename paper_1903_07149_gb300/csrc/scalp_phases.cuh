@@ -114,9 +114,9 @@ __device__ __forceinline__ void update_cluster(const SolveArgs &a, int k, int fr
     bool check_projection = false;
     int label_at_end = k;
     if (from_acc && k == 0) {
-        // the orphans of the assignment just finished decide the projection's
+        // the projection searches the orphans of the assignment just finished
         // region; the count starts again for the next assignment
-        a.ctr->proj_all = atomicExch(&a.ctr->orphans, 0) > 0;
+        a.ctr->proj_orphans = atomicExch(&a.ctr->orphans, 0);
     }
     if (from_acc) {
         const ClusterAcc c = a.acc[k];
@@ -165,9 +165,30 @@ __device__ __forceinline__ void update_cluster(const SolveArgs &a, int k, int fr
     }
 }
 
-// Eq. 4 for queued cluster j of one image by one warp, over the window the
-// last assignment used (which holds S_k): the same argmin, with the same
-// exact comparison and tie rule, as the CTA-wide search.
+// S_k lies in the window the last assignment used for cluster k, apart from
+// the pixels that no window reached and that kept their label k.  The
+// assignment lists those (there are seldom more than a few, but one was
+// enough to make every search take the whole image: 0.8 ms more per HD solve
+// for such inputs, 3.7 ms for the 32 x 240 x 320 video), and the searches go
+// through the window and the list.  Larger lists are left to whole CTAs.
+constexpr int PROJ_WARP_ORPHANS = 1024;
+
+// The listed orphans' candidates for cluster k; thread t of `threads`.
+__device__ __forceinline__ void project_orphans(const SolveArgs &a, int k, long long n, long long sx, long long sy,
+                                                bool small, int t, int threads, ProjBest &b)
+{
+    const int count = a.ctr->proj_orphans;
+    for (int i = t; i < count; i += threads) {
+        const int p = a.orphan_list[i];
+        if (a.labels[p] != k) continue;
+        const int y = p / a.W;
+        const ProjBest c = proj_candidate(p, p - y * a.W, y, n, sx, sy, small);
+        if (proj_less(c, b)) b = c;
+    }
+}
+
+// Eq. 4 for queued cluster j of one image by one warp: the same argmin, with
+// the same exact comparison and tie rule, as the CTA-wide search.
 __device__ __forceinline__ void project_warp(const SolveArgs &a, int j)
 {
     constexpr int BATCH = 4;
@@ -203,6 +224,7 @@ __device__ __forceinline__ void project_warp(const SolveArgs &a, int j)
             if (proj_less(c, b)) b = c;
         }
     }
+    project_orphans(a, k, n, sx, sy, small, lane, 32, b);
     proj_shfl_min(b);
     if (lane == 0) {
         if (b.p == LLONG_MAX) {
@@ -216,15 +238,13 @@ __device__ __forceinline__ void project_warp(const SolveArgs &a, int j)
     }
 }
 
-// Queued projections: S_k lies inside the window the last assignment used for
-// cluster k, unless some pixel kept its old label for lack of any candidate;
-// then (or with whole_image, at set-up) the whole image is searched.  One CTA
-// per queued cluster.  Queue entries j0, j0 + stride, ... of one image.
+// Queued projections over the window and the orphans (with whole_image, at
+// set-up, the whole image).  One CTA per queued cluster.  Queue entries j0,
+// j0 + stride, ... of one image.
 __device__ __forceinline__ void project_cta(const SolveArgs &a, int whole_image, int j0, int stride)
 {
     __shared__ ProjBest s_best[PROJ_THREADS / 32];
     const int nproj = a.ctr->nproj;
-    const bool all = whole_image || a.ctr->proj_all;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const double bound = (double)max(a.W, a.H);
     // (the step cannot overflow: a stride past the queue's end ends the loop)
@@ -232,7 +252,7 @@ __device__ __forceinline__ void project_cta(const SolveArgs &a, int whole_image,
         const int k = a.proj_list[j];
         const long long n = a.st_n[k], sx = a.st_sx[k], sy = a.st_sy[k];
         int xlo = 0, xhi = a.W - 1, ylo = 0, yhi = a.H - 1;
-        if (!all) {
+        if (!whole_image) {
             const int4 w4 = a.prev_win[k];
             xlo = w4.x; xhi = w4.y; ylo = w4.z; yhi = w4.w;
         }
@@ -266,6 +286,7 @@ __device__ __forceinline__ void project_cta(const SolveArgs &a, int whole_image,
                 if (proj_less(c, b)) b = c;
             }
         }
+        if (!whole_image) project_orphans(a, k, n, sx, sy, small, tid, PROJ_THREADS, b);
         proj_shfl_min(b);
         if (lane == 0) s_best[warp] = b;
         __syncthreads();

@@ -70,6 +70,7 @@ struct VoxArgs {
     VoxAcc *acc;
     int *prev_win;            // 6 ints per cluster: the window the last assignment used
     int *proj_list;
+    int *orphan_list;         // voxel indices of the last assignment's orphans (room for N)
     int *tile_count, *tile_off, *tile_cursor, *tile_list;
     DevCounters *ctr;
     const float *lut;
@@ -255,13 +256,33 @@ __global__ void k_vupdate(VoxArgs a, int from_acc)
 // Projection (Eq. 4) of the queued clusters: argmin over the voxels labelled
 // k of (n*x - Sx)^2 + (n*y - Sy)^2 + (n*t - St)^2 in 128-bit integers, ties
 // to the smallest voxel index; searched over the window the last assignment
-// used (it holds S_k) unless some voxel kept its label for lack of a
-// candidate, or at set-up: then over the whole volume.
+// used and the listed voxels that kept their label for lack of a candidate
+// (together they hold S_k), or at set-up over the whole volume.
 // ---------------------------------------------------------------------------
 struct VBest {
     unsigned long long hi, lo;
     long long p;
 };
+
+// Voxel (x, y, t) of index p as a candidate for X_k^* of cluster (n, sx, sy, st).
+__device__ __forceinline__ VBest vcandidate(long long p, int x, int y, int t, long long n, long long sx,
+                                            long long sy, long long st, bool small)
+{
+    VBest c;
+    c.p = p;
+    if (small) {
+        const long long dx = n * x - sx, dy = n * y - sy, dt = n * t - st;
+        c.hi = 0;
+        c.lo = (unsigned long long)(dx * dx) + (unsigned long long)(dy * dy) + (unsigned long long)(dt * dt);
+    } else {
+        const __int128 dx = (__int128)n * x - sx, dy = (__int128)n * y - sy, dt = (__int128)n * t - st;
+        const unsigned __int128 d2 =
+            (unsigned __int128)(dx * dx) + (unsigned __int128)(dy * dy) + (unsigned __int128)(dt * dt);
+        c.hi = (unsigned long long)(d2 >> 64);
+        c.lo = (unsigned long long)d2;
+    }
+    return c;
+}
 
 __device__ __forceinline__ bool vless(const VBest &u, const VBest &v)
 {
@@ -285,13 +306,13 @@ __global__ void __launch_bounds__(VPROJ_THREADS) k_vproject(VoxArgs a, int whole
     pdl_release();
     __shared__ VBest s_best[VPROJ_THREADS / 32];
     const int nproj = a.ctr->nproj;
-    const bool all = whole || a.ctr->orphans > 0;
+    const int n_orphans = whole ? 0 : a.ctr->orphans;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     for (int j = blockIdx.x; j < nproj; j += gridDim.x) {
         const int k = a.proj_list[j];
         const long long n = a.st_n[k], sx = a.st_sx[k], sy = a.st_sy[k], st = a.st_st[k];
         int xlo = 0, xhi = a.W - 1, ylo = 0, yhi = a.H - 1, tlo = 0, thi = a.T - 1;
-        if (!all) {
+        if (!whole) {
             const int *pw = a.prev_win + 6 * (long long)k;
             xlo = pw[0]; xhi = pw[1]; ylo = pw[2]; yhi = pw[3]; tlo = pw[4]; thi = pw[5];
         }
@@ -323,22 +344,16 @@ __global__ void __launch_bounds__(VPROJ_THREADS) k_vproject(VoxArgs a, int whole
                 const long long row = div_w.row(i), fr = div_h.row(row);
                 const int x = xlo + (int)(i - row * w), y = ylo + (int)(row - fr * h), t = tlo + (int)fr;
                 const long long p = ((long long)t * a.H + y) * a.W + x;
-                VBest c;
-                c.p = p;
-                if (small) {
-                    const long long dx = n * x - sx, dy = n * y - sy, dt = n * t - st;
-                    c.hi = 0;
-                    c.lo = (unsigned long long)(dx * dx) + (unsigned long long)(dy * dy) +
-                           (unsigned long long)(dt * dt);
-                } else {
-                    const __int128 dx = (__int128)n * x - sx, dy = (__int128)n * y - sy, dt = (__int128)n * t - st;
-                    const unsigned __int128 d2 = (unsigned __int128)(dx * dx) + (unsigned __int128)(dy * dy) +
-                                                 (unsigned __int128)(dt * dt);
-                    c.hi = (unsigned long long)(d2 >> 64);
-                    c.lo = (unsigned long long)d2;
-                }
+                const VBest c = vcandidate(p, x, y, t, n, sx, sy, st, small);
                 if (vless(c, b)) b = c;
             }
+        }
+        for (int i = tid; i < n_orphans; i += VPROJ_THREADS) {
+            const int p = a.orphan_list[i];
+            if (a.labels[p] != k) continue;
+            const int t = (int)(p / a.HW), q = (int)(p - t * a.HW), y = q / a.W;
+            const VBest c = vcandidate(p, q - y * a.W, y, t, n, sx, sy, st, small);
+            if (vless(c, b)) b = c;
         }
         vshfl_min(b);
         if (lane == 0) s_best[warp] = b;
@@ -734,7 +749,7 @@ __global__ void __launch_bounds__(VTILE) k_vassign(VoxArgs a)
             a.labels[p] = lab;
         } else {
             lab = a.labels[p];  // no window reaches the voxel: keep its label
-            atomicAdd(&a.ctr->orphans, 1);
+            a.orphan_list[atomicAdd(&a.ctr->orphans, 1)] = (int)p;
         }
     }
     // a warp = 32 voxels of one frame: 16 columns x 2 rows
@@ -986,6 +1001,8 @@ int scalp_voxel_init(scalp_vctx **out, const scalp_volume *vol, int32_t K, float
     a.cdev = reinterpret_cast<VoxCluster *>(c->ws + L.cdev);
     a.acc = reinterpret_cast<VoxAcc *>(c->ws + L.acc);
     a.prev_win = reinterpret_cast<int *>(c->ws + L.prev_win);
+    // (the contour's staging area, read by the set-up alone)
+    a.orphan_list = reinterpret_cast<int *>(c->ws + L.contour);
     a.proj_list = reinterpret_cast<int *>(c->ws + L.proj);
     a.tile_count = reinterpret_cast<int *>(c->ws + L.tile_count);
     a.tile_off = reinterpret_cast<int *>(c->ws + L.tile_off);
