@@ -16,15 +16,8 @@ __device__ __forceinline__ uint32_t smem_u32(const void *p)
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
-// One FP32 pair of a distance map, by 32-bit shared-memory byte address.
-__device__ __forceinline__ float2 lds_pair(uint32_t addr)
-{
-    float2 v;
-    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(addr));
-    return v;
-}
-
-// The same pair as the two floats' bits in one 64-bit word (d_c low).
+// One FP32 pair of a distance map, by 32-bit shared-memory byte address: the
+// two floats' bits in one 64-bit word (d_c low).
 __device__ __forceinline__ unsigned long long lds_pair_bits(uint32_t addr)
 {
     unsigned long long v;
@@ -39,21 +32,34 @@ __device__ __forceinline__ void add_pair(unsigned long long &acc, unsigned long 
     asm("add.rn.f32x2 %0, %0, %1;" : "+l"(acc) : "l"(v));
 }
 
-// Path sums of Eq. 1 and Eq. 2 over a distance map (row pitch `bw` pairs,
-// pair (0,0) = image pixel (bx0, by0)).  The same samples, in the same order
-// and with the same FP32 additions, as path_sums over the plane.
-__device__ __forceinline__ int path_sums_map(uint32_t map, int bw, int bx0, int by0,
-                                             const PathSetup &s, float &sum_dc, float &sum_w)
+// Path of Eq. 1 and Eq. 2 between tile pixel (X, Y) and the endpoint (ex, ey)
+// over a distance map: places count from the tile's corner, which lies at
+// shared-memory address `at` (it may lie outside the map), rows are p8 bytes
+// apart.  Yields d_c of the pixel itself and the sums over the path, the same
+// samples in the same order and with the same FP32 additions as path_sums()
+// over the plane; returns |P|.  The walk starts at the lexicographically
+// smaller end, the sign of dx * 2^16 + dy (a map's sides are far below 2^15:
+// its rows hold at least four pairs).
+__device__ __forceinline__ int path_sums_map(uint32_t at, int p8, int X, int Y, int ex, int ey, float &dcp,
+                                             float &sum_dc, float &sum_w)
 {
-    int smaj, smin;
-    path_strides(s, bw, smaj, smin);
-    const uint32_t q0 = map + (uint32_t)(((s.ay - by0) * bw + (s.ax - bx0)) * 8);
+    const uint32_t own = at + (uint32_t)(Y * p8 + X * 8);
+    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(dcp) : "r"(own));
+    const int dx = ex - X, dy = ey - Y, key = dx * 65536 + dy;
+    const int adx = abs(dx), ady = abs(dy);
+    const bool xmajor = adx >= ady;
+    PathSetup s;  // (its steps and slope)
+    s.ns = max(adx, ady);
+    s.dmin = min(adx, ady);
+    const int ys = (dy ^ key) < 0 ? -p8 : p8;  // y falls along the walk, or rises
+    const int smaj = xmajor ? 8 : ys, smin = xmajor ? ys : 8;
+    const uint32_t q0 = key < 0 ? at + (uint32_t)(ey * p8 + ex * 8) : own;
     unsigned long long acc = 0;  // (+0.0f, +0.0f)
     const auto visit = [&](uint32_t q) { add_pair(acc, lds_pair_bits(q)); };
     // the fixed-point forms of the steps (fewer instructions per sample)
     // cover every path of up to FIXED_STEP_MAX_NS steps
-    const int len = s.ns <= FIXED_STEP_MAX_NS ? walk_grouped<4>(q0, smaj * 8, smin * 8, s, visit)
-                                              : walk_with<ErrorTermStep>(q0, smaj * 8, smin * 8, s, visit);
+    const int len = s.ns <= FIXED_STEP_MAX_NS ? walk_grouped<4>(q0, smaj, smin, s, visit)
+                                              : walk_with<ErrorTermStep>(q0, smaj, smin, s, visit);
     sum_dc = __uint_as_float((unsigned)acc);
     sum_w = __uint_as_float((unsigned)(acc >> 32));
     return len;
@@ -77,7 +83,8 @@ static_assert(AssignSmem::queue % 16 == 0 && AssignSmem::misc % 16 == 0 && Assig
 //   rec0 = (columns, rows, K bits, g_y bits)         its rectangle as a mask of
 //          the tile's columns and one of its rows; terms of the bound
 //   rec1 = (ex, ey, xk bits, yk bits)                endpoint, X_k
-//   rec2 = (bx0, by0, pitch, map byte offset, or -1: walk the plane)
+//   rec2 = (endpoint from the tile's corner, address of that corner on the
+//          map, bytes per map row, or 0: walk the plane)
 // the map box for the build, box = (bx0, by0, pitch, 32-bit reciprocal of
 // the pitch), the colour C_k, col = (l_k, a_k, b_k, g_x), the cluster index
 // cid, the box area and the prefixes mfirst and cfirst of the map layout.
@@ -407,7 +414,9 @@ __device__ __forceinline__ void assign_tile(const SolveArgs &a, int tile, unsign
         if (tid < cnt) {
             const int4 b = box[tid];
             const bool mapped = area[tid] > 0 && mfirst[tid + 1] <= used;
-            rec2[tid] = make_int4(b.x, b.y, b.z, mapped ? mfirst[tid] * (int)sizeof(float2) : -1);
+            rec2[tid] = make_int4(rec1[tid].x - x0, rec1[tid].y - y0,
+                                  (int)(maps_u32 + 8u * (uint32_t)(mfirst[tid] - (b.y - y0) * b.z - (b.x - x0))),
+                                  mapped ? b.z * 8 : 0);
         }
         // warps take the chunks in turn; within one the candidate is uniform
         // and the lanes read consecutive entries (coalesced plane rows).  No
@@ -456,29 +465,23 @@ __device__ __forceinline__ void assign_tile(const SolveArgs &a, int tile, unsign
 #pragma unroll
     for (int j = 0; j < PIX_PER_THREAD; ++j) bestk[j] = INT_MAX;
 
-    // D of pixel (qx, qy) for candidate slot c (Eq. 1-3), its path length in
-    // *len; on a map when the candidate has one, else on the plane
-    auto pair_distance = [&](int qx, int qy, int c, int4 r1, int4 r2, float dcp, float ds, int *len) {
-        const PathSetup s = path_setup(qx, qy, r1.x, r1.y);
-        float sdc, sw;
-        if (r2.w >= 0) {
-            *len = path_sums_map(maps_u32 + (uint32_t)r2.w, r2.z, r2.x, r2.y, s, sdc, sw);
+    // D of tile pixel (X, Y) for candidate slot c (Eq. 1-3), its path length
+    // in len: on a map when the candidate has one, else on the plane
+    auto pair_distance = [&](int X, int Y, int c, int &len) {
+        const int4 r2 = rec2[c];
+        const float2 xk = *reinterpret_cast<const float2 *>(&rec1[c].z);
+        const int qx = x0 + X, qy = y0 + Y;
+        const float ddx = (float)qx - xk.x, ddy = (float)qy - xk.y;
+        float dcp, sdc, sw;
+        if (r2.w != 0) {
+            len = path_sums_map((uint32_t)r2.z, r2.w, X, Y, r2.x, r2.y, dcp, sdc, sw);
         } else {
             const float4 ck = col[c];
-            *len = path_sums<T>(plane, a.pitch, 0, 0, s, ck.x, ck.y, ck.z, sdc, sw);
+            const int4 r1 = rec1[c];
+            dcp = colour_dist(fetch_sample<T>(plane + (long long)qy * a.pitch + qx), ck.x, ck.y, ck.z);
+            len = path_sums<T>(plane, a.pitch, 0, 0, path_setup(qx, qy, r1.x, r1.y), ck.x, ck.y, ck.z, sdc, sw);
         }
-        return scalp_distance(dcp, sdc, sw, *len, a.lam, a.gamma, a.ms2, ds);
-    };
-    // the pixel's own colour distance d_c(p, C_c) (map entry, else the plane)
-    auto own_distance = [&](int qx, int qy, int c, int4 r2) {
-        if (r2.w >= 0)
-            return lds_pair(maps_u32 + (uint32_t)r2.w + (uint32_t)(((qy - r2.y) * r2.z + (qx - r2.x)) * 8)).x;
-        const float4 ck = col[c];
-        return colour_dist(fetch_sample<T>(plane + (long long)qy * a.pitch + qx), ck.x, ck.y, ck.z);
-    };
-    auto spatial = [&](int qx, int qy, int4 r1) {
-        const float ddx = (float)qx - __int_as_float(r1.z), ddy = (float)qy - __int_as_float(r1.w);
-        return fmaf(ddx, ddx, ddy * ddy);
+        return scalp_distance(dcp, sdc, sw, len, a.lam, a.gamma, a.ms2, fmaf(ddx, ddx, ddy * ddy));
     };
     auto count_pair = [&](int len) {
         if (COUNT && a.count_samples) {
@@ -505,10 +508,8 @@ __device__ __forceinline__ void assign_tile(const SolveArgs &a, int tile, unsign
             for (int i = 1; i < PIX_PER_THREAD; ++i)  // (registers: constant indices)
                 if (i == j) c = slot[i];
             if (c >= 0) {
-                const int4 r1 = rec1[c], r2 = rec2[c];
                 int len;
-                const float D = pair_distance(px, py, c, r1, r2, own_distance(px, py, c, r2), spatial(px, py, r1),
-                                              &len);
+                const float D = pair_distance(px - x0, py - y0, c, len);
                 best[(py - y0) * TILE_X + (px - x0)] = pack_best(D, c);  // (the pixel's first D)
 #pragma unroll
                 for (int i = 0; i < PIX_PER_THREAD; ++i)
@@ -603,12 +604,11 @@ __device__ __forceinline__ void assign_tile(const SolveArgs &a, int tile, unsign
             for (; more ? from + 32 <= queued : from < queued; from += 32) {
                 if (from + lane >= queued) continue;
                 const int e = wq[from + lane], c = e >> 6;
-                const int qx = bx + (e & 31) % WARP_BLOCK_X;
-                const int qy = by + (e & 31) / WARP_BLOCK_X + ((e >> 5) & 1) * ROW_STEP;
-                const int4 r1 = rec1[c], r2 = rec2[c];
+                const int X = bx - x0 + (e & 31) % WARP_BLOCK_X;
+                const int Y = by - y0 + (e & 31) / WARP_BLOCK_X + ((e >> 5) & 1) * ROW_STEP;
                 int len;
-                const float D = pair_distance(qx, qy, c, r1, r2, own_distance(qx, qy, c, r2), spatial(qx, qy, r1), &len);
-                atomicMin(&best[(qy - y0) * TILE_X + (qx - x0)], pack_best(D, c));
+                const float D = pair_distance(X, Y, c, len);
+                atomicMin(&best[Y * TILE_X + X], pack_best(D, c));
                 count_pair(len);
             }
             if (more) {  // the pairs left over start the next queue
@@ -694,7 +694,7 @@ __device__ __forceinline__ void assign_tile(const SolveArgs &a, int tile, unsign
             unsigned long long on_map = 0, on_plane = 0;
             for (int c = 0; c < cnt; ++c) {
                 if (fast && rec0[c].x == 0) continue;  // no pixel
-                if (fast && rec2[c].w >= 0) ++on_map;
+                if (fast && rec2[c].w != 0) ++on_map;
                 else ++on_plane;
             }
             atomicAdd(&a.ctr->map_rects, on_map);
