@@ -85,8 +85,8 @@ static_assert(AssignSmem::queue % 16 == 0 && AssignSmem::misc % 16 == 0 && Assig
 //   rec1 = (ex, ey, xk bits, yk bits)                endpoint, X_k
 //   rec2 = (endpoint from the tile's corner, address of that corner on the
 //          map, bytes per map row, or 0: walk the plane)
-// the map box for the build, box = (bx0, by0, pitch, 32-bit reciprocal of
-// the pitch), the colour C_k, col = (l_k, a_k, b_k, g_x), the cluster index
+// the map box for the build, box = (bx0, by0, pitch, width | height << 16),
+// the colour C_k, col = (l_k, a_k, b_k, g_x), the cluster index
 // cid, the box area and the prefixes mfirst and cfirst of the map layout.
 struct TileLayout {
     uint32_t rec0, rec1, rec2, box, col, cid, area, mfirst, cfirst, maps;
@@ -162,11 +162,11 @@ __device__ __forceinline__ unsigned long long pack_best(float D, int slot)
 
 // The map layout by one warp: mfirst = exclusive prefix of the box areas
 // (cnt + 1 entries); the leading candidates whose boxes end within cap get a
-// map, of CHUNK-entry chunks whose prefix goes to cfirst (cnt + 1 entries;
-// none for the others).  Returns the map entries used.
-template <int CHUNK>
-__device__ __forceinline__ int warp_scan_maps(const int *area, int *mfirst, int *cfirst, int cnt, int cap,
-                                              int lane)
+// map, of BUILD_STRIP-column strips whose prefix goes to cfirst (cnt + 1
+// entries; none for the others).  Returns the map entries used.
+constexpr int BUILD_STRIP = 8;
+__device__ __forceinline__ int warp_scan_maps(const int *area, const int4 *box, int *mfirst, int *cfirst, int cnt,
+                                              int cap, int lane)
 {
     constexpr int PER = MAX_TILE_CANDIDATES / 32;
     int v[PER], ch[PER], sum = 0;
@@ -190,7 +190,7 @@ __device__ __forceinline__ int warp_scan_maps(const int *area, int *mfirst, int 
         run += v[i];
         const bool mapped = c < cnt && v[i] > 0 && run <= cap;
         if (c < cnt && run <= cap) fit = run;
-        ch[i] = mapped ? (v[i] + CHUNK - 1) / CHUNK : 0;
+        ch[i] = mapped ? ((box[c].w & 0xffff) + BUILD_STRIP - 1) / BUILD_STRIP : 0;
         csum += ch[i];
     }
     if (lane == 31) mfirst[cnt] = incl;
@@ -223,8 +223,7 @@ __device__ __forceinline__ void assign_tile(const SolveArgs &a, int tile, unsign
     constexpr int THREADS = ASSIGN_THREADS;
     constexpr int PIX_PER_THREAD = TILE_PIXELS / THREADS;
     constexpr int WARPS = THREADS / 32;
-    constexpr int BUILD_UNROLL = 4;
-    constexpr int BUILD_CHUNK = BUILD_UNROLL * 32;  // map entries per warp task
+    constexpr int BUILD_UNROLL = 4;  // samples per lane in flight
     const T *__restrict__ plane = reinterpret_cast<const T *>(
         sizeof(T) == 16 ? (const void *)a.plane32 : (const void *)a.plane16);
     const int tx = tile % a.n_tx, ty = tile / a.n_tx;
@@ -323,20 +322,19 @@ __device__ __forceinline__ void assign_tile(const SolveArgs &a, int tile, unsign
         // map box: the rectangle and the endpoint (both inside the image).
         // Rows are padded to a pitch = 4 (mod 8) pairs: the walks of a warp
         // then spread over the shared-memory banks (neighbouring rows start
-        // 8 banks apart); 32-bit reciprocal of the pitch for the build.
-        int bx0 = 0, by0 = 0, pitch = 1;
+        // 8 banks apart).  A mapped box has width and height below 2^16 (its
+        // pitch is at least 4, its area at most the buffer's).
+        int bx0 = 0, by0 = 0, pitch = 4, size = 0;
         long long n = 0;
         if (some) {
             bx0 = min(xa, cd.ex);
             by0 = min(ya, cd.ey);
-            const int bw = max(xb, cd.ex) - bx0 + 1;
+            const int bw = max(xb, cd.ex) - bx0 + 1, bh = max(yb, cd.ey) - by0 + 1;
             pitch = bw + ((4 - bw) & 7);
-            n = (long long)pitch * (max(yb, cd.ey) - by0 + 1);
+            n = (long long)pitch * bh;
+            size = min(bw, 0xffff) | (min(bh, 0xffff) << 16);
         }
-        // ceil(2^32 / pitch) = floor((2^32 - 1) / pitch) + 1 for pitch >= 2
-        // (an empty box has pitch 1 and no map)
-        const unsigned rcp = pitch > 1 ? 0xffffffffu / (unsigned)pitch + 1u : 0u;
-        box[rank] = make_int4(bx0, by0, pitch, (int)rcp);
+        box[rank] = make_int4(bx0, by0, pitch, size);
         // a box larger than the whole buffer never fits: clamp it so that the
         // prefix sums stay small
         area[rank] = map_cap > 0 ? (int)min(n, (long long)map_cap + 1) : 0;
@@ -356,7 +354,7 @@ __device__ __forceinline__ void assign_tile(const SolveArgs &a, int tile, unsign
             for (int j = 0; j < 32; ++j) rank += __shfl_sync(0xffffffffu, myid, j) < myid;
             if (lane < cnt) write_records(rank, myid, cd);
             __syncwarp();
-            const int used = warp_scan_maps<BUILD_CHUNK>(area, mfirst, cfirst, cnt, map_cap, lane);
+            const int used = warp_scan_maps(area, box, mfirst, cfirst, cnt, map_cap, lane);
             if (lane == 0) misc[2] = used;
         }
 #pragma unroll
@@ -384,7 +382,7 @@ __device__ __forceinline__ void assign_tile(const SolveArgs &a, int tile, unsign
         __syncthreads();
         for (int i = tid; i < TILE_PIXELS; i += THREADS) best[i] = ~0ull;
         if (warp == 0 && fast) {
-            const int used = warp_scan_maps<BUILD_CHUNK>(area, mfirst, cfirst, cnt, map_cap, lane);
+            const int used = warp_scan_maps(area, box, mfirst, cfirst, cnt, map_cap, lane);
             if (lane == 0) misc[2] = used;
         }
     }
@@ -418,41 +416,44 @@ __device__ __forceinline__ void assign_tile(const SolveArgs &a, int tile, unsign
                                   (int)(maps_u32 + 8u * (uint32_t)(mfirst[tid] - (b.y - y0) * b.z - (b.x - x0))),
                                   mapped ? b.z * 8 : 0);
         }
-        // warps take the chunks in turn; within one the candidate is uniform
-        // and the lanes read consecutive entries (coalesced plane rows).  No
-        // branch per entry: a padding column reads its row's last sample and
-        // an entry past the box the last one, and only the latter's store is
-        // left out (the padding is inside the box's own part of the buffer).
-        const int n_chunks = cfirst[cnt];
+        // Warps take the boxes' strips of BUILD_STRIP columns in turn: 8
+        // columns x 4 rows of lanes move down the strip, so an entry costs
+        // two additions for its places instead of a division by the pitch,
+        // and a candidate's record is read once per strip (about nine rows of
+        // lanes on HD).  A row of lanes covers rows {0, 2, 1, 3}: the two rows of a half warp
+        // then lie 16 banks apart.  Lanes past the box read its last column
+        // or row and store nothing.
+        const int n_strips = cfirst[cnt];
+        const int lrow = ((lane >> 3) & 1) << 1 | lane >> 4, lcol = lane & 7;
         int c = 0;
-        for (int g = warp; g < n_chunks; g += WARPS) {
+        for (int g = warp; g < n_strips; g += WARPS) {
             while (g >= cfirst[c + 1]) ++c;
             const int4 b = box[c];
-            // last unpadded column: the rectangle's right edge or e_k
-            const int last = max(x0 + 31 - __clz(rec0[c].x), rec1[c].x) - b.x;
             const float4 ck = col[c];
-            const int m0 = mfirst[c];
-            const int n_le = mfirst[c + 1] - m0;
-            const int le0 = (g - cfirst[c]) * BUILD_CHUNK + lane;
+            const int bw = b.w & 0xffff, bh = (int)((unsigned)b.w >> 16);
+            const int cx = (g - cfirst[c]) * BUILD_STRIP + lcol;
             // the box's first pixel; offsets within the box fit 32 bits: a
             // box of at most map_cap pairs has row < min(H, map_cap / 4) and
             // the plane pitch is at most W + 3, so row * pitch + column < 2^31
             const T *__restrict__ pbox = plane + (long long)b.y * a.pitch + b.x;
-            float2 *mrow = maps + (m0 + le0);
-            T v[BUILD_UNROLL];  // raw samples: all loads issue before any use
+            const int cc = min(cx, bw - 1), last = (bh - 1) * a.pitch + cc, step = 4 * a.pitch;
+            int off = lrow * a.pitch + cc;
+            // (entries of columns past the box are not stored: limit < off)
+            const int limit = cx < bw ? last : -1;
+            float2 *m = maps + (mfirst[c] + lrow * b.z + cx);
+            const int mstep = 4 * b.z;
+            for (int r = 0; r < bh; r += 4 * BUILD_UNROLL) {
+                T v[BUILD_UNROLL];  // raw samples: all loads issue before any use
 #pragma unroll
-            for (int u = 0; u < BUILD_UNROLL; ++u) {
-                const int le = min(le0 + u * 32, n_le - 1);
-                // a mapped box has pitch >= 4 and le * pitch < 2^32, so the
-                // 32-bit reciprocal gives the exact row
-                const int row = (int)__umulhi((unsigned)le, (unsigned)b.w);
-                v[u] = __ldg(pbox + (row * a.pitch + min(le - row * b.z, last)));
-            }
+                for (int u = 0; u < BUILD_UNROLL; ++u) v[u] = __ldg(pbox + min(off + u * step, last));
 #pragma unroll
-            for (int u = 0; u < BUILD_UNROLL; ++u) {
-                const float4 q = sample_value(v[u]);
-                const float2 pair = make_float2(colour_dist(q, ck.x, ck.y, ck.z), q.w);
-                if (le0 + u * 32 < n_le) mrow[u * 32] = pair;
+                for (int u = 0; u < BUILD_UNROLL; ++u) {
+                    const float4 q = sample_value(v[u]);
+                    const float2 pair = make_float2(colour_dist(q, ck.x, ck.y, ck.z), q.w);
+                    if (off <= limit) *m = pair;
+                    off += step;
+                    m += mstep;
+                }
             }
         }
     }
