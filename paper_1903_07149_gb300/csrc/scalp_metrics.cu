@@ -88,70 +88,246 @@ namespace {
 
 struct QualityWs {
     int *ov;                       // n_labels x n_gt overlaps
-    unsigned long long *area, *perim;
+    unsigned long long *perim;
     long long *best, *ue;          // per superpixel
     double *co;                    // per superpixel
     unsigned long long *counts;    // [0] gt boundary pixels, [1] hits
     double *result;                // br, asa, ue, co
 };
 
-__device__ __forceinline__ bool bnd(const int *__restrict__ l, int H, int W, int x, int y)
-{
-    const long long p = (long long)y * W + x;
-    const int c = l[p];
-    return (x > 0 && l[p - 1] != c) || (x < W - 1 && l[p + 1] != c) || (y > 0 && l[p - W] != c) ||
-           (y < H - 1 && l[p + W] != c);
-}
+// The offsets at distance < eps, as half-widths: row offset dy takes the
+// columns within half[|dy|] (-1: none).  Up to QUALITY_RADIUS rows, the larger
+// radii test the distance itself.
+constexpr int QUALITY_RADIUS = 15;
+struct Disk {
+    int r;
+    signed char half[QUALITY_RADIUS + 1];
+};
 
-__global__ void k_quality_pixels(const int *__restrict__ lab, const int *__restrict__ gt, int n_gt,
-                                 int H, int W, double eps, QualityWs w)
+// The pixels of both maps in one pass.  A CTA takes 64 x 64 pixels, a warp 32
+// columns x QUALITY_ROWS rows of them, a lane one column.
+//   * Boundary pixels of the superpixels as one 64-bit mask per row, the
+//     warp's columns and 16 on either side, dilated by the disk with shifts;
+//     a ground-truth boundary pixel is found iff its bit is set.
+//   * Overlaps and perimeters: a lane adds up its run of pixels of one
+//     (superpixel, segment) pair and hands it over when the pair changes;
+//     the runs that reach the strip's end are merged across the warp first.
+//     They are summed in a small hash table in shared memory (a CTA meets
+//     some twenty pairs; one that finds no place goes straight to global
+//     memory) and added to the global sums once per pair.
+// 1080 x 1920, 2000 superpixels with ragged borders: 438 us with one atomic
+// per pixel and counter (most of it on the two counters that every pixel
+// shares), 27.8 us now: 16.6 MB from DRAM, the rest is the row steps' chain of
+// shuffles and ballots.
+constexpr int QUALITY_ROWS = 16, QUALITY_THREADS = 256, QUALITY_SLOTS = 256, QUALITY_PROBES = 8;
+
+template <bool FAR>
+__global__ void __launch_bounds__(QUALITY_THREADS)
+    k_quality_pixels(const int *__restrict__ lab, const int *__restrict__ gt, int n_gt, int H, int W, double eps,
+                     Disk disk, QualityWs w)
 {
-    const long long N = (long long)H * W;
-    const int r = (int)ceil(eps);
-    for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < N;
-         p += (long long)gridDim.x * blockDim.x) {
-        const int y = (int)((unsigned)p / (unsigned)W), x = (int)p - y * W;  // N <= 2^30
-        const int k = lab[p];
-        atomicAdd(&w.ov[(long long)k * n_gt + gt[p]], 1);
-        atomicAdd(&w.area[k], 1ull);
-        const unsigned e = (x == 0 || lab[p - 1] != k) + (x == W - 1 || lab[p + 1] != k) +
-                           (y == 0 || lab[p - W] != k) + (y == H - 1 || lab[p + W] != k);
+    constexpr int WARPS = QUALITY_THREADS / 32;
+    __shared__ unsigned long long s_mask[WARPS][QUALITY_ROWS + 2 * QUALITY_RADIUS];
+    __shared__ unsigned s_gt[WARPS][QUALITY_ROWS];
+    __shared__ unsigned s_count[2];
+    __shared__ int s_key[QUALITY_SLOTS], s_n[QUALITY_SLOTS], s_e[QUALITY_SLOTS];
+    const unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (threadIdx.x < 2) s_count[threadIdx.x] = 0u;
+    for (int i = threadIdx.x; i < QUALITY_SLOTS; i += QUALITY_THREADS) {
+        s_key[i] = -1;
+        s_n[i] = s_e[i] = 0;
+    }
+    __syncthreads();
+    static_assert(WARPS == 8 && QUALITY_ROWS == 16, "a CTA's warps cover 64 x 64 pixels");
+    const unsigned bands = (unsigned)(W + 63) / 64u;
+    const int x0 = (int)(blockIdx.x % bands) * 64 + (warp & 1) * 32;
+    const int y0 = (int)min((long long)(blockIdx.x / bands) * 64 + (warp >> 1) * QUALITY_ROWS, (long long)H);
+    const int y1 = min(H, y0 + QUALITY_ROWS);
+    const int x = x0 + lane;
+    unsigned n_bnd = 0, n_hit = 0;
+    int run_key = -1, run_k = 0, run_n = 0, run_e = 0;  // the lane's run: pair, superpixel, pixels, edges
+    const auto hand_over = [&](int key, int k, int n, int e) {
+        unsigned h = (unsigned)key * 2654435761u >> 24;
+        static_assert(QUALITY_SLOTS == 256, "the hash's top eight bits");
+        for (int i = 0; i < QUALITY_PROBES; ++i, h = (h + 1) % QUALITY_SLOTS) {
+            int was = s_key[h];
+            if (was == -1) was = atomicCAS(&s_key[h], -1, key);
+            if (was == -1 || was == key) {
+                atomicAdd(&s_n[h], n);
+                if (e) atomicAdd(&s_e[h], e);
+                return;
+            }
+        }
+        atomicAdd(&w.ov[key], n);
         if (e) atomicAdd(&w.perim[k], (unsigned long long)e);
-        if (bnd(gt, H, W, x, y)) {
-            atomicAdd(&w.counts[0], 1ull);
-            bool found = false;
-            for (int dy = -r; dy <= r && !found; ++dy)
-                for (int dx = -r; dx <= r && !found; ++dx) {
-                    const int qx = x + dx, qy = y + dy;
-                    if (qx < 0 || qy < 0 || qx >= W || qy >= H) continue;
-                    if (sqrt((double)(dx * dx + dy * dy)) >= eps) continue;
-                    if (bnd(lab, H, W, qx, qy)) found = true;
+    };
+    if (y0 < y1 && x0 < W) {
+        // Rows y0 - r .. y1 - 1 + r from top to bottom, each read once: the
+        // lane's column of both maps, a column of the 16 on either side of
+        // the warp's (superpixels) and of the two next to it (segments).
+        // Places outside the image move to its edge, where a neighbour then
+        // equals the pixel itself.
+        const int r = FAR ? 0 : disk.r, rows = y1 - y0 + 2 * r;
+        const bool valid = x < W, halo_valid = lane < 16 ? x >= 16 : x + 16 < W;
+        const int xc = min(x, W - 1), xh = lane < 16 ? max(x - 16, 0) : min(x + 16, W - 1);
+        const int xg = lane == 0 ? max(x - 1, 0) : lane == 31 ? min(x + 1, W - 1) : xc;
+        struct Row {
+            int c, h, g, e;  // superpixel: own column, halo column; segment: own column, next to the warp's
+        };
+        const auto load = [&](int i) {
+            const long long o = (long long)min(max(y0 - r + i, 0), H - 1) * W;
+            return Row{lab[o + xc], lab[o + xh], gt[o + xc], gt[o + xg]};
+        };
+        const auto process = [&](int i, const Row &up, const Row &at, const Row &down) {
+            const int y = y0 - r + i;
+            const bool in = y >= 0 && y < H;
+            int l = __shfl_up_sync(FULL, at.c, 1), rt = __shfl_down_sync(FULL, at.c, 1);
+            const int h_lo = __shfl_sync(FULL, at.h, 15), h_hi = __shfl_sync(FULL, at.h, 16);
+            if (lane == 0) l = h_lo;
+            if (lane == 31) rt = h_hi;
+            const int e4 = (l != at.c) + (rt != at.c) + (up.c != at.c) + (down.c != at.c);
+            if (!FAR) {
+                int hl = __shfl_up_sync(FULL, at.h, 1), hr = __shfl_down_sync(FULL, at.h, 1);
+                const int c_lo = __shfl_sync(FULL, at.c, 0), c_hi = __shfl_sync(FULL, at.c, 31);
+                if (lane == 16) hl = c_hi;
+                if (lane == 15) hr = c_lo;
+                // (bits 0 and 63 lack a neighbour; no disk reaches them)
+                const unsigned mc = __ballot_sync(FULL, in && valid && e4);
+                const unsigned mh = __ballot_sync(FULL, in && halo_valid && (hl != at.h || hr != at.h || up.h != at.h ||
+                                                                             down.h != at.h));
+                if (lane == 0)
+                    s_mask[warp][i] = (mh & 0xffffu) | (unsigned long long)mc << 16 | (unsigned long long)(mh >> 16) << 48;
+            }
+            if (i < r || i >= rows - r) return;
+            int gl = __shfl_up_sync(FULL, at.g, 1), gr = __shfl_down_sync(FULL, at.g, 1);
+            if (lane == 0) gl = at.e;
+            if (lane == 31) gr = at.e;
+            const bool bnd_gt = valid && (gl != at.g || gr != at.g || up.g != at.g || down.g != at.g);
+            if (FAR) {
+                const auto far_at = [&](int qx, int qy) {
+                    return lab[(long long)min(max(qy, 0), H - 1) * W + min(max(qx, 0), W - 1)];
+                };
+                bool found = false;
+                if (bnd_gt)
+                    for (int dy = -disk.r; dy <= disk.r && !found; ++dy)
+                        for (int dx = -disk.r; dx <= disk.r && !found; ++dx) {
+                            const int qx = x + dx, qy = y + dy;
+                            if (qx < 0 || qy < 0 || qx >= W || qy >= H) continue;
+                            if (sqrt((double)dx * dx + (double)dy * dy) >= eps) continue;
+                            const int c = far_at(qx, qy);
+                            found = far_at(qx - 1, qy) != c || far_at(qx + 1, qy) != c || far_at(qx, qy - 1) != c ||
+                                    far_at(qx, qy + 1) != c;
+                        }
+                n_bnd += bnd_gt;
+                n_hit += found;
+            } else {
+                const unsigned G = __ballot_sync(FULL, bnd_gt);
+                if (lane == 0) s_gt[warp][i - r] = G;
+            }
+            const int e = e4 + (x == 0) + (x == W - 1) + (y == 0) + (y == H - 1);
+            const int key = valid ? at.c * n_gt + at.g : -1;  // (n_labels * n_gt <= 2^28)
+            if (key != run_key) {
+                if (run_key >= 0) hand_over(run_key, run_k, run_n, run_e);
+                run_key = key;
+                run_k = at.c;
+                run_n = run_e = 0;
+            }
+            run_n += 1;
+            run_e += e;
+        };
+        // four rows at a time, the next four on their way meanwhile
+        constexpr int B = 4;
+        Row now[B + 2];
+#pragma unroll
+        for (int u = 0; u < B + 2; ++u) now[u] = load(u - 1);
+#pragma unroll 1
+        for (int i = 0; i < rows; i += B) {
+            Row next[B];
+#pragma unroll
+            for (int u = 0; u < B; ++u) next[u] = load(i + B + 1 + u);
+#pragma unroll
+            for (int u = 0; u < B; ++u)
+                if (i + u < rows) process(i + u, now[u], now[u + 1], now[u + 2]);
+            now[0] = now[B];
+            now[1] = now[B + 1];
+#pragma unroll
+            for (int u = 0; u < B; ++u) now[u + 2] = next[u];
+        }
+        if (!FAR) {
+            __syncwarp();
+            if (lane < y1 - y0) {
+                // row y0 + lane: the dilated boundary against the segments'
+                unsigned long long d = 0;
+                for (int dy = -r; dy <= r; ++dy) {
+                    const int h = disk.half[abs(dy)];
+                    if (h < 0) continue;
+                    const unsigned long long m = s_mask[warp][lane + r + dy];
+                    d |= m;
+                    for (int t = 1; t <= h; ++t) d |= m << t | m >> t;
                 }
-            if (found) atomicAdd(&w.counts[1], 1ull);
+                const unsigned G = s_gt[warp][lane];
+                n_bnd = __popc(G);
+                n_hit = __popc(G & (unsigned)(d >> 16));
+            }
+            __syncwarp();
         }
     }
+    // what is left, one hand-over per pair of the warp
+    for (unsigned pending = __ballot_sync(FULL, run_key >= 0); pending;) {
+        const int leader = __ffs(pending) - 1, key = __shfl_sync(FULL, run_key, leader);
+        const unsigned grp = __ballot_sync(FULL, run_key == key);
+        const int n = __reduce_add_sync(FULL, run_key == key ? run_n : 0);
+        const int e = __reduce_add_sync(FULL, run_key == key ? run_e : 0);
+        if (lane == leader) hand_over(key, run_k, n, e);
+        pending &= ~grp;
+    }
+    n_bnd = __reduce_add_sync(FULL, n_bnd);
+    n_hit = __reduce_add_sync(FULL, n_hit);
+    if (lane == 0 && n_bnd) {
+        atomicAdd(&s_count[0], n_bnd);
+        atomicAdd(&s_count[1], n_hit);
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < QUALITY_SLOTS; i += QUALITY_THREADS) {
+        const int key = s_key[i];
+        if (key < 0) continue;
+        atomicAdd(&w.ov[key], s_n[i]);
+        if (s_e[i]) atomicAdd(&w.perim[key / n_gt], (unsigned long long)s_e[i]);
+    }
+    if (threadIdx.x < 2 && s_count[threadIdx.x])
+        atomicAdd(&w.counts[threadIdx.x], (unsigned long long)s_count[threadIdx.x]);
 }
 
-__global__ void k_quality_rows(int n_labels, int n_gt, QualityWs w)
+// One warp per superpixel: its row of overlaps gives its size (their sum), the
+// largest, and the sum of |S_k| - o over the o > 0.
+__global__ void __launch_bounds__(256) k_quality_rows(int n_labels, int n_gt, QualityWs w)
 {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    pdl_wait();
+    const int k = blockIdx.x * (int)(blockDim.x / 32) + (int)(threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (k >= n_labels) return;
-    const long long a = (long long)w.area[k];
-    long long best = 0, ue = 0;
-    for (int i = 0; i < n_gt; ++i) {
-        const long long o = w.ov[(long long)k * n_gt + i];
+    unsigned a = 0, best = 0, met = 0;
+    for (int i = lane; i < n_gt; i += 32) {
+        const unsigned o = (unsigned)w.ov[(long long)k * n_gt + i];
+        a += o;
         best = max(best, o);
-        if (o > 0) ue += a - o;
+        met += o > 0;
     }
-    w.best[k] = best;
-    w.ue[k] = ue;
-    const double pr = (double)w.perim[k];
-    w.co[k] = a > 0 ? 4.0 * M_PI * (double)a * (double)a / (pr * pr) : 0.0;
+    a = __reduce_add_sync(0xffffffffu, a);
+    best = __reduce_max_sync(0xffffffffu, best);
+    met = __reduce_add_sync(0xffffffffu, met);
+    if (lane == 0) {
+        w.best[k] = best;
+        w.ue[k] = (long long)a * met - a;
+        const double pr = (double)w.perim[k], area = (double)a;
+        w.co[k] = a > 0 ? 4.0 * M_PI * area * area / (pr * pr) : 0.0;
+    }
 }
 
 // One CTA, a fixed summation order: deterministic.
 __global__ void __launch_bounds__(1024) k_quality_total(int n_labels, long long N, QualityWs w)
 {
+    pdl_wait();
     __shared__ long long s_best[1024], s_ue[1024];
     __shared__ double s_co[1024];
     long long b = 0, u = 0;
@@ -200,7 +376,7 @@ size_t quality_layout(int n_labels, int n_gt, QualityWs *w, unsigned char *base)
     unsigned char *result = take(4 * 8);
     if (w) {
         w->ov = reinterpret_cast<int *>(ov);
-        w->area = reinterpret_cast<unsigned long long *>(area);
+        (void)area;  // (the sizes are the overlaps' sums)
         w->perim = reinterpret_cast<unsigned long long *>(perim);
         w->best = reinterpret_cast<long long *>(best);
         w->ue = reinterpret_cast<long long *>(ue);
@@ -236,10 +412,19 @@ extern "C" int scalp_quality_metrics(const int32_t *labels, int32_t n_labels, co
     cudaError_t e = cudaMemsetAsync(workspace, 0, need, st);
     const long long N = (long long)H * W;
     if (e == cudaSuccess) {
-        const int blocks = (int)std::min<long long>((N + 255) / 256, 152 * 16);
-        k_quality_pixels<<<blocks, 256, 0, st>>>(labels, gt, n_gt, H, W, eps, w);
-        k_quality_rows<<<(n_labels + 255) / 256, 256, 0, st>>>(n_labels, n_gt, w);
-        k_quality_total<<<1, 1024, 0, st>>>(n_labels, N, w);
+        Disk disk{};
+        disk.r = (int)std::min(std::ceil(eps), (double)std::max(H, W));
+        const bool far = disk.r > QUALITY_RADIUS;
+        for (int dy = 0; dy <= QUALITY_RADIUS; ++dy) {
+            disk.half[dy] = -1;
+            for (int dx = 0; !far && dx <= disk.r && !(std::sqrt((double)(dx * dx + dy * dy)) >= eps); ++dx)
+                disk.half[dy] = (signed char)dx;
+        }
+        const unsigned blocks = (unsigned)((long long)((W + 63) / 64) * ((H + 63) / 64));
+        if (far) k_quality_pixels<true><<<blocks, QUALITY_THREADS, 0, st>>>(labels, gt, n_gt, H, W, eps, disk, w);
+        else k_quality_pixels<false><<<blocks, QUALITY_THREADS, 0, st>>>(labels, gt, n_gt, H, W, eps, disk, w);
+        pdl_launch(true, k_quality_rows, dim3((unsigned)((n_labels + 7) / 8)), dim3(256), 0, st, n_labels, n_gt, w);
+        pdl_launch(true, k_quality_total, dim3(1), dim3(1024), 0, st, n_labels, N, w);
         e = cudaGetLastError();
     }
     double r[4];

@@ -843,8 +843,8 @@ def quality_metrics(labels, gt, eps: float = 2.0, stream=None):
 
     stream = stream if stream is not None else torch.cuda.current_stream()
     H, W = int(labels.shape[0]), int(labels.shape[1])
-    n_labels = int(labels.max().item()) + 1
-    n_gt = int(gt.max().item()) + 1
+    # one read-back for both label counts
+    n_labels, n_gt = (int(v) + 1 for v in torch.stack((labels.max(), gt.max())).tolist())
     nbytes = scalp_quality_workspace_bytes(H, W, n_labels, n_gt)
     if nbytes == 0:
         raise ScalpError(SCALP_E_ARG, "invalid sizes for the quality metrics")
