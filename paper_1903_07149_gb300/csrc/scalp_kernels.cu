@@ -366,28 +366,46 @@ void launch_setup_batch(const BatchArgs &b, const SetupInput *in, const int *set
 }
 
 
-__global__ void k_update(SolveArgs a, int from_acc)
+// Small blocks: the update is bound by latency, so its clusters spread out.
+constexpr int UPDATE_THREADS = 64;
+
+template <int LANES>
+__global__ void __launch_bounds__(UPDATE_THREADS) k_update(SolveArgs a, int from_acc)
 {
     pdl_wait();
     pdl_release();
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k < a.Keff) update_cluster(a, k, from_acc);
+    const int t = blockIdx.x * UPDATE_THREADS + (int)threadIdx.x;
+    if (LANES == 1) {
+        if (t < a.Keff) update_cluster(a, t, from_acc);
+    } else {
+        update_cluster_lanes(a, t / LANES, t / LANES < a.Keff, from_acc);
+    }
 }
 
-__global__ void k_update_batch(BatchArgs b, int from_acc)
+template <int LANES>
+__global__ void __launch_bounds__(UPDATE_THREADS) k_update_batch(BatchArgs b, int from_acc)
 {
     pdl_wait();
     pdl_release();
-    const int g = blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= b.clus_base[b.count]) return;
-    const int i = batch_find(b.clus_base, b.count, g);
-    update_cluster(b.args[i], g - b.clus_base[i], from_acc);
+    const int g = (blockIdx.x * UPDATE_THREADS + (int)threadIdx.x) / LANES, total = b.clus_base[b.count];
+    const int gc = min(g, total - 1), i = batch_find(b.clus_base, b.count, gc);
+    if (LANES == 1) {
+        if (g < total) update_cluster(b.args[i], g - b.clus_base[i], from_acc);
+    } else {
+        update_cluster_lanes(b.args[i], gc - b.clus_base[i], g < total, from_acc);
+    }
+}
+
+static unsigned update_blocks(int clusters, bool lanes)
+{
+    return (unsigned)ceil_div_ll((long long)clusters * (lanes ? UPDATE_LANES : 1), UPDATE_THREADS);
 }
 
 void launch_update(const SolveArgs &a, int from_acc, cudaStream_t st, bool pdl)
 {
-    // small blocks: one thread per cluster is latency-bound, so spread them
-    pdl_launch(pdl, k_update, dim3((a.Keff + 63) / 64), dim3(64), 0, st, a, from_acc);
+    const bool lanes = a.Keff <= UPDATE_LANES_MAX;
+    pdl_launch(pdl, lanes ? k_update<UPDATE_LANES> : k_update<1>, dim3(update_blocks(a.Keff, lanes)),
+               dim3(UPDATE_THREADS), 0, st, a, from_acc);
 }
 
 __global__ void __launch_bounds__(PROJ_THREADS) k_project(SolveArgs a, int whole_image)
@@ -560,7 +578,9 @@ void launch_batch_update(const BatchArgs &b, int total_clusters, int total_fill,
                          cudaStream_t side, cudaEvent_t fork, cudaEvent_t join, int whole_image)
 {
     if (b.count <= 0) return;
-    pdl_launch(pdl, k_update_batch, dim3((total_clusters + 63) / 64), dim3(64), 0, st, b, 1);
+    const bool lanes = total_clusters <= UPDATE_LANES_MAX;
+    pdl_launch(pdl, lanes ? k_update_batch<UPDATE_LANES> : k_update_batch<1>,
+               dim3(update_blocks(total_clusters, lanes)), dim3(UPDATE_THREADS), 0, st, b, 1);
     if (side) {  // the lists on a second branch, beside the projection
         cudaEventRecord(fork, st);
         cudaStreamWaitEvent(side, fork, 0);

@@ -115,7 +115,6 @@ __device__ __noinline__ void phase_update(const BatchArgs &b, int total_clusters
     }
 }
 
-
 // The searches of an image whose last assignment left many pixels with no
 // candidate, one CTA per queued cluster: out of line, so that their registers
 // stay out of the other phases' allocation.

@@ -25,16 +25,42 @@ __device__ __forceinline__ bool in_window(long long v, long long n, long long s,
     return lhs <= rhs;
 }
 
-__device__ inline bool window_range(long long n, long long s, long long N, long long K, double r,
-                             int limit, int &lo, int &hi)
+// One end of a window, unclipped: the first (up) or last place inside, from a
+// start at most a few places outside; false when the search finds none.  The
+// places tried lie within r + 3 of s / n, so 64 bits hold both sides when
+// they hold them at that distance (small clusters: no 128-bit products).
+__device__ inline bool window_end(long long n, long long s, long long N, long long K, double r, int limit, bool up,
+                                  long long &end)
+{
+    long long lo, hi;
+    window_start(s, n, r, limit, lo, hi);
+    long long v = up ? lo : hi;
+    const int step = up ? 1 : -1;
+    const float reach = (float)n * ((float)r + 68.0f);  // (64 further places at most)
+    bool in;
+    int guard = 0;
+    if ((float)K * reach * reach < 9.0e18f && (float)N * (float)n * (float)n < 9.0e18f) {
+        const unsigned long long rhs = (unsigned long long)N * (unsigned long long)n * (unsigned long long)n;
+        do {
+            const long long d = n * v - s;
+            in = (unsigned long long)K * (unsigned long long)(d * d) <= rhs;
+            if (!in) v += step;
+        } while (!in && ++guard <= 64);
+    } else {
+        do {
+            in = in_window(v, n, s, N, K);
+            if (!in) v += step;
+        } while (!in && ++guard <= 64);
+    }
+    end = v;
+    return in;
+}
+
+__device__ __forceinline__ bool window_range(long long n, long long s, long long N, long long K, double r, int limit,
+                                             int &lo, int &hi)
 {
     long long l, h;
-    window_start(s, n, r, limit, l, h);
-    int guard = 0;
-    while (!in_window(l, n, s, N, K) && guard++ < 64) ++l;
-    guard = 0;
-    while (!in_window(h, n, s, N, K) && guard++ < 64) --h;
-    if (!in_window(l, n, s, N, K) || !in_window(h, n, s, N, K)) return false;
+    if (!window_end(n, s, N, K, r, limit, true, l) || !window_end(n, s, N, K, r, limit, false, h)) return false;
     lo = (int)max(0LL, l);
     hi = (int)min((long long)limit - 1, h);
     return true;
@@ -93,15 +119,26 @@ __device__ __forceinline__ ProjBest proj_candidate(long long p, int x, int y, lo
 }
 
 // ---------------------------------------------------------------------------
-// Cluster update (Algorithm 1) and everything derived from it, one thread per
-// cluster.  With from_acc: the means over S_k from the integer sums (an empty
-// cluster keeps its colour, barycenter and endpoint), the endpoint X_k rounded
-// half-up, and a projection request (Eq. 4) when the pixel there is not
-// labelled k; the sums are cleared for the next assignment.  Then, from the
-// state: the window, the cluster record the assignment reads, and the count
-// of each tile the window overlaps (for the candidate lists).  The window the
-// last assignment used is kept for the projection search.
+// Cluster update (Algorithm 1) and everything derived from it.  With
+// from_acc: the means over S_k from the integer sums (an empty cluster keeps
+// its colour, barycenter and endpoint), the endpoint X_k rounded half-up, and
+// a projection request (Eq. 4) when the pixel there is not labelled k; the
+// sums are cleared for the next assignment.  Then, from the state: the window,
+// the cluster record the assignment reads, and the count of each tile the
+// window overlaps (for the candidate lists).  The window the last assignment
+// used is kept for the projection search.
+//
+// Two forms with the same results.  Up to UPDATE_LANES_MAX clusters a launch
+// is bound by its chain of dependent steps, and eight lanes take a cluster:
+// on one thread the five FP64 divisions (slow on this part), two 64-bit
+// divisions and four window searches come one after the other (8.4 and 8.6
+// us a launch for 60 and 2000 clusters, 5.4 and 6.5 on eight lanes).  Above
+// it the chip is full and the extra warps only cost (120,000 clusters of a
+// batch: 39.6 us on one thread each, 84.6 on eight lanes).
 // ---------------------------------------------------------------------------
+constexpr int UPDATE_LANES = 8, UPDATE_LANES_MAX = 32768;
+
+// One thread per cluster.
 __device__ __forceinline__ void update_cluster(const SolveArgs &a, int k, int from_acc)
 {
     // every load that does not depend on another is issued first: the
@@ -164,6 +201,124 @@ __device__ __forceinline__ void update_cluster(const SolveArgs &a, int k, int fr
         a.proj_list[slot] = k;
     }
 }
+
+// Eight lanes per cluster.  Lane i holds word i of the sums (n, Sx, Sy, SL,
+// Sa, Sb), so lanes 1-5 divide side by side; lanes 0-3 search one end of the
+// window each; the tiles' counts and the record's stores are spread over the
+// eight.  Called by whole warps; lanes of a cluster past the last pass valid =
+// false.
+__device__ __forceinline__ void update_cluster_lanes(const SolveArgs &a, int k, bool valid, int from_acc)
+{
+    const unsigned FULL = 0xffffffffu;
+    const int j = (int)(threadIdx.x % UPDATE_LANES);
+    const auto from = [&](auto v, int lane) { return __shfl_sync(FULL, v, lane, UPDATE_LANES); };
+    // every load that does not depend on another is issued first
+    ClusterDev old{};
+    long long n = 1, sx = 0, sy = 0, word = 0;
+    float4 col{};
+    int2 e{};
+    if (valid) {
+        old = a.cdev[k];
+        n = a.st_n[k];
+        sx = a.st_sx[k];
+        sy = a.st_sy[k];
+        col = a.st_col[k];
+        e = a.st_end[k];
+        if (from_acc) {
+            static_assert(sizeof(ClusterAcc) == UPDATE_LANES * 8, "one word per lane");
+            unsigned long long *acc = &a.acc[k].n + j;
+            word = (long long)*acc;
+            *acc = 0ull;
+        }
+    }
+    if (from_acc && valid && k == 0 && j == 0) {
+        // the projection searches the orphans of the assignment just finished
+        a.ctr->proj_orphans = atomicExch(&a.ctr->orphans, 0);
+    }
+    const long long n_new = from(word, 0);
+    const bool fresh = n_new > 0;  // (never without from_acc)
+    if (fresh) n = n_new;
+    {
+        const long long tx = from(word, 1), ty = from(word, 2);
+        if (fresh) {
+            sx = tx;
+            sy = ty;
+        }
+    }
+    // lane 1, 2: Sx / n, Sy / n; lanes 3-5: the mean colour
+    float mean = 0.0f;
+    if (j >= 1 && j <= 5) {
+        const long long num = j == 1 ? sx : j == 2 ? sy : word;
+        const double den = j <= 2 ? (double)n : (double)n * (double)(1 << COLOR_FRAC_BITS);
+        mean = (float)((double)num / den);
+    }
+    const float xk = from(mean, 1), yk = from(mean, 2), mL = from(mean, 3), ma = from(mean, 4), mb = from(mean, 5);
+    if (fresh) col = make_float4(mL, ma, mb, 0.f);
+    // even lanes x, odd lanes y: the endpoint, and one end of the window
+    // (lanes 0, 1 the lower, 2, 3 the upper)
+    const long long s = j & 1 ? sy : sx;
+    int end = 0, edge = 0;
+    bool ok = true;
+    if (j < 4) {
+        const unsigned long long num = 2ull * (unsigned long long)s + (unsigned long long)n, den = 2ull * (unsigned long long)n;
+        end = (int)((num | den) >> 32 ? num / den : (unsigned long long)((unsigned)num / (unsigned)den));
+        const int limit = j & 1 ? a.H : a.W;
+        long long v;
+        ok = window_end(n, s, a.N, a.K, a.r, limit, j < 2, v);
+        edge = (int)(j < 2 ? max(0LL, v) : min((long long)limit - 1, v));
+    }
+    const int ex = from(end, 0), ey = from(end, 1);
+    ok = from((int)ok, 0) & from((int)ok, 1) & from((int)ok, 2) & from((int)ok, 3);
+    ClusterDev cd;
+    cd.xlo = from(edge, 0); cd.ylo = from(edge, 1); cd.xhi = from(edge, 2); cd.yhi = from(edge, 3);
+    __syncwarp();  // the cluster's old state is read before its lanes write the new one
+    if (!valid) return;
+    int label_at_end = k;
+    if (fresh) {
+        e = make_int2(ex, ey);
+        // Eq. 4 is needed when the endpoint's pixel is not in S_k; the label
+        // is read now and used last
+        if (j == 0) label_at_end = a.labels[(long long)e.y * a.W + e.x];
+    }
+    if (!ok) {
+        if (j == 0) atomicExch(&a.ctr->error, ERR_BAD_LABEL);
+        cd.xlo = 1; cd.xhi = 0; cd.ylo = 1; cd.yhi = 0;
+    }
+    cd.L = col.x; cd.a = col.y; cd.b = col.z;
+    cd.xk = xk; cd.yk = yk;
+    cd.ex = e.x; cd.ey = e.y;
+    cd.pad = k;
+    if (ok) {
+        // the window's tiles, one per lane in turn (one division for the
+        // lane's first, then steps of UPDATE_LANES)
+        const int tx0 = cd.xlo / TILE_X, ty0 = cd.ylo / TILE_Y;
+        const int nx = cd.xhi / TILE_X - tx0 + 1, nt = nx * (cd.yhi / TILE_Y - ty0 + 1);
+        for (int t = j; t < nt; t += UPDATE_LANES)
+            atomicAdd(&a.tile_count[(ty0 + t / nx) * a.n_tx + tx0 + t % nx], 1);
+    }
+    int4 *rec = reinterpret_cast<int4 *>(&a.cdev[k]);
+    if (j == 1) {
+        rec[0] = make_int4(__float_as_int(cd.L), __float_as_int(cd.a), __float_as_int(cd.b), __float_as_int(cd.xk));
+        a.prev_win[k] = make_int4(old.xlo, old.xhi, old.ylo, old.yhi);
+    } else if (j == 2) {
+        rec[1] = make_int4(__float_as_int(cd.yk), cd.ex, cd.ey, cd.xlo);
+    } else if (j == 3) {
+        rec[2] = make_int4(cd.xhi, cd.ylo, cd.yhi, cd.pad);
+    } else if (fresh && j == 4) {
+        a.st_n[k] = n;
+        a.st_sx[k] = sx;
+    } else if (fresh && j == 5) {
+        a.st_sy[k] = sy;
+        a.st_col[k] = col;
+    } else if (fresh && j == 6) {
+        a.st_end[k] = e;
+    } else if (j == 0 && label_at_end != k) {
+        a.proj_list[atomicAdd(&a.ctr->nproj, 1)] = k;
+    }
+}
+static_assert(offsetof(ClusterDev, xk) == 12 && offsetof(ClusterDev, yk) == 16 && offsetof(ClusterDev, xlo) == 28 &&
+                  offsetof(ClusterDev, xhi) == 32 && offsetof(ClusterDev, pad) == 44,
+              "the record's three quarters");
 
 // S_k lies in the window the last assignment used for cluster k, apart from
 // the pixels that no window reached and that kept their label k.  The
