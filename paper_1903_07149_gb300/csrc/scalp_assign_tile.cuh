@@ -144,15 +144,8 @@ __device__ __forceinline__ int find_slot(const int *cid, int cnt, int k)
 // subtracts P') therefore has a larger D: it can neither win nor tie.  The
 // host turns the pruning off where these estimates do not hold (bound_valid()
 // in scalp_assign.cu: products that could leave the FP32 range, coordinates
-// above 2^24).
-constexpr float BOUND_SCALE = 1.0f - 1.0f / 131072.0f;
-
-// What f . g + K' must exceed for the pair to lose; NaN (no pair loses) for a
-// pixel without a pass-1 D, or with one near the end of the FP32 range.
-__device__ __forceinline__ float bound_threshold(float D, float P)
-{
-    return D < 1e30f ? fmaf(D, 1.0f + 1.0f / 1048576.0f, -BOUND_SCALE * P) : __int_as_float(0x7fffffff);
-}
+// above 2^24).  BOUND_SCALE and bound_threshold() are in scalp_internal.cuh
+// (the supervoxels use them too).
 
 __device__ __forceinline__ unsigned long long pack_best(float D, int slot)
 {

@@ -552,6 +552,16 @@ __device__ __forceinline__ float scalp_distance(float dcp, float sum_dc, float s
     return fmaf(dcol, dcon, ms2 * ds);
 }
 
+// The pruning bound's scale and threshold (see scalp_assign_tile.cuh).
+constexpr float BOUND_SCALE = 1.0f - 1.0f / 131072.0f;
+
+// What f . g + K' must exceed for the pair to lose; NaN (no pair loses) for a
+// pixel without a pass-1 D, or with one near the end of the FP32 range.
+__device__ __forceinline__ float bound_threshold(float D, float P)
+{
+    return D < 1e30f ? fmaf(D, 1.0f + 1.0f / 1048576.0f, -BOUND_SCALE * P) : __int_as_float(0x7fffffff);
+}
+
 // ---------------------------------------------------------------------------
 // Warp-aggregated segmented reduction.  Lanes holding the same key are summed
 // with warp reductions and the group's first lane hands the sums to `sink`.

@@ -61,6 +61,7 @@ struct VoxArgs {
     int tpw_x, tpw_y, tpw_t;  // bound on the tiles one window spans, per axis
     long long tile_cap;
     int count_samples;
+    int prune;                // 1: skip pairs whose lower bound exceeds the voxel's pass-1 D
     const float4 *plane;      // (L, a, b, w) per voxel
     int *labels;
     long long *st_n, *st_sx, *st_sy, *st_st;
@@ -506,16 +507,10 @@ __device__ __forceinline__ int vpath_sums(const float4 *__restrict__ plane, int 
     return ns + 1;
 }
 
-// Work items: the voxels of the tile inside candidate c's window form a box
-// (x fastest, then y, then t: a warp's paths then start in neighbouring
-// columns, so their global-memory samples share cache lines; ordering by the
-// paths' dominant axis instead was measured slower); every 32 consecutive
-// voxels of it are one warp's item.  Lanes walk their voxel's path and take a 64-bit shared-memory
-// atomicMin of (D bits, candidate slot); slots follow the cluster index, so
-// ties go to the smallest k.  A tile with more than VITEM_CAND candidates
+// Candidate clusters of one tile held in shared memory; a tile with more
 // evaluates voxel by voxel over the global list instead.
-constexpr int VITEM_CAND = 128;
-constexpr int VMAX_ITEMS = VITEM_CAND * (VTILE / 32);
+constexpr int VCAND = 128;
+constexpr int VQUEUE = 96;  // pairs a warp's queue holds (pass 2)
 
 __device__ __forceinline__ unsigned long long vpack_best(float D, int slot)
 {
@@ -534,186 +529,195 @@ __device__ __forceinline__ int vfind_slot(const int *ids, int cnt, int k)
     return lo < cnt && ids[lo] == k ? lo : -1;
 }
 
-// The pruning of the 2-D assignment, in 3-D.  Pass 1 evaluates each voxel's
-// previous label (when it is a candidate of the voxel); pass 2 skips every
-// other candidate whose FP32 lower bound fl(fl(lam*d_c(p)) + fl(m^2/r^2*d_s))
-// exceeds the voxel's best D so far (the computed D is never below that
-// bound: dcol >= fl(lam*dcp), dcon >= 1, and rounding is monotone), so the
-// argmin is unchanged; the surviving pairs are queued per warp and walked 32
-// at a time.
+// The assignment of one tile, a voxel per thread, pruned as in 2-D.  Each warp
+// (32 voxels, 16 columns x 2 rows of a frame) works alone after the set-up:
+// pass 1 evaluates each voxel's previous label (when it is a candidate of the
+// voxel); pass 2 checks the other candidates whose boxes meet the warp's
+// voxels against a lower bound of D, queues the pairs it cannot rule out and
+// walks them 32 at a time.  The bound is the 2-D one with one axis more
+// (scalp_assign_tile.cuh: q = P + K + f . g, its rounding covered by the same
+// margin), six multiply-adds on values in registers.  Its first form cut each
+// candidate's box into 32-voxel items taken from a shared counter, each lane
+// reading its voxel's sample and forming both squared distances, behind six
+// block barriers instead of one or two: 226 us a launch on 32 x 240 x 320 with
+// 2000 clusters, 200 now (185.7 M against 164.3 M warp instructions; the walks
+// are most of what is left).
+//
+// Per candidate (slot c): the record, and for the bound
+//   s_rec = (box, K bits, g_x bits, g_y bits), s_col = (c, g_t)
+// with the box as one bit per column (0-15), row (16-23) and frame (24-27) of
+// the tile.
 __global__ void __launch_bounds__(VTILE) k_vassign(VoxArgs a)
 {
-    __shared__ VoxCluster cand[VITEM_CAND];
-    __shared__ int s_sorted[VITEM_CAND];   // candidate ids in slot order
-    __shared__ unsigned char s_prev[VTILE];  // each voxel's previous label as a slot, 0xff if none
-    __shared__ unsigned s_queue[VTILE / 32][64];
-    __shared__ int4 s_box[VITEM_CAND];     // (xa, ya, ta, w | h << 8 | d << 16)
-    __shared__ int2 s_rcp[VITEM_CAND];     // 16-bit reciprocals of w and h
-    __shared__ int s_ids[VITEM_CAND];
-    __shared__ int s_nit[VITEM_CAND];
-    __shared__ int s_first[VITEM_CAND + 1];
-    __shared__ unsigned char s_owner[VMAX_ITEMS];
+    static_assert(VTX == 16 && VTY == 8 && VTT == 4, "a box is 16 + 8 + 4 bits, a warp 16 x 2 voxels");
+    __shared__ VoxCluster cand[VCAND];
+    __shared__ int4 s_rec[VCAND];
+    __shared__ float4 s_col[VCAND];
+    __shared__ int s_sorted[VCAND];   // candidate ids in slot order
+    __shared__ int s_ids[VCAND];
+    __shared__ uint16_t s_queue[VTILE / 32][VQUEUE];  // slot << 5 | lane
     __shared__ unsigned long long s_best[VTILE];
-    __shared__ int s_counter;
+    const unsigned FULL = 0xffffffffu;
     pdl_wait();
     pdl_release();
     const int tile = blockIdx.x;
     const int tx = tile % a.n_tx, ty = (tile / a.n_tx) % a.n_ty, tt = tile / (a.n_tx * a.n_ty);
     const int x0 = tx * VTX, y0 = ty * VTY, t0 = tt * VTT;
-    const int tid = threadIdx.x, lane = tid & 31;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int lx = tid % VTX, ly = (tid / VTX) % VTY, lt = tid / (VTX * VTY);
     const int x = x0 + lx, y = y0 + ly, t = t0 + lt;
     const bool valid = x < a.W && y < a.H && t < a.T;
     const int off = a.tile_off[tile];
     const int cnt = (int)max(0LL, min((long long)a.tile_off[tile + 1], a.tile_cap) - off);
-    const bool fast = cnt <= VITEM_CAND;
+    const bool fast = cnt <= VCAND;
     const long long p = ((long long)t * a.H + y) * a.W + x;
     unsigned my_samples = 0, my_pairs = 0;
     int lab = -1;
     const int prev = fast && valid ? a.labels[p] : -1;  // overlaps the set-up
 
     if (fast) {
-        // candidates sorted by cluster index (ranks of distinct ids)
-        int myid = INT_MAX;
-        if (tid < cnt) {
-            myid = a.tile_list[off + tid];
-            s_ids[tid] = myid;
-        }
-        s_best[tid] = ~0ull;
-        if (tid == 0) s_counter = 0;
-        __syncthreads();
-        if (tid < cnt) {
-            int rank = 0;
-            for (int j = 0; j < cnt; ++j) rank += s_ids[j] < myid;
-            const VoxCluster cd = a.cdev[myid];
+        const auto write_records = [&](int rank, int id, const VoxCluster &cd) {
             cand[rank] = cd;
-            s_sorted[rank] = myid;
+            s_sorted[rank] = id;
             const int xa = max(cd.xlo, x0), xb = min(min(cd.xhi, x0 + VTX - 1), a.W - 1);
             const int ya = max(cd.ylo, y0), yb = min(min(cd.yhi, y0 + VTY - 1), a.H - 1);
             const int ta = max(cd.tlo, t0), tb = min(min(cd.thi, t0 + VTT - 1), a.T - 1);
-            const int w = max(xb - xa + 1, 0), h = max(yb - ya + 1, 0), d = max(tb - ta + 1, 0);
-            s_box[rank] = make_int4(xa, ya, ta, w | (h << 8) | (d << 16));
-            s_rcp[rank] = make_int2((65536 + max(w, 1) - 1) / max(w, 1), (65536 + max(h, 1) - 1) / max(h, 1));
-            s_nit[rank] = (w * h * d + 31) >> 5;
-        }
-        __syncthreads();
-        if (tid < 32) {  // exclusive prefix of the item counts
-            constexpr int PER = VITEM_CAND / 32;
-            int v[PER], sum = 0;
-#pragma unroll
-            for (int i = 0; i < PER; ++i) {
-                const int c = lane * PER + i;
-                v[i] = c < cnt ? s_nit[c] : 0;
-                sum += v[i];
-            }
-            int incl = sum;
-            for (int o = 1; o < 32; o <<= 1) {
-                const int u = __shfl_up_sync(0xffffffffu, incl, o);
-                if (lane >= o) incl += u;
-            }
-            int run = incl - sum;
-#pragma unroll
-            for (int i = 0; i < PER; ++i) {
-                const int c = lane * PER + i;
-                if (c < cnt) s_first[c] = run;
-                run += v[i];
-            }
-            if (lane == 31) s_first[cnt] = incl;
-        }
-        __syncthreads();
-        if (tid < cnt) {
-            const int f = s_first[tid], n = s_nit[tid];
-            for (int j = 0; j < n; ++j) s_owner[f + j] = (unsigned char)tid;
-        }
-        // this voxel's previous label as a slot when the voxel is in that box
-        int pslot = prev >= 0 ? vfind_slot(s_sorted, cnt, prev) : -1;
-        if (pslot >= 0) {
-            const int4 b = s_box[pslot];
-            if (x < b.x || x >= b.x + (b.w & 0xff) || y < b.y || y >= b.y + ((b.w >> 8) & 0xff) || t < b.z ||
-                t >= b.z + (b.w >> 16))
-                pslot = -1;
-        }
-        s_prev[tid] = (unsigned char)(pslot >= 0 ? pslot : 0xff);
-        __syncthreads();
-        // D of voxel (qx, qy, qt) for candidate slot c, from its own sample
-        auto own_dc = [&](int qx, int qy, int qt, const VoxCluster &cd) {
-            return colour_dist(__ldg(a.plane + ((long long)qt * a.H + qy) * a.W + qx), cd.L, cd.a, cd.b);
+            unsigned box = 0u;
+            if (xa <= xb && ya <= yb && ta <= tb)
+                box = (0xffffffffu >> (31 - (xb - xa))) << (xa - x0) |
+                      (0xffffffffu >> (31 - (yb - ya))) << (ya - y0 + 16) |
+                      (0xffffffffu >> (31 - (tb - ta))) << (ta - t0 + 24);
+            const float kx = cd.xk - (float)x0, ky = cd.yk - (float)y0, kt = cd.tk - (float)t0;
+            const float K = BOUND_SCALE * fmaf(a.lam, fmaf(cd.L, cd.L, fmaf(cd.a, cd.a, cd.b * cd.b)),
+                                               a.ms2 * fmaf(kx, kx, fmaf(ky, ky, kt * kt)));
+            s_rec[rank] = make_int4((int)box, __float_as_int(K), __float_as_int(-2.0f * a.ms2 * kx),
+                                    __float_as_int(-2.0f * a.ms2 * ky));
+            s_col[rank] = make_float4(cd.L, cd.a, cd.b, -2.0f * a.ms2 * kt);
         };
-        auto vspatial = [&](int qx, int qy, int qt, const VoxCluster &cd) {
-            const float ddx = (float)qx - cd.xk, ddy = (float)qy - cd.yk, ddt = (float)qt - cd.tk;
-            return fmaf(ddx, ddx, fmaf(ddy, ddy, ddt * ddt));
-        };
-        auto evaluate = [&](int qx, int qy, int qt, int c) {
+        // candidates sorted by cluster index (ranks of distinct ids): by one
+        // warp with shuffles when they fit its lanes
+        if (cnt <= 32) {
+            if (warp == 0) {
+                int myid = INT_MAX;
+                VoxCluster cd;
+                if (lane < cnt) {
+                    myid = a.tile_list[off + lane];
+                    cd = a.cdev[myid];
+                }
+                int rank = 0;
+                for (int j = 0; j < 32; ++j) rank += __shfl_sync(FULL, myid, j) < myid;
+                if (lane < cnt) write_records(rank, myid, cd);
+            }
+        } else {
+            int myid = INT_MAX;
+            if (tid < cnt) {
+                myid = a.tile_list[off + tid];
+                s_ids[tid] = myid;
+            }
+            __syncthreads();
+            if (tid < cnt) {
+                int rank = 0;
+                for (int j = 0; j < cnt; ++j) rank += s_ids[j] < myid;
+                write_records(rank, myid, a.cdev[myid]);
+            }
+        }
+        __syncthreads();
+        // D of the warp's voxel v (a lane) for candidate slot c
+        const int wy = y0 + (ly & ~1);  // the warp's first row
+        const auto evaluate = [&](int v, int c, int &len) {
             const VoxCluster &cd = cand[c];
+            const int qx = x0 + (v & 15), qy = wy + (v >> 4);
+            const float dcp = colour_dist(__ldg(a.plane + ((long long)t * a.H + qy) * a.W + qx), cd.L, cd.a, cd.b);
             float sdc, sw;
-            const int len = vpath_sums(a.plane, a.W, a.HW, qx, qy, qt, cd.ex, cd.ey, cd.et, cd.L, cd.a, cd.b,
-                                       sdc, sw);
-            const float D = scalp_distance(own_dc(qx, qy, qt, cd), sdc, sw, len, a.lam, a.gamma, a.ms2,
-                                           vspatial(qx, qy, qt, cd));
-            atomicMin(&s_best[((qt - t0) * VTY + (qy - y0)) * VTX + (qx - x0)], vpack_best(D, c));
+            len = vpath_sums(a.plane, a.W, a.HW, qx, qy, t, cd.ex, cd.ey, cd.et, cd.L, cd.a, cd.b, sdc, sw);
+            const float ddx = (float)qx - cd.xk, ddy = (float)qy - cd.yk, ddt = (float)t - cd.tk;
+            return scalp_distance(dcp, sdc, sw, len, a.lam, a.gamma, a.ms2, fmaf(ddx, ddx, fmaf(ddy, ddy, ddt * ddt)));
+        };
+        const auto count_pair = [&](int len) {
             my_samples += len;
             my_pairs += 1;
         };
-        // pass 1: the previous label (no barrier before pass 2: a voxel whose
-        // pass 1 is still running elsewhere is simply not pruned yet)
-        if (pslot >= 0) evaluate(x, y, t, pslot);
-        // pass 2: the candidates' boxes, cut into items; survivors queued
-        unsigned *wq = s_queue[tid >> 5];
-        const unsigned lanes_below = (1u << lane) - 1u;
-        int queued = 0;
-        auto walk_queued = [&](unsigned e) {
-            const int v = (int)(e & (VTILE - 1)), c = (int)(e >> 9);
-            evaluate(x0 + v % VTX, y0 + (v / VTX) % VTY, t0 + v / (VTX * VTY), c);
-        };
-        static_assert(VTILE == 512, "queued pairs are (slot << 9 | voxel)");
-        const int n_items = s_first[cnt];
-        while (true) {
-            int item = 0;
-            if (lane == 0) item = atomicAdd(&s_counter, 1);
-            item = __shfl_sync(0xffffffffu, item, 0);
-            if (item >= n_items) break;
-            const int c = s_owner[item];
-            const int4 b = s_box[c];
-            const int w = b.w & 0xff, h = (b.w >> 8) & 0xff, d = b.w >> 16;
-            const int j = ((item - s_first[c]) << 5) + lane;
-            bool keep = false;
-            int vox = 0;
-            if (j < w * h * d) {
-                const int2 r = s_rcp[c];
-                // exact: j < 512 and w, h <= 16, so the 16-bit reciprocals give floor
-                const int q = (j * r.x) >> 16;  // j / w
-                const int qx = b.x + (j - q * w);
-                const int qt = (q * r.y) >> 16;  // q / h
-                const int qy = b.y + (q - qt * h);
-                const int qtt = b.z + qt;
-                vox = ((qtt - t0) * VTY + (qy - y0)) * VTX + (qx - x0);
-                if (s_prev[vox] != c) {  // else evaluated in pass 1
-                    const VoxCluster &cd = cand[c];
-                    const float lb = __fadd_rn(__fmul_rn(a.lam, own_dc(qx, qy, qtt, cd)),
-                                               __fmul_rn(a.ms2, vspatial(qx, qy, qtt, cd)));
-                    // s_best holds (D bits, slot); all ones (a NaN) until a D arrives
-                    keep = !(lb > __uint_as_float((unsigned)(s_best[vox] >> 32)));
-                    if (!keep) {  // cannot win: not walked (counted as the method's work)
-                        my_samples += max(abs(qx - cd.ex), max(abs(qy - cd.ey), abs(qtt - cd.et))) + 1;
-                        my_pairs += 1;
-                    }
-                }
+        // pass 1: the previous label, when the voxel is in its box
+        const unsigned bits = 1u << lx | 1u << (16 + ly) | 1u << (24 + lt);
+        int slot = prev >= 0 ? vfind_slot(s_sorted, cnt, prev) : -1;
+        if (slot >= 0 && ((unsigned)s_rec[slot].x & bits) != bits) slot = -1;
+        float dprev = __int_as_float(0x7fffffff);  // NaN: none
+        unsigned long long mine = ~0ull;
+        if (slot >= 0) {
+            int len;
+            dprev = evaluate(lane, slot, len);
+            mine = vpack_best(dprev, slot);
+            count_pair(len);
+        }
+        s_best[tid] = mine;
+        __syncwarp();
+        // pass 2: the other candidates
+        uint16_t *wq = s_queue[warp];
+        const unsigned warp_rows = 3u << (16 + (ly & ~1)), warp_frame = 1u << (24 + lt);
+        int queued = 0, c0 = -32;  // warp-uniform, as all that follows
+        unsigned any = 0u;         // candidates c0 + bit that meet the warp's voxels and are left
+        for (bool more = true; more;) {
+            const float X = (float)lx, Y = (float)ly, Z = (float)lt;
+            float fL, fa, fb, thr;
+            {
+                const float4 v = valid ? __ldg(a.plane + p) : make_float4(0.f, 0.f, 0.f, 0.f);
+                thr = a.prune ? bound_threshold(dprev, fmaf(a.lam, fmaf(v.x, v.x, fmaf(v.y, v.y, v.z * v.z)),
+                                                            a.ms2 * fmaf(X, X, fmaf(Y, Y, Z * Z))))
+                              : __int_as_float(0x7fffffff);
+                fL = -2.0f * a.lam * v.x;
+                fa = -2.0f * a.lam * v.y;
+                fb = -2.0f * a.lam * v.z;
             }
-            const unsigned kept = __ballot_sync(0xffffffffu, keep);
-            if (keep) wq[queued + __popc(kept & lanes_below)] = ((unsigned)c << 9) | (unsigned)vox;
-            queued += __popc(kept);
-            __syncwarp();
-            if (queued >= 32) {
-                const unsigned e = wq[lane];
+            const unsigned lanes_below = (1u << lane) - 1u;
+            while (queued <= VQUEUE - 32) {
+                if (!any) {
+                    c0 += 32;
+                    more = c0 < cnt;
+                    if (!more) break;
+                    const unsigned m = c0 + lane < cnt ? (unsigned)s_rec[c0 + lane].x : 0u;
+                    any = __ballot_sync(FULL, (m & warp_rows) && (m & warp_frame));
+                    continue;
+                }
+                const int c = c0 + __ffs(any) - 1;
+                any &= any - 1;
+                const int4 r = s_rec[c];
+                const float4 ck = s_col[c];
+                // (a voxel of the box lies in the volume)
+                const bool in = ((unsigned)r.x & bits) == bits && c != slot;
+                const float bound =
+                    fmaf(fL, ck.x, fmaf(fa, ck.y, fmaf(fb, ck.z, fmaf(X, __int_as_float(r.z),
+                                        fmaf(Y, __int_as_float(r.w), fmaf(Z, ck.w, __int_as_float(r.y)))))));
+                const bool loses = bound > thr;
+                if (a.count_samples && in && loses) {
+                    // a pair that cannot win is not walked (counted as the method's work)
+                    const VoxCluster &cd = cand[c];
+                    count_pair(max(abs(x - cd.ex), max(abs(y - cd.ey), abs(t - cd.et))) + 1);
+                }
+                const bool keep = in && !loses;
+                const unsigned kept = __ballot_sync(FULL, keep);
+                if (keep) wq[queued + __popc(kept & lanes_below)] = (uint16_t)(c << 5 | lane);
+                queued += __popc(kept);
+            }
+            __syncwarp();  // the queued pairs
+            int done = 0;
+#pragma unroll 1
+            for (; more ? done + 32 <= queued : done < queued; done += 32) {
+                if (done + lane >= queued) continue;
+                const int e = wq[done + lane], v = e & 31, c = e >> 5;
+                int len;
+                const float D = evaluate(v, c, len);
+                atomicMin(&s_best[warp * 32 + v], vpack_best(D, c));
+                count_pair(len);
+            }
+            if (more) {  // the pairs left over start the next queue
+                queued -= done;
+                const uint16_t e = lane < queued ? wq[done + lane] : (uint16_t)0;
                 __syncwarp();
-                if (lane < queued - 32) wq[lane] = wq[32 + lane];
-                queued -= 32;
+                if (lane < queued) wq[lane] = e;
                 __syncwarp();
-                walk_queued(e);
             }
         }
-        if (lane < queued) walk_queued(wq[lane]);
-        __syncthreads();
+        __syncwarp();
         if (valid) {
             const unsigned long long bb = s_best[tid];
             // slot -> cluster index (the record's pad field holds k)
@@ -987,6 +991,7 @@ int scalp_voxel_init(scalp_vctx **out, const scalp_volume *vol, int32_t K, float
     a.lam = params->lambda;
     a.gamma = (float)c->gamma;
     a.ms2 = (float)((double)m * (double)m / (c->r * c->r));
+    a.prune = bound_valid(c->H, c->W, a.lam, a.ms2) ? 1 : 0;
     a.n_tx = L.n_tx; a.n_ty = L.n_ty; a.n_tt = L.n_tt;
     a.tpw_x = L.tpw_x; a.tpw_y = L.tpw_y; a.tpw_t = L.tpw_t;
     a.tile_cap = L.tile_cap;
