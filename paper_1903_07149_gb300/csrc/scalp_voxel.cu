@@ -14,10 +14,11 @@
 //   * update and projection (Eq. 4) as in 2-D, with the voxel index as the
 //     tie-break; there is no connectivity step.
 //
-// One iteration is four kernels: assignment (one 512-thread CTA per 16x8x4
+// One iteration is three kernels: assignment (one 512-thread CTA per 16x8x4
 // tile, one voxel per thread, paths walked in global memory, warp-aggregated
-// integer sums), update (one thread per cluster), projection (one CTA per
-// queued cluster), candidate lists (count scan, then slot fill).
+// integer sums), update (eight lanes per cluster), and one launch for the
+// candidate lists (count scan and slot fill) and the projection (one CTA per
+// queued cluster).
 #include <algorithm>
 #include <cfloat>
 #include <climits>
@@ -101,16 +102,18 @@ __device__ __forceinline__ bool vin_window(long long v, long long n, long long s
     return lhs <= rhs;
 }
 
-__device__ __forceinline__ void vwindow(long long n, long long s, long long N, long long K, double r, int lim,
-                                        int &lo, int &hi)
+// One end of a window clipped to [0, lim): the first (up) or last place inside
+// (past the other end's start when none is: the window is empty).
+__device__ __forceinline__ int vwindow_end(long long n, long long s, long long N, long long K, double r, int lim,
+                                           bool up)
 {
-    long long a0, b0;
-    window_start(s, n, r, lim, a0, b0);
-    int a = (int)max(a0, 0LL), b = (int)min(b0, (long long)lim - 1);
-    while (a <= b && !vin_window(a, n, s, N, K, r)) ++a;
-    while (b >= a && !vin_window(b, n, s, N, K, r)) --b;
-    lo = a;
-    hi = b;
+    long long lo, hi;
+    window_start(s, n, r, lim, lo, hi);
+    const int first = (int)max(lo, 0LL), last = (int)min(hi, (long long)lim - 1);
+    int v = up ? first : last;
+    const int step = up ? 1 : -1;
+    while (v >= first && v <= last && !vin_window(v, n, s, N, K, r)) v += step;
+    return v;
 }
 
 // ---------------------------------------------------------------------------
@@ -201,57 +204,110 @@ __global__ void __launch_bounds__(256) k_vsetup(VoxArgs a, const uint8_t *__rest
 // ---------------------------------------------------------------------------
 // Update: means, endpoint, projection request, window, record, tile counts.
 // ---------------------------------------------------------------------------
-__global__ void k_vupdate(VoxArgs a, int from_acc)
+// Eight lanes per cluster, as in 2-D (scalp_phases.cuh): lane i holds word i
+// of the sums, lanes 1-6 divide side by side, lanes 0-5 search one end of the
+// window each, and the stores are spread (12.3 us a launch for 2000 clusters
+// on one thread each, 7.5 now).
+constexpr int VUPDATE_LANES = 8, VUPDATE_THREADS = 64;
+
+__global__ void __launch_bounds__(VUPDATE_THREADS) k_vupdate(VoxArgs a, int from_acc)
 {
     pdl_wait();
     pdl_release();
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= a.Keff) return;
-    if (from_acc) {
-        const VoxAcc c = a.acc[k];
-        a.acc[k] = VoxAcc{};
-        const long long n = (long long)c.n;
-        if (n > 0) {
-            const long long sx = (long long)c.sx, sy = (long long)c.sy, st = (long long)c.st;
-            a.st_n[k] = n;
-            a.st_sx[k] = sx;
-            a.st_sy[k] = sy;
-            a.st_st[k] = st;
-            const double den = (double)n * (double)(1 << COLOR_FRAC_BITS);
-            a.st_col[k] = make_float4((float)((double)(long long)c.sL / den),
-                                      (float)((double)(long long)c.sa / den),
-                                      (float)((double)(long long)c.sb / den), 0.f);
-            const int ex = (int)((2 * sx + n) / (2 * n));
-            const int ey = (int)((2 * sy + n) / (2 * n));
-            const int et = (int)((2 * st + n) / (2 * n));
-            a.st_end[k] = make_int4(ex, ey, et, 0);
-            if (a.labels[((long long)et * a.H + ey) * a.W + ex] != k)
-                a.proj_list[atomicAdd(&a.ctr->nproj, 1)] = k;
-        }
-    }
-    const long long n = a.st_n[k], sx = a.st_sx[k], sy = a.st_sy[k], st = a.st_st[k];
+    const unsigned FULL = 0xffffffffu;
+    const int g = (blockIdx.x * VUPDATE_THREADS + (int)threadIdx.x) / VUPDATE_LANES;
+    const int k = min(g, a.Keff - 1), j = (int)(threadIdx.x % VUPDATE_LANES);
+    const bool valid = g < a.Keff;
+    const auto from = [&](auto v, int lane) { return __shfl_sync(FULL, v, lane, VUPDATE_LANES); };
     const VoxCluster old = a.cdev[k];
-    int *pw = a.prev_win + 6 * (long long)k;
-    pw[0] = old.xlo; pw[1] = old.xhi; pw[2] = old.ylo; pw[3] = old.yhi; pw[4] = old.tlo; pw[5] = old.thi;
+    long long n = a.st_n[k], sx = a.st_sx[k], sy = a.st_sy[k], st = a.st_st[k], word = 0;
+    float4 col = a.st_col[k];
+    int4 e = a.st_end[k];
+    if (from_acc && valid) {
+        static_assert(sizeof(VoxAcc) == VUPDATE_LANES * 8, "one word per lane");
+        unsigned long long *acc = &a.acc[k].n + j;
+        word = (long long)*acc;
+        *acc = 0ull;
+        // the projection searches the orphans of the assignment just finished
+        if (k == 0 && j == 0) a.ctr->proj_orphans = atomicExch(&a.ctr->orphans, 0);
+    }
+    const long long n_new = from(word, 0), nsx = from(word, 1), nsy = from(word, 2), nst = from(word, 3);
+    const bool fresh = n_new > 0;  // an empty cluster keeps its state
+    if (fresh) {
+        n = n_new;
+        sx = nsx;
+        sy = nsy;
+        st = nst;
+    }
+    const auto axis = [&](int i) { return i == 0 ? sx : i == 1 ? sy : st; };
+    float mean = 0.0f;  // lanes 1-3: the barycenter, 4-6: the mean colour
+    if (j >= 1 && j <= 6) {
+        const double den = j <= 3 ? (double)n : (double)n * (double)(1 << COLOR_FRAC_BITS);
+        mean = (float)((double)(j <= 3 ? axis(j - 1) : word) / den);
+    }
     VoxCluster cd;
-    const float4 col = a.st_col[k];
-    const int4 e = a.st_end[k];
+    cd.xk = from(mean, 1); cd.yk = from(mean, 2); cd.tk = from(mean, 3);
+    const float mL = from(mean, 4), ma = from(mean, 5), mb = from(mean, 6);
+    if (fresh) col = make_float4(mL, ma, mb, 0.f);
+    int end = 0, edge = 0;  // axis j mod 3: the endpoint, and the lower (0-2) or upper (3-5) end of the window
+    if (j < 6) {
+        const int i = j % 3;
+        const long long s = axis(i);
+        const unsigned long long num = 2ull * (unsigned long long)s + (unsigned long long)n, den = 2ull * (unsigned long long)n;
+        end = (int)((num | den) >> 32 ? num / den : (unsigned long long)((unsigned)num / (unsigned)den));
+        edge = vwindow_end(n, s, a.N, a.K, a.r, i == 0 ? a.W : i == 1 ? a.H : a.T, j < 3);
+    }
+    const int ex = from(end, 0), ey = from(end, 1), et = from(end, 2);
+    cd.xlo = from(edge, 0); cd.ylo = from(edge, 1); cd.tlo = from(edge, 2);
+    cd.xhi = from(edge, 3); cd.yhi = from(edge, 4); cd.thi = from(edge, 5);
+    __syncwarp();  // the cluster's old state is read before its lanes write the new one
+    if (!valid) return;
+    int label_at_end = k;
+    if (fresh) {
+        e = make_int4(ex, ey, et, 0);
+        if (j == 0) label_at_end = a.labels[((long long)et * a.H + ey) * a.W + ex];
+    }
     cd.L = col.x; cd.a = col.y; cd.b = col.z;
-    cd.xk = (float)((double)sx / (double)n);
-    cd.yk = (float)((double)sy / (double)n);
-    cd.tk = (float)((double)st / (double)n);
     cd.ex = e.x; cd.ey = e.y; cd.et = e.z;
     cd.pad = k;
-    vwindow(n, sx, a.N, a.K, a.r, a.W, cd.xlo, cd.xhi);
-    vwindow(n, sy, a.N, a.K, a.r, a.H, cd.ylo, cd.yhi);
-    vwindow(n, st, a.N, a.K, a.r, a.T, cd.tlo, cd.thi);
-    a.cdev[k] = cd;
-    if (cd.xlo > cd.xhi || cd.ylo > cd.yhi || cd.tlo > cd.thi) return;
-    for (int tt = cd.tlo / VTT; tt <= cd.thi / VTT; ++tt)
-        for (int ty = cd.ylo / VTY; ty <= cd.yhi / VTY; ++ty)
-            for (int tx = cd.xlo / VTX; tx <= cd.xhi / VTX; ++tx)
-                atomicAdd(&a.tile_count[(tt * a.n_ty + ty) * a.n_tx + tx], 1);
+    if (cd.xlo <= cd.xhi && cd.ylo <= cd.yhi && cd.tlo <= cd.thi) {
+        const int tx0 = cd.xlo / VTX, ty0 = cd.ylo / VTY, tt0 = cd.tlo / VTT;
+        const int nx = cd.xhi / VTX - tx0 + 1, ny = cd.yhi / VTY - ty0 + 1, nt = nx * ny * (cd.thi / VTT - tt0 + 1);
+        for (int i = j; i < nt; i += VUPDATE_LANES) {
+            const int row = i / nx, fr = row / ny;
+            atomicAdd(&a.tile_count[((tt0 + fr) * a.n_ty + ty0 + row - fr * ny) * a.n_tx + tx0 + i - row * nx], 1);
+        }
+    }
+    int4 *rec = reinterpret_cast<int4 *>(&a.cdev[k]);
+    const auto fi = [](float v) { return __float_as_int(v); };
+    if (j == 1) {
+        rec[0] = make_int4(fi(cd.L), fi(cd.a), fi(cd.b), fi(cd.xk));
+        if (fresh) a.st_col[k] = col;
+    } else if (j == 2) {
+        rec[1] = make_int4(fi(cd.yk), fi(cd.tk), cd.ex, cd.ey);
+        if (fresh) a.st_end[k] = e;
+    } else if (j == 3) {
+        rec[2] = make_int4(cd.et, cd.xlo, cd.xhi, cd.ylo);
+    } else if (j == 4) {
+        rec[3] = make_int4(cd.yhi, cd.tlo, cd.thi, cd.pad);
+    } else if (j == 5) {
+        int2 *pw = reinterpret_cast<int2 *>(a.prev_win + 6 * (long long)k);
+        pw[0] = make_int2(old.xlo, old.xhi);
+        pw[1] = make_int2(old.ylo, old.yhi);
+        pw[2] = make_int2(old.tlo, old.thi);
+    } else if (fresh && j == 6) {
+        a.st_n[k] = n;
+        a.st_sx[k] = sx;
+    } else if (fresh && j == 7) {
+        a.st_sy[k] = sy;
+        a.st_st[k] = st;
+    } else if (j == 0 && label_at_end != k) {
+        a.proj_list[atomicAdd(&a.ctr->nproj, 1)] = k;
+    }
 }
+static_assert(offsetof(VoxCluster, yk) == 16 && offsetof(VoxCluster, ex) == 24 && offsetof(VoxCluster, et) == 32 &&
+                  offsetof(VoxCluster, yhi) == 48 && offsetof(VoxCluster, pad) == 60,
+              "the record's four quarters");
 
 // ---------------------------------------------------------------------------
 // Projection (Eq. 4) of the queued clusters: argmin over the voxels labelled
@@ -301,15 +357,64 @@ __device__ __forceinline__ void vshfl_min(VBest &b)
     }
 }
 
-__global__ void __launch_bounds__(VPROJ_THREADS) k_vproject(VoxArgs a, int whole)
+// The voxels of one box for cluster k, thread t of `threads`: eight label loads
+// before any is compared where the box's rows and frames come from exact 32-bit
+// reciprocals and 64 bits hold the squared distances; the matches one by one
+// (compact code: it is cold on every launch).
+__device__ __forceinline__ void vproject_scan(const VoxArgs &a, int k, long long n, long long sx, long long sy,
+                                              long long st, bool small, int xlo, int ylo, int tlo, long long w,
+                                              long long h, long long vol, int t, int threads, VBest &b)
 {
-    pdl_wait();
-    pdl_release();
+    constexpr int VB = 8;
+    // voxel i of the box: row i / w, frame row / h
+    const RowDiv div_w(w, vol), div_h(h, w > 0 ? vol / w : 0);
+    if (div_w.fast && (div_h.fast || h == 1) && small) {
+        const unsigned end = (unsigned)vol;  // (vol * w < 2^32)
+        const auto place = [&](unsigned i, int &x, int &y, int &z) {
+            const unsigned row = __umulhi(i, div_w.rcp), fr = h == 1 ? row : __umulhi(row, div_h.rcp);
+            x = xlo + (int)(i - row * (unsigned)w);
+            y = ylo + (int)(row - fr * (unsigned)h);
+            z = tlo + (int)fr;
+        };
+        for (unsigned base = (unsigned)t; base < end; base += (unsigned)(threads * VB)) {
+            unsigned match = 0u;
+            int lab[VB];
+#pragma unroll
+            for (int u = 0; u < VB; ++u) {  // (past the end: the last voxel, which changes nothing)
+                int x, y, z;
+                place(min(base + (unsigned)(u * threads), end - 1u), x, y, z);
+                lab[u] = a.labels[((long long)z * a.H + y) * a.W + x];
+            }
+#pragma unroll
+            for (int u = 0; u < VB; ++u) match |= lab[u] == k ? 1u << u : 0u;
+            for (; match; match &= match - 1) {
+                int x, y, z;
+                place(min(base + (unsigned)((__ffs(match) - 1) * threads), end - 1u), x, y, z);
+                const VBest c = vcandidate(((long long)z * a.H + y) * a.W + x, x, y, z, n, sx, sy, st, true);
+                if (vless(c, b)) b = c;
+            }
+        }
+    } else {
+#pragma unroll 1
+        for (long long i = t; i < vol; i += threads) {
+            const long long row = div_w.row(i), fr = div_h.row(row);
+            const int x = xlo + (int)(i - row * w), y = ylo + (int)(row - fr * h), z = tlo + (int)fr;
+            const long long p = ((long long)z * a.H + y) * a.W + x;
+            if (a.labels[p] != k) continue;
+            const VBest c = vcandidate(p, x, y, z, n, sx, sy, st, small);
+            if (vless(c, b)) b = c;
+        }
+    }
+}
+
+// Queue entries j0, j0 + stride, ...: one CTA per queued cluster.
+__device__ __forceinline__ void vproject_cta(const VoxArgs &a, int whole, int j0, int stride)
+{
     __shared__ VBest s_best[VPROJ_THREADS / 32];
     const int nproj = a.ctr->nproj;
-    const int n_orphans = whole ? 0 : a.ctr->orphans;
+    const int n_orphans = whole ? 0 : a.ctr->proj_orphans;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    for (int j = blockIdx.x; j < nproj; j += gridDim.x) {
+    for (int j = j0; j < nproj; j += stride) {
         const int k = a.proj_list[j];
         const long long n = a.st_n[k], sx = a.st_sx[k], sy = a.st_sy[k], st = a.st_st[k];
         int xlo = 0, xhi = a.W - 1, ylo = 0, yhi = a.H - 1, tlo = 0, thi = a.T - 1;
@@ -319,36 +424,11 @@ __global__ void __launch_bounds__(VPROJ_THREADS) k_vproject(VoxArgs a, int whole
         }
         const long long w = xhi - xlo + 1, h = yhi - ylo + 1;
         const long long vol = max(0LL, w) * max(0LL, h) * max(0LL, (long long)(thi - tlo + 1));
-        // voxel i of the box: row i / w, frame row / h, by reciprocals
-        const RowDiv div_w(w, vol), div_h(h, w > 0 ? vol / w : 0);
         // 64-bit squared distances when 3 (n * largest dimension)^2 < 2^62
         const double bound = (double)max(a.W, max(a.H, a.T));
         const bool small = 3.0 * ((double)n * bound) * ((double)n * bound) < 4.0e18;
         VBest b = {~0ull, ~0ull, LLONG_MAX};
-        constexpr int VB = 8;  // label loads issued before any comparison
-        for (long long base = 0; base < vol; base += (long long)VPROJ_THREADS * VB) {
-            int lab[VB];
-#pragma unroll
-            for (int u = 0; u < VB; ++u) {
-                const long long i = base + (long long)u * VPROJ_THREADS + tid;
-                lab[u] = -1;
-                if (i < vol) {
-                    const long long row = div_w.row(i), fr = div_h.row(row);
-                    const int x = xlo + (int)(i - row * w), y = ylo + (int)(row - fr * h), t = tlo + (int)fr;
-                    lab[u] = a.labels[((long long)t * a.H + y) * a.W + x];
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < VB; ++u) {
-                if (lab[u] != k) continue;
-                const long long i = base + (long long)u * VPROJ_THREADS + tid;
-                const long long row = div_w.row(i), fr = div_h.row(row);
-                const int x = xlo + (int)(i - row * w), y = ylo + (int)(row - fr * h), t = tlo + (int)fr;
-                const long long p = ((long long)t * a.H + y) * a.W + x;
-                const VBest c = vcandidate(p, x, y, t, n, sx, sy, st, small);
-                if (vless(c, b)) b = c;
-            }
-        }
+        vproject_scan(a, k, n, sx, sy, st, small, xlo, ylo, tlo, w, h, vol, tid, VPROJ_THREADS, b);
         for (int i = tid; i < n_orphans; i += VPROJ_THREADS) {
             const int p = a.orphan_list[i];
             if (a.labels[p] != k) continue;
@@ -380,11 +460,43 @@ __global__ void __launch_bounds__(VPROJ_THREADS) k_vproject(VoxArgs a, int whole
     }
 }
 
+__global__ void __launch_bounds__(VPROJ_THREADS) k_vproject(VoxArgs a, int whole)
+{
+    pdl_wait();
+    pdl_release();
+    vproject_cta(a, whole, blockIdx.x, gridDim.x);
+}
+
 // ---------------------------------------------------------------------------
-// Candidate lists: exclusive scan of the tile counts (one CTA), then one
-// thread per (cluster, tile slot).
+// Candidate lists: exclusive scan of the tile counts, then the (cluster, tile)
+// slots, one thread each.  The assignment of a tile zeroes its count and
+// cursor once it has read its list, so the lists touch nothing the projection
+// reads, and both run in one launch (VLISTS_MAX_TILES bounds the scan in shared
+// memory, as in 2-D); volumes of more tiles take a scan and a fill kernel after
+// the projection.
 // ---------------------------------------------------------------------------
 constexpr int VSCAN_THREADS = 1024;
+constexpr int VLISTS_MAX_TILES = 12287;  // (n + 1) ints of shared memory <= 48 KB
+
+__device__ __forceinline__ void vfill_slot(const VoxArgs &a, const int *tile_off, long long i)
+{
+    const unsigned slots = (unsigned)(a.tpw_x * a.tpw_y * a.tpw_t);
+    const long long total = (long long)a.Keff * slots;
+    if (i >= total) return;
+    const int k = total < (1LL << 32) ? (int)((unsigned)i / slots) : (int)(i / slots);
+    int j = (int)(i - (long long)k * slots);
+    const VoxCluster &cd = a.cdev[k];
+    const int xlo = cd.xlo, xhi = cd.xhi, ylo = cd.ylo, yhi = cd.yhi, tlo = cd.tlo, thi = cd.thi;
+    if (xlo > xhi || ylo > yhi || tlo > thi) return;
+    const int jx = j % a.tpw_x;
+    j /= a.tpw_x;
+    const int jy = j % a.tpw_y, jt = j / a.tpw_y;
+    const int tx = xlo / VTX + jx, ty = ylo / VTY + jy, tt = tlo / VTT + jt;
+    if (tx > xhi / VTX || ty > yhi / VTY || tt > thi / VTT) return;
+    const int tile = (tt * a.n_ty + ty) * a.n_tx + tx;
+    const int pos = tile_off[tile] + atomicAdd(&a.tile_cursor[tile], 1);
+    if (pos < a.tile_cap) a.tile_list[pos] = k;
+}
 
 __global__ void __launch_bounds__(VSCAN_THREADS) k_vscan(VoxArgs a)
 {
@@ -393,36 +505,39 @@ __global__ void __launch_bounds__(VSCAN_THREADS) k_vscan(VoxArgs a)
     __shared__ int s_warp[32];
     const int n = a.n_tx * a.n_ty * a.n_tt;
     cta_scan(a.tile_count, a.tile_off, n, VSCAN_THREADS, s_warp);  // (ends with a barrier)
-    for (int i = threadIdx.x; i < n; i += VSCAN_THREADS) {
-        a.tile_cursor[i] = 0;
-        a.tile_count[i] = 0;
-    }
-    if (threadIdx.x == 0) {  // (tile_off[n] is this thread's own write)
-        if (a.tile_off[n] > a.tile_cap) atomicExch(&a.ctr->error, ERR_TILE_LIST_OVERFLOW);
-        a.ctr->nproj = 0;
-        a.ctr->orphans = 0;
-    }
+    // (tile_off[n] is this thread's own write)
+    if (threadIdx.x == 0 && a.tile_off[n] > a.tile_cap) atomicExch(&a.ctr->error, ERR_TILE_LIST_OVERFLOW);
 }
 
 __global__ void k_vfill(VoxArgs a)
 {
     pdl_wait();
     pdl_release();
-    const long long slots = (long long)a.tpw_x * a.tpw_y * a.tpw_t;
-    const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (i >= (long long)a.Keff * slots) return;
-    const int k = (int)(i / slots);
-    int j = (int)(i - (long long)k * slots);
-    const VoxCluster cd = a.cdev[k];
-    if (cd.xlo > cd.xhi || cd.ylo > cd.yhi || cd.tlo > cd.thi) return;
-    const int jx = j % a.tpw_x;
-    j /= a.tpw_x;
-    const int jy = j % a.tpw_y, jt = j / a.tpw_y;
-    const int tx = cd.xlo / VTX + jx, ty = cd.ylo / VTY + jy, tt = cd.tlo / VTT + jt;
-    if (tx > cd.xhi / VTX || ty > cd.yhi / VTY || tt > cd.thi / VTT) return;
-    const int tile = (tt * a.n_ty + ty) * a.n_tx + tx;
-    const int pos = a.tile_off[tile] + atomicAdd(&a.tile_cursor[tile], 1);
-    if (pos < a.tile_cap) a.tile_list[pos] = k;
+    vfill_slot(a, a.tile_off, blockIdx.x * (long long)blockDim.x + threadIdx.x);
+}
+
+// The lists by CTAs [0, n_lists), placed first, and the projection by the
+// others (none without a queue: set_state).
+__global__ void __launch_bounds__(VPROJ_THREADS) k_vproject_lists(VoxArgs a, int whole, int n_lists)
+{
+    pdl_wait();
+    pdl_release();
+    extern __shared__ int s_off[];
+    __shared__ int s_warp[32];
+    const int blk = (int)blockIdx.x;
+    if (blk >= n_lists) {
+        vproject_cta(a, whole, blk - n_lists, (int)gridDim.x - n_lists);
+        return;
+    }
+    const int n = a.n_tx * a.n_ty * a.n_tt;
+    cta_scan(a.tile_count, s_off, n, VPROJ_THREADS, s_warp);
+    if (blk == 0) {
+        for (int i = threadIdx.x; i <= n; i += VPROJ_THREADS) a.tile_off[i] = s_off[i];
+        if (threadIdx.x == 0 && s_off[n] > a.tile_cap) atomicExch(&a.ctr->error, ERR_TILE_LIST_OVERFLOW);
+    }
+    const long long slots = (long long)a.Keff * a.tpw_x * a.tpw_y * a.tpw_t;
+    for (long long i = blk * (long long)VPROJ_THREADS + threadIdx.x; i < slots; i += (long long)n_lists * VPROJ_THREADS)
+        vfill_slot(a, s_off, i);
 }
 
 // ---------------------------------------------------------------------------
@@ -570,6 +685,12 @@ __global__ void __launch_bounds__(VTILE) k_vassign(VoxArgs a)
     const int off = a.tile_off[tile];
     const int cnt = (int)max(0LL, min((long long)a.tile_off[tile + 1], a.tile_cap) - off);
     const bool fast = cnt <= VCAND;
+    if (tid == 0) {  // this tile's list is read: ready the counts for the next update
+        a.tile_count[tile] = 0;
+        a.tile_cursor[tile] = 0;
+        // the last projection completed before this launch: its queue starts again
+        if (tile == 0) a.ctr->nproj = 0;
+    }
     const long long p = ((long long)t * a.H + y) * a.W + x;
     unsigned my_samples = 0, my_pairs = 0;
     int lab = -1;
@@ -909,22 +1030,27 @@ int vcheck(cudaError_t e, const char *what)
 
 // Programmatic launches (each kernel placed while the one before drains),
 // except around the profiling event records.
-void venqueue_lists(scalp_vctx *c)
-{
-    const bool pdl = !c->profiling;
-    pdl_launch(pdl, k_vscan, dim3(1), dim3(VSCAN_THREADS), 0, c->st, c->a);
-    const long long slots = (long long)c->Keff * c->a.tpw_x * c->a.tpw_y * c->a.tpw_t;
-    pdl_launch(pdl, k_vfill, dim3((unsigned)((slots + 255) / 256)), dim3(256), 0, c->st, c->a);
-}
-
 void venqueue_update(scalp_vctx *c, int from_acc, int whole)
 {
     const bool pdl = !c->profiling;
-    pdl_launch(pdl, k_vupdate, dim3((c->Keff + 63) / 64), dim3(64), 0, c->st, c->a, from_acc);
+    const long long threads = (long long)c->Keff * VUPDATE_LANES;
+    pdl_launch(pdl, k_vupdate, dim3((unsigned)ceil_div_ll(threads, VUPDATE_THREADS)), dim3(VUPDATE_THREADS), 0, c->st,
+               c->a, from_acc);
+    const int n = c->a.n_tx * c->a.n_ty * c->a.n_tt;
+    const long long slots = (long long)c->Keff * c->a.tpw_x * c->a.tpw_y * c->a.tpw_t;
+    if (n <= VLISTS_MAX_TILES) {
+        // one resident wave: list CTAs of four slots per thread, the projection in the rest
+        const int n_lists = (int)std::max(std::min(ceil_div_ll(slots, 4LL * VPROJ_THREADS), 64LL), 1LL);
+        const int n_proj = from_acc ? std::max(std::min(c->Keff, 2 * 152 - n_lists), 1) : 0;
+        pdl_launch(pdl, k_vproject_lists, dim3((unsigned)(n_lists + n_proj)), dim3(VPROJ_THREADS),
+                   (size_t)(n + 1) * sizeof(int), c->st, c->a, whole, n_lists);
+        return;
+    }
     if (from_acc)
         pdl_launch(pdl, k_vproject, dim3(std::min(c->Keff, 2 * 152)), dim3(VPROJ_THREADS), 0, c->st, c->a,
                    whole);
-    venqueue_lists(c);
+    pdl_launch(pdl, k_vscan, dim3(1), dim3(VSCAN_THREADS), 0, c->st, c->a);
+    pdl_launch(pdl, k_vfill, dim3((unsigned)((slots + 255) / 256)), dim3(256), 0, c->st, c->a);
 }
 
 // The counters go to the thread's pinned status buffer behind the stream's
@@ -1030,6 +1156,7 @@ int scalp_voxel_init(scalp_vctx **out, const scalp_volume *vol, int32_t K, float
     const size_t n_tiles = (size_t)L.n_tx * L.n_ty * L.n_tt;
     if (!rc) rc = vcheck(cudaMemsetAsync(a.acc, 0, sizeof(VoxAcc) * c->Keff, c->st), "memset");
     if (!rc) rc = vcheck(cudaMemsetAsync(a.tile_count, 0, 4 * n_tiles, c->st), "memset");
+    if (!rc) rc = vcheck(cudaMemsetAsync(a.tile_cursor, 0, 4 * n_tiles, c->st), "memset");
     if (!rc) rc = vcheck(cudaMemsetAsync(a.cdev, 0, sizeof(VoxCluster) * c->Keff, c->st), "memset");
     if (!rc) rc = vcheck(cudaMemsetAsync(a.ctr, 0, sizeof(DevCounters), c->st), "memset");
     if (!rc) rc = vcheck(srgb_table(&a.lut, c->st), "transfer-function table");
@@ -1154,6 +1281,7 @@ int scalp_voxel_set_state(scalp_vctx *c, const scalp_voxel_state *s)
     if (!rc) rc = vcheck(cudaMemcpy(c->a.st_end, end.data(), 16 * K, cudaMemcpyHostToDevice), "copy");
     if (!rc) rc = vcheck(cudaMemset(c->a.acc, 0, sizeof(VoxAcc) * K), "memset");
     if (!rc) rc = vcheck(cudaMemset(c->a.tile_count, 0, 4 * n_tiles), "memset");
+    if (!rc) rc = vcheck(cudaMemset(c->a.tile_cursor, 0, 4 * n_tiles), "memset");
     if (rc) return rc;
     venqueue_update(c, 0, 0);
     rc = vcheck(cudaGetLastError(), "derive kernels");
