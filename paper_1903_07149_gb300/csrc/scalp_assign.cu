@@ -73,13 +73,20 @@ int assign_map_capacity(int device)
     return cap > 0 ? (int)cap : 0;
 }
 
-template <typename T, bool COUNT>
-__global__ void __launch_bounds__(ASSIGN_THREADS, ASSIGN_CTAS_PER_SM) k_assign(SolveArgs a)
+// A grid that leaves SMs without a second tile is bound by the time of one
+// tile: with 1024 threads (a pixel each, one CTA per SM) its chain of map
+// strips, walks and sums is half as long.  96 x 160 (15 tiles): WIDE_US.
+// Above one tile per SM two 512-thread CTAs share an SM instead.
+constexpr int ASSIGN_WIDE_THREADS = 1024;
+constexpr int ASSIGN_WIDE_TILES = 152;  // SMs
+
+template <typename T, bool COUNT, int THREADS>
+__global__ void __launch_bounds__(THREADS, THREADS == ASSIGN_THREADS ? ASSIGN_CTAS_PER_SM : 1) k_assign(SolveArgs a)
 {
     pdl_wait();
     pdl_release();
     extern __shared__ __align__(16) unsigned char smem[];
-    assign_tile<T, false, COUNT>(a, blockIdx.x, smem);
+    assign_tile<T, false, COUNT, THREADS>(a, blockIdx.x, smem);
 }
 
 // All tiles of all images of a batch in one launch: block g is tile
@@ -98,7 +105,11 @@ __global__ void __launch_bounds__(ASSIGN_THREADS, ASSIGN_CTAS_PER_SM) k_assign_b
 template <typename T, bool COUNT>
 static void launch_assign_as(const SolveArgs &a, size_t smem_bytes, cudaStream_t st, bool pdl)
 {
-    pdl_launch(pdl, k_assign<T, COUNT>, dim3(a.n_tx * a.n_ty), dim3(ASSIGN_THREADS), smem_bytes, st, a);
+    const int tiles = a.n_tx * a.n_ty;
+    if (tiles <= ASSIGN_WIDE_TILES)
+        pdl_launch(pdl, k_assign<T, COUNT, ASSIGN_WIDE_THREADS>, dim3(tiles), dim3(ASSIGN_WIDE_THREADS), smem_bytes, st, a);
+    else
+        pdl_launch(pdl, k_assign<T, COUNT, ASSIGN_THREADS>, dim3(tiles), dim3(ASSIGN_THREADS), smem_bytes, st, a);
 }
 
 void launch_assign(const SolveArgs &a, int storage, size_t smem_bytes, cudaStream_t st, bool pdl)
@@ -150,13 +161,20 @@ static cudaError_t configure(const void *f)
                                 (int)assign_smem_bytes(assign_map_capacity(dev)));
 }
 
-// (the kernels with and without counting)
+// (the kernels with and without counting, in both widths)
+template <typename T, bool COUNT>
+static cudaError_t configure_as(bool batch)
+{
+    if (batch) return configure((const void *)k_assign_batch<T, COUNT>);
+    const cudaError_t e = configure((const void *)k_assign<T, COUNT, ASSIGN_THREADS>);
+    return e != cudaSuccess ? e : configure((const void *)k_assign<T, COUNT, ASSIGN_WIDE_THREADS>);
+}
+
 template <typename T>
 static cudaError_t configure_pair(bool batch)
 {
-    const cudaError_t e = configure(batch ? (const void *)k_assign_batch<T, false> : (const void *)k_assign<T, false>);
-    if (e != cudaSuccess) return e;
-    return configure(batch ? (const void *)k_assign_batch<T, true> : (const void *)k_assign<T, true>);
+    const cudaError_t e = configure_as<T, false>(batch);
+    return e != cudaSuccess ? e : configure_as<T, true>(batch);
 }
 
 cudaError_t assign_batch_configure(int storage)

@@ -70,11 +70,11 @@ __device__ __forceinline__ int path_sums_map(uint32_t at, int p8, int X, int Y, 
 // per-candidate records follow, sized for the tile's own candidate count, and
 // the distance maps fill the rest (a tile with few candidates has more room).
 __host__ __device__ constexpr size_t align16(size_t x) { return (x + 15) & ~(size_t)15; }
-constexpr int ASSIGN_QUEUE = 160;  // pairs a warp's queue holds (pass 2)
+constexpr int ASSIGN_QUEUES = 2560;  // pairs the warps' queues hold together (pass 2)
 struct AssignSmem {
     static constexpr size_t best = 0;
     static constexpr size_t queue = align16(best + TILE_PIXELS * sizeof(unsigned long long));
-    static constexpr size_t misc = align16(queue + (ASSIGN_THREADS / 32) * ASSIGN_QUEUE * sizeof(uint16_t));
+    static constexpr size_t misc = align16(queue + ASSIGN_QUEUES * sizeof(uint16_t));
     static constexpr size_t records = align16(misc + 64);
 };
 static_assert(AssignSmem::queue % 16 == 0 && AssignSmem::misc % 16 == 0 && AssignSmem::records % 16 == 0,
@@ -210,12 +210,12 @@ __device__ __forceinline__ int warp_scan_maps(const int *area, const int4 *box, 
 // whose planes outgrow L2; an image whose plane stays in L2 only pays for it).
 // COUNT: the work is counted when a.count_samples asks for it (the counting
 // code costs the walks and the bound even when it is off).
-template <typename T, bool PREFETCH_TILE = false, bool COUNT = true>
+template <typename T, bool PREFETCH_TILE = false, bool COUNT = true, int THREADS = ASSIGN_THREADS>
 __device__ __forceinline__ void assign_tile(const SolveArgs &a, int tile, unsigned char *smem)
 {
-    constexpr int THREADS = ASSIGN_THREADS;
     constexpr int PIX_PER_THREAD = TILE_PIXELS / THREADS;
     constexpr int WARPS = THREADS / 32;
+    constexpr int QUEUE = ASSIGN_QUEUES / WARPS;  // pairs a warp's queue holds
     constexpr int BUILD_UNROLL = 4;  // samples per lane in flight
     const T *__restrict__ plane = reinterpret_cast<const T *>(
         sizeof(T) == 16 ? (const void *)a.plane32 : (const void *)a.plane16);
@@ -522,12 +522,13 @@ __device__ __forceinline__ void assign_tile(const SolveArgs &a, int tile, unsign
         // fills: held across the walks as well they spill registers (FP32, HD
         // 140.0 us a launch against 134.7).
         static_assert(WARPS % (TILE_X / WARP_BLOCK_X) == 0, "the warp's blocks lie in one column of blocks");
-        static_assert(PIX_PER_THREAD == 2 && MAX_TILE_CANDIDATES <= 1024, "queued pairs pack into 16 bits");
+        static_assert(PIX_PER_THREAD <= 2 && MAX_TILE_CANDIDATES <= 1024, "queued pairs pack into 16 bits");
+        static_assert(QUEUE > 32 * PIX_PER_THREAD, "a queue takes a candidate's pairs after a full batch is left over");
         constexpr int ROW_STEP = WARPS / (TILE_X / WARP_BLOCK_X) * WARP_BLOCK_Y;  // block 1 lies this far below block 0
         int px, py;
         my_pixel(0, px, py);
         const int bx = px - lane % WARP_BLOCK_X, by = py - lane / WARP_BLOCK_X;
-        uint16_t *wq = reinterpret_cast<uint16_t *>(smem + AssignSmem::queue) + warp * ASSIGN_QUEUE;
+        uint16_t *wq = reinterpret_cast<uint16_t *>(smem + AssignSmem::queue) + warp * QUEUE;
         int queued = 0, c0 = -32;                    // warp-uniform, as all that follows
         unsigned meets[PIX_PER_THREAD] = {}, any = 0;  // candidates c0 + bit left, per block and over both
         for (bool more = true; more;) {
@@ -550,7 +551,7 @@ __device__ __forceinline__ void assign_tile(const SolveArgs &a, int tile, unsign
                 }
             }
             const unsigned lanes_below = (1u << lane) - 1u;
-            while (queued <= ASSIGN_QUEUE - 64) {
+            while (queued <= QUEUE - 32 * PIX_PER_THREAD) {
                 if (!any) {
                     // the next 32 candidates: which of their rectangles meet
                     // each of the warp's blocks, one candidate per lane
