@@ -30,6 +30,7 @@ struct Layout {
     size_t total;
     long long tile_cap, scan_tmp_len;
     int n_tx, n_ty, pitch;
+    int side;  // of a tile
 };
 
 constexpr size_t ALIGN = 256;
@@ -61,7 +62,9 @@ bool sizes_ok(int H, int W, int K)
     return K <= N;
 }
 
-Layout make_layout(int H, int W, int K, int storage)
+// A batched image has TILE_SIDE tiles whatever its size (one launch labels
+// the tiles of every image); its layout is never larger than the single one.
+Layout make_layout(int H, int W, int K, int storage, bool batched = false)
 {
     Layout L{};
     long long N = (long long)H * W;
@@ -70,10 +73,11 @@ Layout make_layout(int H, int W, int K, int storage)
     grid_dims(H, W, K, nx, ny, r);
     long long Keff = (long long)nx * ny;
     L.pitch = (W + 3) & ~3;
-    L.n_tx = (int)ceil_div_ll(W, TILE_X);
-    L.n_ty = (int)ceil_div_ll(H, TILE_Y);
+    L.side = !batched && small_tiles(H, W, r) ? TILE_SIDE_SMALL : TILE_SIDE;
+    L.n_tx = (int)ceil_div_ll(W, L.side);
+    L.n_ty = (int)ceil_div_ll(H, L.side);
     long long n_tiles = (long long)L.n_tx * L.n_ty;
-    L.tile_cap = Keff * tiles_per_window(r, TILE_X) * tiles_per_window(r, TILE_Y);
+    L.tile_cap = Keff * tiles_per_window(r, L.side) * tiles_per_window(r, L.side);
     L.scan_tmp_len = ccl_scan_tmp_len(N);
     size_t elem = storage == 0 ? 16 : 8;
     size_t cur = 0;
@@ -436,8 +440,8 @@ size_t scalp_workspace_bytes(int32_t H, int32_t W, int32_t K, const scalp_params
     return make_layout(H, W, K, storage).total;
 }
 
-int scalp_init(scalp_ctx **out, const scalp_image *image, const scalp_contour *contour, int32_t K,
-               float m, const scalp_params *params)
+static int init_ctx(scalp_ctx **out, const scalp_image *image, const scalp_contour *contour, int32_t K,
+                    float m, const scalp_params *params, bool batched)
 {
     const char *why = nullptr;
     if (!out) return fail(nullptr, SCALP_E_ARG, "out is NULL");
@@ -459,7 +463,7 @@ int scalp_init(scalp_ctx **out, const scalp_image *image, const scalp_contour *c
     if (params->storage != 0 && params->storage != 1)
         return fail(nullptr, SCALP_E_ARG, "storage must be SCALP_STORAGE_F32 or _F16");
     const int H = image->H, W = image->W;
-    Layout L = make_layout(H, W, K, params->storage);
+    Layout L = make_layout(H, W, K, params->storage, batched);
     if (!params->workspace || params->workspace_bytes < L.total)
         return fail(nullptr, SCALP_E_NOMEM, "workspace of %zu bytes needed, %zu given", L.total,
                     params->workspace ? params->workspace_bytes : (size_t)0);
@@ -486,6 +490,8 @@ int scalp_init(scalp_ctx **out, const scalp_image *image, const scalp_contour *c
     a.sigma = params->sigma;
     a.ms2 = (float)((double)m * (double)m * (double)K / (double)c->N);  // m^2 / r^2
     a.n_tx = L.n_tx; a.n_ty = L.n_ty;
+    a.tile_shift = L.side == TILE_SIDE ? 5 : 4;
+    static_assert(TILE_SIDE == 32 && TILE_SIDE_SMALL == 16, "tile shifts");
     a.pitch = L.pitch;
     a.grid_rcp_x = grid_reciprocal(W, c->nx);
     a.plane32 = params->storage == 0 ? reinterpret_cast<const float4 *>(c->ws + L.plane) : nullptr;
@@ -504,8 +510,8 @@ int scalp_init(scalp_ctx **out, const scalp_image *image, const scalp_contour *c
     a.tile_cursor = reinterpret_cast<int *>(c->ws + L.tile_cursor);
     a.tile_list = reinterpret_cast<int *>(c->ws + L.tile_list);
     a.tile_cap = L.tile_cap;
-    a.tpw_x = tiles_per_window(c->r, TILE_X);
-    a.tpw_y = tiles_per_window(c->r, TILE_Y);
+    a.tpw_x = tiles_per_window(c->r, L.side);
+    a.tpw_y = tiles_per_window(c->r, L.side);
     a.prev_win = reinterpret_cast<int4 *>(c->ws + L.prev_win);
     // (the connectivity's buffer: the enforcement never runs beside an iteration)
     a.orphan_list = reinterpret_cast<int *>(c->ws + L.parent);
@@ -520,9 +526,9 @@ int scalp_init(scalp_ctx **out, const scalp_image *image, const scalp_contour *c
     // distance maps of the assignment CTAs (none: every path walks the plane)
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) dev = 0;
-    a.map_cap = (params->global_walk & 1) ? 0 : assign_map_capacity(dev);
+    a.map_cap = (params->global_walk & 1) ? 0 : assign_map_capacity(dev, L.side, L.n_tx * L.n_ty);
     a.prune = (params->global_walk & 2) || !bound_valid(H, W, a.lam, a.ms2) ? 0 : 1;
-    c->smem = assign_smem_bytes(a.map_cap);
+    c->smem = assign_smem_bytes(a.map_cap, L.side);
     int rc = cuda_check(c, assign_configure(params->storage), "configure kernel");
     if (rc == SCALP_OK) rc = cuda_check(c, srgb_table(&a.lut, c->st), "transfer-function table");
     if (rc == SCALP_OK) rc = load_inputs(c, image, contour);
@@ -532,6 +538,12 @@ int scalp_init(scalp_ctx **out, const scalp_image *image, const scalp_contour *c
     }
     *out = c;
     return SCALP_OK;
+}
+
+int scalp_init(scalp_ctx **out, const scalp_image *image, const scalp_contour *contour, int32_t K,
+               float m, const scalp_params *params)
+{
+    return init_ctx(out, image, contour, K, m, params, false);
 }
 
 int scalp_reload(scalp_ctx *c, const scalp_image *image, const scalp_contour *contour)
@@ -923,6 +935,12 @@ int scalp_gradient_prior(const scalp_image *image, float *out, int64_t out_strid
 // ---------------------------------------------------------------------------
 namespace scalp {
 
+int scalp_init_batched(scalp_ctx **out, const scalp_image *image, const scalp_contour *contour, int32_t K, float m,
+                       const scalp_params *params)
+{
+    return init_ctx(out, image, contour, K, m, params, true);
+}
+
 SolveArgs scalp_ctx_args(const scalp_ctx *c) { return c->a; }
 void scalp_ctx_set_stream(scalp_ctx *c, cudaStream_t st) { c->st = st; }
 size_t scalp_ctx_smem(const scalp_ctx *c) { return c->smem; }
@@ -1282,7 +1300,7 @@ int scalp_batch_init(scalp_batch **out, int32_t count, const scalp_image *images
         p.workspace_bytes = scalp_workspace_bytes(Hs[i], Ws[i], K[i], params);
         off += (p.workspace_bytes + ALIGN - 1) & ~(ALIGN - 1);
         scalp_ctx *c = nullptr;
-        const int rc = scalp_init(&c, &images[i], contours ? &contours[i] : nullptr, K[i], m[i], &p);
+        const int rc = init_ctx(&c, &images[i], contours ? &contours[i] : nullptr, K[i], m[i], &p, true);
         if (rc != SCALP_OK) {
             char msg[512];
             snprintf(msg, sizeof msg, "image %d: %s", i, g_last_error.c_str());

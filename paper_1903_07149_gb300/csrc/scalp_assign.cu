@@ -7,7 +7,8 @@
 // clusters (those whose window holds it, from its tile's candidate list) and
 // keeps the smallest (D, k) pair: the same result, in any evaluation order.
 //
-// One CTA of 512 threads (two per SM) labels a 32 x 32 tile:
+// One CTA of 512 threads (two per SM) labels a 32 x 32 tile (for grids of few
+// tiles: 1024 threads, or 256 on a 16 x 16 tile):
 //   1. The tile's candidate clusters are copied to shared memory, sorted by
 //      cluster index.
 //   2. Distance maps.  For a candidate k, every path from a tile pixel in its
@@ -23,10 +24,10 @@
 //      again, and its D stays in the thread's registers.
 //   4. Pass 2: each warp checks its pixels against the other candidates
 //      whose rectangle (the tile's pixels inside the window) holds them.  A
-//      pair whose lower bound fl(fl(lam*d_c(p)) + fl(m^2/r^2*d_s)) exceeds
-//      the pixel's pass-1 D cannot win or tie (its computed D is never below
-//      the bound) and is not walked; the others are queued per warp and
-//      walked 32 at a time by that warp.
+//      pair whose lower bound lam*d_c(p) + m^2/r^2*d_s (a dot product of
+//      pixel and candidate terms, less a margin for its rounding) exceeds the
+//      pixel's pass-1 D cannot win or tie and is not walked; the others are
+//      queued per warp and walked 32 at a time by that warp.
 //   5. Each walk follows the pixel's path to the candidate's endpoint (one
 //      8-byte map load and one packed two-float add per sample), forms D
 //      (Eq. 1-3) and takes a 64-bit shared-memory atomicMin of (D bits,
@@ -48,13 +49,16 @@
 
 namespace scalp {
 
-size_t assign_smem_bytes(int map_cap)
+// Dynamic shared memory of a CTA with map_cap distance-map pairs.
+size_t assign_smem_bytes(int map_cap, int side)
 {
-    return tile_layout(MAX_TILE_CANDIDATES).maps + (size_t)map_cap * sizeof(float2);
+    const uint32_t maps = side == TILE_SIDE ? tile_layout<TILE_SIDE>(MAX_TILE_CANDIDATES).maps
+                                            : tile_layout<TILE_SIDE_SMALL>(MAX_TILE_CANDIDATES).maps;
+    return maps + (size_t)map_cap * sizeof(float2);
 }
 
-// Map capacity (pairs) when ASSIGN_CTAS_PER_SM CTAs share an SM's shared memory.
-int assign_map_capacity(int device)
+// Map capacity (pairs) when `ctas` CTAs share an SM's shared memory.
+static int map_capacity(int device, int ctas, int side)
 {
     int per_sm = 0, per_cta_max = 0, reserved = 0;
     if (cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, device) !=
@@ -66,27 +70,52 @@ int assign_map_capacity(int device)
         return 0;
     // PERSIST_STATIC_SMEM stays free for the persistent batched kernel's own
     // static shared memory (the same capacity serves every assignment kernel)
-    long long per_cta = std::min((long long)per_cta_max,
-                                 (long long)per_sm / ASSIGN_CTAS_PER_SM - reserved) - PERSIST_STATIC_SMEM;
+    long long per_cta = std::min((long long)per_cta_max, (long long)per_sm / ctas - reserved) - PERSIST_STATIC_SMEM;
     per_cta &= ~15LL;
-    const long long cap = (per_cta - (long long)tile_layout(MAX_TILE_CANDIDATES).maps) / (long long)sizeof(float2);
+    const long long cap = (per_cta - (long long)assign_smem_bytes(0, side)) / (long long)sizeof(float2);
     return cap > 0 ? (int)cap : 0;
+}
+
+constexpr int SMS = 152;
+
+// Small tiles leave as much shared memory to a CTA as the grid's CTAs per SM
+// allow, between three and four of them.  (With two, 300 tiles filled every
+// SM's shared memory, and the next kernels were placed late: a 240 x 320 solve
+// 313 us against 279.)
+int assign_map_capacity(int device, int side, int tiles)
+{
+    const int ctas = side == TILE_SIDE ? ASSIGN_CTAS_PER_SM
+                                       : std::min(std::max((tiles + SMS - 1) / SMS, 3), 4);
+    return map_capacity(device, ctas, side);
+}
+
+// Whether a single image takes small tiles.  A 32 x 32 tile is about 47,000 warp
+// instructions, 6 us of an SM at best, so an image of few tiles waits for one
+// SM's work while others idle.  Quarter tiles cost a fifth more in all (each
+// reads its candidates and builds its maps for 256 pixels) but spread: solves
+// of 96 x 160 274 -> 229 us, 200 x 300 290 -> 263, 240 x 320 291 -> 279,
+// 321 x 481 357 -> 337, 360 x 480 (180 tiles) 373 -> 362; from 208 tiles on they
+// are no faster (400 x 500 386 -> 385 and 377 -> 393, 448 x 512 386 -> 398).
+// Above r = 24 a small tile's boxes outgrow its map buffer.
+bool small_tiles(int H, int W, double r)
+{
+    const long long tiles = ceil_div_ll(W, TILE_SIDE) * ceil_div_ll(H, TILE_SIDE);
+    return tiles <= 192 && r <= 24.0;
 }
 
 // A grid that leaves SMs without a second tile is bound by the time of one
 // tile: with 1024 threads (a pixel each, one CTA per SM) its chain of map
-// strips, walks and sums is half as long.  96 x 160 (15 tiles): WIDE_US.
-// Above one tile per SM two 512-thread CTAs share an SM instead.
-constexpr int ASSIGN_WIDE_THREADS = 1024;
-constexpr int ASSIGN_WIDE_TILES = 152;  // SMs
+// strips, walks and sums is half as long.  Above one tile per SM two
+// 512-thread CTAs share an SM instead.
+constexpr int ASSIGN_WIDE_THREADS = 1024, ASSIGN_SMALL_THREADS = 256;
 
-template <typename T, bool COUNT, int THREADS>
-__global__ void __launch_bounds__(THREADS, THREADS == ASSIGN_THREADS ? ASSIGN_CTAS_PER_SM : 1) k_assign(SolveArgs a)
+template <typename T, bool COUNT, int THREADS, int SIDE>
+__global__ void __launch_bounds__(THREADS, 1024 / THREADS) k_assign(SolveArgs a)
 {
     pdl_wait();
     pdl_release();
     extern __shared__ __align__(16) unsigned char smem[];
-    assign_tile<T, false, COUNT, THREADS>(a, blockIdx.x, smem);
+    assign_tile<T, false, COUNT, THREADS, SIDE>(a, blockIdx.x, smem);
 }
 
 // All tiles of all images of a batch in one launch: block g is tile
@@ -106,10 +135,15 @@ template <typename T, bool COUNT>
 static void launch_assign_as(const SolveArgs &a, size_t smem_bytes, cudaStream_t st, bool pdl)
 {
     const int tiles = a.n_tx * a.n_ty;
-    if (tiles <= ASSIGN_WIDE_TILES)
-        pdl_launch(pdl, k_assign<T, COUNT, ASSIGN_WIDE_THREADS>, dim3(tiles), dim3(ASSIGN_WIDE_THREADS), smem_bytes, st, a);
+    const auto launch = [&](auto kernel, int threads) {
+        pdl_launch(pdl, kernel, dim3(tiles), dim3(threads), smem_bytes, st, a);
+    };
+    if (1 << a.tile_shift == TILE_SIDE_SMALL)
+        launch(k_assign<T, COUNT, ASSIGN_SMALL_THREADS, TILE_SIDE_SMALL>, ASSIGN_SMALL_THREADS);
+    else if (tiles <= SMS)
+        launch(k_assign<T, COUNT, ASSIGN_WIDE_THREADS, TILE_SIDE>, ASSIGN_WIDE_THREADS);
     else
-        pdl_launch(pdl, k_assign<T, COUNT, ASSIGN_THREADS>, dim3(tiles), dim3(ASSIGN_THREADS), smem_bytes, st, a);
+        launch(k_assign<T, COUNT, ASSIGN_THREADS, TILE_SIDE>, ASSIGN_THREADS);
 }
 
 void launch_assign(const SolveArgs &a, int storage, size_t smem_bytes, cudaStream_t st, bool pdl)
@@ -151,23 +185,26 @@ bool bound_valid(int H, int W, float lam, float ms2)
 }
 
 // The limit is a property of the kernel, shared by every context on the
-// device: it is always set to the full map buffer, which covers any launch.
-static cudaError_t configure(const void *f)
+// device: it is always set to the largest map buffer, which covers any launch.
+static cudaError_t configure(const void *f, int side)
 {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)assign_smem_bytes(assign_map_capacity(dev)));
+                                (int)assign_smem_bytes(assign_map_capacity(dev, side, 1), side));
 }
 
-// (the kernels with and without counting, in both widths)
+// (the kernels with and without counting, in every form)
 template <typename T, bool COUNT>
 static cudaError_t configure_as(bool batch)
 {
-    if (batch) return configure((const void *)k_assign_batch<T, COUNT>);
-    const cudaError_t e = configure((const void *)k_assign<T, COUNT, ASSIGN_THREADS>);
-    return e != cudaSuccess ? e : configure((const void *)k_assign<T, COUNT, ASSIGN_WIDE_THREADS>);
+    if (batch) return configure((const void *)k_assign_batch<T, COUNT>, TILE_SIDE);
+    cudaError_t e = configure((const void *)k_assign<T, COUNT, ASSIGN_THREADS, TILE_SIDE>, TILE_SIDE);
+    if (e == cudaSuccess) e = configure((const void *)k_assign<T, COUNT, ASSIGN_WIDE_THREADS, TILE_SIDE>, TILE_SIDE);
+    if (e == cudaSuccess)
+        e = configure((const void *)k_assign<T, COUNT, ASSIGN_SMALL_THREADS, TILE_SIDE_SMALL>, TILE_SIDE_SMALL);
+    return e;
 }
 
 template <typename T>

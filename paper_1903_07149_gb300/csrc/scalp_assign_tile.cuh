@@ -1,4 +1,4 @@
-// scalp_assign_tile.cuh -- the assignment of one 32 x 32 tile (Algorithm 1's
+// scalp_assign_tile.cuh -- the assignment of one tile (32 x 32 or 16 x 16; Algorithm 1's
 // inner loops restated per tile, with the fused partial sums of the update):
 // the body shared by the per-iteration assignment kernels (scalp_assign.cu)
 // and the persistent batched kernel (scalp_persistent.cu).
@@ -70,15 +70,15 @@ __device__ __forceinline__ int path_sums_map(uint32_t at, int p8, int X, int Y, 
 // per-candidate records follow, sized for the tile's own candidate count, and
 // the distance maps fill the rest (a tile with few candidates has more room).
 __host__ __device__ constexpr size_t align16(size_t x) { return (x + 15) & ~(size_t)15; }
-constexpr int ASSIGN_QUEUES = 2560;  // pairs the warps' queues hold together (pass 2)
+// Pairs the warps' queues of a tile hold together (pass 2): 2.5 a pixel.
+__host__ __device__ constexpr int assign_queues(int side) { return side * side * 5 / 2; }
+template <int SIDE>
 struct AssignSmem {
     static constexpr size_t best = 0;
-    static constexpr size_t queue = align16(best + TILE_PIXELS * sizeof(unsigned long long));
-    static constexpr size_t misc = align16(queue + ASSIGN_QUEUES * sizeof(uint16_t));
+    static constexpr size_t queue = align16(best + SIDE * SIDE * sizeof(unsigned long long));
+    static constexpr size_t misc = align16(queue + assign_queues(SIDE) * sizeof(uint16_t));
     static constexpr size_t records = align16(misc + 64);
 };
-static_assert(AssignSmem::queue % 16 == 0 && AssignSmem::misc % 16 == 0 && AssignSmem::records % 16 == 0,
-              "shared-memory sections aligned");
 // Per candidate (rank c): three 16-byte records the walk reads,
 //   rec0 = (columns, rows, K bits, g_y bits)         its rectangle as a mask of
 //          the tile's columns and one of its rows; terms of the bound
@@ -91,10 +91,11 @@ static_assert(AssignSmem::queue % 16 == 0 && AssignSmem::misc % 16 == 0 && Assig
 struct TileLayout {
     uint32_t rec0, rec1, rec2, box, col, cid, area, mfirst, cfirst, maps;
 };
+template <int SIDE>
 __host__ __device__ constexpr TileLayout tile_layout(int n)
 {
     TileLayout t{};
-    t.rec0 = (uint32_t)AssignSmem::records;
+    t.rec0 = (uint32_t)AssignSmem<SIDE>::records;
     t.rec1 = t.rec0 + (uint32_t)n * 16u;
     t.rec2 = t.rec1 + (uint32_t)n * 16u;
     t.box = t.rec2 + (uint32_t)n * 16u;
@@ -108,11 +109,11 @@ __host__ __device__ constexpr TileLayout tile_layout(int n)
 }
 // The map pairs a tile of n candidates has beyond the capacity sized for
 // MAX_TILE_CANDIDATES.
+template <int SIDE>
 __host__ __device__ constexpr int extra_map_pairs(int n)
 {
-    return (int)((tile_layout(MAX_TILE_CANDIDATES).maps - tile_layout(n).maps) / 8u);
+    return (int)((tile_layout<SIDE>(MAX_TILE_CANDIDATES).maps - tile_layout<SIDE>(n).maps) / 8u);
 }
-static_assert(TILE_PIXELS <= 1024 && MAX_TILE_CANDIDATES < (1 << 21), "queued pairs pack into 32 bits");
 static_assert(MAX_TILE_CANDIDATES % 32 == 0, "the scans give each lane whole candidates");
 
 // Rank of cluster k among the tile's candidates (cid sorted ascending), or -1.
@@ -204,34 +205,35 @@ __device__ __forceinline__ int warp_scan_maps(const int *area, const int4 *box, 
 }
 
 // One tile of one image (the body shared by the single-image and the batched
-// kernels).  The pixels of a candidate's window that lie in the tile form a
-// rectangle; each warp owns 64 pixels of the tile (two blocks of 8 x 4).
+// kernels), SIDE x SIDE pixels by THREADS threads.  The pixels of a candidate's
+// window that lie in the tile form a rectangle; each warp owns one or two
+// blocks of 8 x 4 pixels of the tile.
 // PREFETCH_TILE: the tile's plane rows are first asked into L2 (for batches,
 // whose planes outgrow L2; an image whose plane stays in L2 only pays for it).
 // COUNT: the work is counted when a.count_samples asks for it (the counting
 // code costs the walks and the bound even when it is off).
-template <typename T, bool PREFETCH_TILE = false, bool COUNT = true, int THREADS = ASSIGN_THREADS>
+template <typename T, bool PREFETCH_TILE = false, bool COUNT = true, int THREADS = ASSIGN_THREADS, int SIDE = TILE_SIDE>
 __device__ __forceinline__ void assign_tile(const SolveArgs &a, int tile, unsigned char *smem)
 {
-    constexpr int PIX_PER_THREAD = TILE_PIXELS / THREADS;
+    constexpr int PIX_PER_THREAD = SIDE * SIDE / THREADS;
     constexpr int WARPS = THREADS / 32;
-    constexpr int QUEUE = ASSIGN_QUEUES / WARPS;  // pairs a warp's queue holds
+    constexpr int QUEUE = assign_queues(SIDE) / WARPS;  // pairs a warp's queue holds
     constexpr int BUILD_UNROLL = 4;  // samples per lane in flight
     const T *__restrict__ plane = reinterpret_cast<const T *>(
         sizeof(T) == 16 ? (const void *)a.plane32 : (const void *)a.plane16);
     const int tx = tile % a.n_tx, ty = tile / a.n_tx;
-    const int x0 = tx * TILE_X, y0 = ty * TILE_Y;
+    const int x0 = tx * SIDE, y0 = ty * SIDE;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
-    unsigned long long *best = reinterpret_cast<unsigned long long *>(smem + AssignSmem::best);
-    int *misc = reinterpret_cast<int *>(smem + AssignSmem::misc);
+    unsigned long long *best = reinterpret_cast<unsigned long long *>(smem + AssignSmem<SIDE>::best);
+    int *misc = reinterpret_cast<int *>(smem + AssignSmem<SIDE>::misc);
 
     // this thread's pixels: block (warp * PIX_PER_THREAD + j) of the tile
     // (a warp's blocks lie side by side), lane within it
     auto my_pixel = [&](int j, int &qx, int &qy) {
         const int blk = warp + j * WARPS;
-        qx = x0 + (blk % (TILE_X / WARP_BLOCK_X)) * WARP_BLOCK_X + (lane % WARP_BLOCK_X);
-        qy = y0 + (blk / (TILE_X / WARP_BLOCK_X)) * WARP_BLOCK_Y + (lane / WARP_BLOCK_X);
+        qx = x0 + (blk % (SIDE / WARP_BLOCK_X)) * WARP_BLOCK_X + (lane % WARP_BLOCK_X);
+        qy = y0 + (blk / (SIDE / WARP_BLOCK_X)) * WARP_BLOCK_Y + (lane / WARP_BLOCK_X);
     };
 
     const int off = a.tile_off[tile];
@@ -240,7 +242,7 @@ __device__ __forceinline__ void assign_tile(const SolveArgs &a, int tile, unsign
     const int cnt = (int)max(0LL, min((long long)a.tile_off[tile + 1], a.tile_cap) - off);
     const bool fast = cnt <= MAX_TILE_CANDIDATES;
     // the records for this tile's candidates, then its maps
-    const TileLayout lay = tile_layout(fast ? cnt : 0);
+    const TileLayout lay = tile_layout<SIDE>(fast ? cnt : 0);
     int4 *rec0 = reinterpret_cast<int4 *>(smem + lay.rec0);
     int4 *rec1 = reinterpret_cast<int4 *>(smem + lay.rec1);
     int4 *rec2 = reinterpret_cast<int4 *>(smem + lay.rec2);
@@ -252,7 +254,7 @@ __device__ __forceinline__ void assign_tile(const SolveArgs &a, int tile, unsign
     int *cfirst = reinterpret_cast<int *>(smem + lay.cfirst);
     const uint32_t maps_u32 = smem_u32(smem + lay.maps);
     float2 *maps = reinterpret_cast<float2 *>(smem + lay.maps);
-    const int map_cap = a.map_cap > 0 ? a.map_cap + extra_map_pairs(fast ? cnt : 0) : 0;
+    const int map_cap = a.map_cap > 0 ? a.map_cap + extra_map_pairs<SIDE>(fast ? cnt : 0) : 0;
     if (tid == 0) {  // this tile's list is read: ready the counts for the next update
         a.tile_count[tile] = 0;
         a.tile_cursor[tile] = 0;
@@ -264,10 +266,10 @@ __device__ __forceinline__ void assign_tile(const SolveArgs &a, int tile, unsign
     // the tile's plane rows into L2 while the set-up runs, so that the map
     // build finds them there (x0 * sizeof(T) and the row pitch are multiples
     // of 16 bytes, and so is every row's length: the bulk prefetch's rules)
-    static_assert(TILE_Y <= 32, "one row per lane");
+    static_assert(SIDE <= 32, "one row per lane");
     if (PREFETCH_TILE && warp == WARPS - 1) {
-        const int rows = min(a.H - y0, TILE_Y);
-        const uint32_t bytes = (uint32_t)(min(TILE_X, a.pitch - x0) * (int)sizeof(T));
+        const int rows = min(a.H - y0, SIDE);
+        const uint32_t bytes = (uint32_t)(min(SIDE, a.pitch - x0) * (int)sizeof(T));
         if (lane < rows) {
             const T *p = plane + (long long)(y0 + lane) * a.pitch + x0;
             asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
@@ -299,10 +301,10 @@ __device__ __forceinline__ void assign_tile(const SolveArgs &a, int tile, unsign
     const auto write_records = [&](int rank, int id, const ClusterDev &cd) {
         cid[rank] = id;
         // window x tile (clipped to the image)
-        const int xa = max(cd.xlo, x0), xb = min(min(cd.xhi, x0 + TILE_X - 1), a.W - 1);
-        const int ya = max(cd.ylo, y0), yb = min(min(cd.yhi, y0 + TILE_Y - 1), a.H - 1);
+        const int xa = max(cd.xlo, x0), xb = min(min(cd.xhi, x0 + SIDE - 1), a.W - 1);
+        const int ya = max(cd.ylo, y0), yb = min(min(cd.yhi, y0 + SIDE - 1), a.H - 1);
         const int w = max(xb - xa + 1, 0), h = max(yb - ya + 1, 0);
-        static_assert(TILE_X == 32 && TILE_Y == 32, "a rectangle is two 32-bit masks");
+        static_assert(SIDE <= 32, "a rectangle is two 32-bit masks");
         const bool some = w > 0 && h > 0;
         const float kx = cd.xk - (float)x0, ky = cd.yk - (float)y0;
         const float K = BOUND_SCALE * fmaf(a.lam, fmaf(cd.L, cd.L, fmaf(cd.a, cd.a, cd.b * cd.b)),
@@ -354,7 +356,7 @@ __device__ __forceinline__ void assign_tile(const SolveArgs &a, int tile, unsign
         for (int j = 0; j < PIX_PER_THREAD; ++j) {
             int px, py;
             my_pixel(j, px, py);
-            best[(py - y0) * TILE_X + (px - x0)] = ~0ull;
+            best[(py - y0) * SIDE + (px - x0)] = ~0ull;
         }
     } else {
         // the id staging reuses the `best` words before they are initialised
@@ -373,7 +375,7 @@ __device__ __forceinline__ void assign_tile(const SolveArgs &a, int tile, unsign
             write_records(rank, myid, cd);
         }
         __syncthreads();
-        for (int i = tid; i < TILE_PIXELS; i += THREADS) best[i] = ~0ull;
+        for (int i = tid; i < SIDE * SIDE; i += THREADS) best[i] = ~0ull;
         if (warp == 0 && fast) {
             const int used = warp_scan_maps(area, box, mfirst, cfirst, cnt, map_cap, lane);
             if (lane == 0) misc[2] = used;
@@ -504,7 +506,7 @@ __device__ __forceinline__ void assign_tile(const SolveArgs &a, int tile, unsign
             if (c >= 0) {
                 int len;
                 const float D = pair_distance(px - x0, py - y0, c, len);
-                best[(py - y0) * TILE_X + (px - x0)] = pack_best(D, c);  // (the pixel's first D)
+                best[(py - y0) * SIDE + (px - x0)] = pack_best(D, c);  // (the pixel's first D)
 #pragma unroll
                 for (int i = 0; i < PIX_PER_THREAD; ++i)
                     if (i == j) dprev[i] = D;
@@ -521,14 +523,14 @@ __device__ __forceinline__ void assign_tile(const SolveArgs &a, int tile, unsign
         // evens out.)  The pixels' samples are at hand only while the queue
         // fills: held across the walks as well they spill registers (FP32, HD
         // 140.0 us a launch against 134.7).
-        static_assert(WARPS % (TILE_X / WARP_BLOCK_X) == 0, "the warp's blocks lie in one column of blocks");
+        static_assert(WARPS % (SIDE / WARP_BLOCK_X) == 0, "the warp's blocks lie in one column of blocks");
         static_assert(PIX_PER_THREAD <= 2 && MAX_TILE_CANDIDATES <= 1024, "queued pairs pack into 16 bits");
         static_assert(QUEUE > 32 * PIX_PER_THREAD, "a queue takes a candidate's pairs after a full batch is left over");
-        constexpr int ROW_STEP = WARPS / (TILE_X / WARP_BLOCK_X) * WARP_BLOCK_Y;  // block 1 lies this far below block 0
+        constexpr int ROW_STEP = WARPS / (SIDE / WARP_BLOCK_X) * WARP_BLOCK_Y;  // block 1 lies this far below block 0
         int px, py;
         my_pixel(0, px, py);
         const int bx = px - lane % WARP_BLOCK_X, by = py - lane / WARP_BLOCK_X;
-        uint16_t *wq = reinterpret_cast<uint16_t *>(smem + AssignSmem::queue) + warp * QUEUE;
+        uint16_t *wq = reinterpret_cast<uint16_t *>(smem + AssignSmem<SIDE>::queue) + warp * QUEUE;
         int queued = 0, c0 = -32;                    // warp-uniform, as all that follows
         unsigned meets[PIX_PER_THREAD] = {}, any = 0;  // candidates c0 + bit left, per block and over both
         for (bool more = true; more;) {
@@ -603,7 +605,7 @@ __device__ __forceinline__ void assign_tile(const SolveArgs &a, int tile, unsign
                 const int Y = by - y0 + (e & 31) / WARP_BLOCK_X + ((e >> 5) & 1) * ROW_STEP;
                 int len;
                 const float D = pair_distance(X, Y, c, len);
-                atomicMin(&best[Y * TILE_X + X], pack_best(D, c));
+                atomicMin(&best[Y * SIDE + X], pack_best(D, c));
                 count_pair(len);
             }
             if (more) {  // the pairs left over start the next queue
@@ -662,7 +664,7 @@ __device__ __forceinline__ void assign_tile(const SolveArgs &a, int tile, unsign
         int lab = -1;
         if (valid) {
             if (fast) {
-                const unsigned long long b = best[(py - y0) * TILE_X + (px - x0)];
+                const unsigned long long b = best[(py - y0) * SIDE + (px - x0)];
                 if (b != ~0ull) lab = cid[(int)(b & 0xffffffffu)];
             } else if (bestk[j] != INT_MAX) {
                 lab = bestk[j];

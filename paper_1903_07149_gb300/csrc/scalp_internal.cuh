@@ -9,12 +9,11 @@
 
 namespace scalp {
 
-// Assignment tile: a CTA labels TILE_X x TILE_Y pixels.  For the reduction a
-// warp takes 8 x 4 blocks of them (one pixel per lane), so the labels a warp
-// sums are spatially coherent.
-constexpr int TILE_X = 32;
-constexpr int TILE_Y = 32;
-constexpr int TILE_PIXELS = TILE_X * TILE_Y;
+// Assignment tile: a CTA labels TILE_SIDE x TILE_SIDE pixels, or for a single
+// small image TILE_SIDE_SMALL x TILE_SIDE_SMALL (small_tiles() in
+// scalp_assign.cu).  For the reduction a warp takes 8 x 4 blocks of them (one
+// pixel per lane), so the labels a warp sums are spatially coherent.
+constexpr int TILE_SIDE = 32, TILE_SIDE_SMALL = 16;
 constexpr int WARP_BLOCK_X = 8;
 constexpr int WARP_BLOCK_Y = 4;
 // Candidate clusters of one tile held in shared memory.  A tile with more
@@ -214,6 +213,7 @@ struct SolveArgs {
     double r;          // sqrt(N/K)
     float lam, gamma, sigma, ms2;  // ms2 = m^2 / r^2
     int n_tx, n_ty;    // tiles
+    int tile_shift;    // their side is 2^tile_shift pixels
     int map_cap;       // distance-map pairs per assignment CTA (0: every path on the plane)
     int pitch;         // plane row pitch in pixels (>= W, multiple of 4)
     // grid column of the set-up, floor(x * nx / W), as a multiply-high by

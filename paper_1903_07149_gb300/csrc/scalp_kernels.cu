@@ -515,8 +515,8 @@ __device__ __forceinline__ void lists_cta(const SolveArgs &a, int blk, int nblk,
         const int j = (int)(i - (long long)k * tpw);
         const ClusterDev cd = a.cdev[k];
         if (cd.xlo > cd.xhi) continue;
-        const int tx = cd.xlo / TILE_X + j % a.tpw_x, ty = cd.ylo / TILE_Y + j / a.tpw_x;
-        if (tx > cd.xhi / TILE_X || ty > cd.yhi / TILE_Y) continue;
+        const int tx = (cd.xlo >> a.tile_shift) + j % a.tpw_x, ty = (cd.ylo >> a.tile_shift) + j / a.tpw_x;
+        if (tx > cd.xhi >> a.tile_shift || ty > cd.yhi >> a.tile_shift) continue;
         const int t = ty * a.n_tx + tx;
         const int pos = s_off[t] + atomicAdd(&a.tile_cursor[t], 1);
         if (pos < a.tile_cap) a.tile_list[pos] = k;

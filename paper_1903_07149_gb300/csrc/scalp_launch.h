@@ -1,9 +1,8 @@
 // scalp_launch.h -- host-side launchers of the libscalp kernels (internal).
 #pragma once
 
+#include "../../include/scalp.h"
 #include "scalp_internal.cuh"
-
-typedef struct scalp_ctx scalp_ctx;
 
 #include <utility>
 
@@ -74,13 +73,18 @@ void launch_batch_update(const BatchArgs &b, int total_clusters, int total_fill,
                          bool pdl = false, cudaStream_t side = nullptr, cudaEvent_t fork = nullptr,
                          cudaEvent_t join = nullptr, int whole_image = 0);
 // Assignment (Algorithm 1 inner loops, Eq. 1-3) with a.map_cap distance-map
-// pairs per CTA; smem_bytes = assign_smem_bytes(a.map_cap).
+// pairs per CTA; smem_bytes = assign_smem_bytes(a.map_cap, tile side).
 void launch_assign(const SolveArgs &a, int storage, size_t smem_bytes, cudaStream_t st, bool pdl = false);
-size_t assign_smem_bytes(int map_cap);
+size_t assign_smem_bytes(int map_cap, int side);
 // Whether the assignment may prune with these sizes and weights.
 bool bound_valid(int H, int W, float lam, float ms2);
-// Distance-map pairs that fit when ASSIGN_CTAS_PER_SM assignment CTAs share an SM.
-int assign_map_capacity(int device);
+// Distance-map pairs of an assignment CTA for a grid of `tiles` tiles.
+int assign_map_capacity(int device, int side, int tiles);
+// Whether a single image is cut into TILE_SIDE_SMALL tiles.
+bool small_tiles(int H, int W, double r);
+// scalp_init() for an image of a batch or a served request: TILE_SIDE tiles.
+int scalp_init_batched(scalp_ctx **out, const scalp_image *image, const scalp_contour *contour, int32_t K, float m,
+                       const scalp_params *params);
 cudaError_t assign_configure(int storage);
 // Debug: record the pixels of M paths.
 void launch_debug_paths(const int *pairs, int M, int *out_xy, int stride_xy, int *out_len,

@@ -192,8 +192,8 @@ __device__ __forceinline__ void update_cluster(const SolveArgs &a, int k, int fr
     }
     a.cdev[k] = cd;
     if (ok) {
-        for (int ty = cd.ylo / TILE_Y; ty <= cd.yhi / TILE_Y; ++ty)
-            for (int tx = cd.xlo / TILE_X; tx <= cd.xhi / TILE_X; ++tx)
+        for (int ty = cd.ylo >> a.tile_shift; ty <= cd.yhi >> a.tile_shift; ++ty)
+            for (int tx = cd.xlo >> a.tile_shift; tx <= cd.xhi >> a.tile_shift; ++tx)
                 atomicAdd(&a.tile_count[ty * a.n_tx + tx], 1);
     }
     if (check_projection && label_at_end != k) {
@@ -291,8 +291,8 @@ __device__ __forceinline__ void update_cluster_lanes(const SolveArgs &a, int k, 
     if (ok) {
         // the window's tiles, one per lane in turn (one division for the
         // lane's first, then steps of UPDATE_LANES)
-        const int tx0 = cd.xlo / TILE_X, ty0 = cd.ylo / TILE_Y;
-        const int nx = cd.xhi / TILE_X - tx0 + 1, nt = nx * (cd.yhi / TILE_Y - ty0 + 1);
+        const int tx0 = cd.xlo >> a.tile_shift, ty0 = cd.ylo >> a.tile_shift;
+        const int nx = (cd.xhi >> a.tile_shift) - tx0 + 1, nt = nx * ((cd.yhi >> a.tile_shift) - ty0 + 1);
         for (int t = j; t < nt; t += UPDATE_LANES)
             atomicAdd(&a.tile_count[(ty0 + t / nx) * a.n_tx + tx0 + t % nx], 1);
     }
@@ -579,8 +579,8 @@ __device__ __forceinline__ void fill_slot(const SolveArgs &a, long long i)
     const int k = (int)(i / slots), j = (int)(i % slots);
     const ClusterDev cd = a.cdev[k];
     if (cd.xlo > cd.xhi) return;
-    const int tx = cd.xlo / TILE_X + j % a.tpw_x, ty = cd.ylo / TILE_Y + j / a.tpw_x;
-    if (tx > cd.xhi / TILE_X || ty > cd.yhi / TILE_Y) return;
+    const int tx = (cd.xlo >> a.tile_shift) + j % a.tpw_x, ty = (cd.ylo >> a.tile_shift) + j / a.tpw_x;
+    if (tx > cd.xhi >> a.tile_shift || ty > cd.yhi >> a.tile_shift) return;
     const int t = ty * a.n_tx + tx;
     const int pos = a.tile_off[t] + atomicAdd(&a.tile_cursor[t], 1);
     if (pos < a.tile_cap) a.tile_list[pos] = k;

@@ -300,7 +300,7 @@ int scalp_server_submit(scalp_server *s, const scalp_image *image, const scalp_c
     p.workspace_bytes = bytes;
     cudaStream_t side = s->side[s->side_next++ % SIDE_STREAMS];
     p.stream = side;
-    int rc = scalp_init(&v->ctx, image, contour, K, m, &p);
+    int rc = scalp_init_batched(&v->ctx, image, contour, K, m, &p);
     if (rc != SCALP_OK) {
         pool_free(s, off, bytes);
         delete v;
