@@ -171,8 +171,8 @@ def whole_job_value(units_per_rank: float, world: int, slowest_ms: float) -> flo
 
 def ccl_launches(H: int, W: int) -> int:
     """Connectivity kernels: tile-local, border (when there is more than one
-    tile), flatten/count, link, resolve/count, chunk scan, numbering, output."""
-    return 7 + (1 if H > 32 or W > 32 else 0)
+    tile), flatten/count, resolve/count, numbering, output."""
+    return 5 + (1 if H > 32 or W > 32 else 0)
 
 
 def kernel_hash() -> str:

@@ -494,6 +494,7 @@ static int init_ctx(scalp_ctx **out, const scalp_image *image, const scalp_conto
     static_assert(TILE_SIDE == 32 && TILE_SIDE_SMALL == 16, "tile shifts");
     a.pitch = L.pitch;
     a.grid_rcp_x = grid_reciprocal(W, c->nx);
+    a.setup_rows = batched ? SETUP_ROWS : setup_rows(H, W, c->ny);
     a.plane32 = params->storage == 0 ? reinterpret_cast<const float4 *>(c->ws + L.plane) : nullptr;
     a.plane16 = params->storage == 1 ? reinterpret_cast<const uint2 *>(c->ws + L.plane) : nullptr;
     a.labels = reinterpret_cast<int *>(c->ws + L.labels);
@@ -614,9 +615,9 @@ int scalp_labels(scalp_ctx *c, int32_t *out, int32_t out_on_device, int32_t enfo
     size_t bytes = sizeof(int) * (size_t)c->N;
     if (enforce) {
         // the final labels go straight to a device output (which must not alias
-        // the workspace), else to the link buffer, free once the links are
+        // the workspace), else to the size buffer, free once the components are
         // resolved, and from there to the host
-        int *dst = out_on_device ? out : c->ccl.link;
+        int *dst = out_on_device ? out : c->ccl.size;
         int *d_nlab = &c->a.ctr->n_labels;  // read back with the counters
         launch_ccl(c->a.labels, c->H, c->W, c->K, dst, c->ccl, d_nlab, c->a.ctr, c->st);
         rc = launch_check(c, "connectivity kernels");
@@ -955,9 +956,9 @@ int scalp_ctx_enqueue_labels(scalp_ctx *c, int32_t *out, int enforce, CtxStatus 
     const int *src = c->a.labels;
     const int *d_nlab = reinterpret_cast<const int *>(c->ws + c->L.nlab);
     if (enforce) {
-        launch_ccl(c->a.labels, c->H, c->W, c->K, c->ccl.link, c->ccl, const_cast<int *>(d_nlab),
+        launch_ccl(c->a.labels, c->H, c->W, c->K, c->ccl.size, c->ccl, const_cast<int *>(d_nlab),
                    c->a.ctr, c->st);
-        src = c->ccl.link;
+        src = c->ccl.size;
     }
     int rc = launch_check(c, "connectivity kernels");
     if (rc) return rc;
@@ -1312,7 +1313,7 @@ int scalp_batch_init(scalp_batch **out, int32_t count, const scalp_image *images
         add(tile_base, i, (long long)c->a.n_tx * c->a.n_ty);
         add(clus_base, i, c->Keff);
         add(fill_base, i, (long long)c->Keff * c->a.tpw_x * c->a.tpw_y);
-        add(setup_base, i, setup_blocks(c->H, c->W, c->ny));
+        add(setup_base, i, setup_blocks(c->a));
         b->zero_parts = std::max(b->zero_parts, zero_blocks(c->Keff, c->a.n_tx * c->a.n_ty));
         long long blocks[CCL_KINDS];
         ccl_batch_blocks(c->H, c->W, blocks);
@@ -1331,6 +1332,7 @@ int scalp_batch_init(scalp_batch **out, int32_t count, const scalp_image *images
         m.T = c->N / (4LL * c->K);
         m.H = c->H;
         m.W = c->W;
+        b->cb.scanned = b->cb.scanned || ccl_scanned(c->N);
         m.n_tx = (c->W + 31) / 32;
         m.n_ty = (c->H + 31) / 32;
         b->smem = std::max(b->smem, c->smem);
@@ -1548,7 +1550,7 @@ int scalp_batch_labels(scalp_batch *b, int32_t *const *outs, int32_t out_on_devi
         // caller's buffers or the images' staging; the passes also gather
         // the label counts and the counters
         std::vector<int *> dst(b->count);
-        for (int i = 0; i < b->count; ++i) dst[i] = out_on_device ? outs[i] : b->ctx[i]->ccl.link;
+        for (int i = 0; i < b->count; ++i) dst[i] = out_on_device ? outs[i] : b->ctx[i]->ccl.size;
         e = b->out_table.upload(dst.data(), b->st);
         if (e == cudaSuccess) {
             launch_ccl_batch(b->cb, b->ccl_total, b->st);

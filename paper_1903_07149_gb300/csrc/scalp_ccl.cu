@@ -238,66 +238,9 @@ __device__ __forceinline__ void ccl_flatten_count(int *parent, int *size, long l
     }
 }
 
-// Four consecutive pixels per thread (one 16-byte load of their parents; the
-// buffers are 256-byte aligned).
-// The four parents from quad g (16-byte aligned buffers); -1 past N.
-__device__ __forceinline__ int4 load_quad(const int *__restrict__ a, long long g, long long N)
-{
-    const long long s0 = 4 * g;
-    if (s0 + 4 <= N) return reinterpret_cast<const int4 *>(a)[g];
-    return make_int4(s0 < N ? a[s0] : -1, s0 + 1 < N ? a[s0 + 1] : -1, s0 + 2 < N ? a[s0 + 2] : -1,
-                     s0 + 3 < N ? a[s0 + 3] : -1);
-}
-
-// Quads per thread and round in the passes below: their loads are issued
-// together before any is used.
-constexpr int CCL_QUAD_ROUND = 4;
-
-__device__ __forceinline__ void ccl_link(const int *__restrict__ parent, const int *__restrict__ size, int *link,
-                                         int W, long long N, long long T, unsigned blk, unsigned nblk)
-{
-    const long long quads = (N + 3) / 4, stride = (long long)nblk * blockDim.x;
-    for (long long g0 = blk * (long long)blockDim.x + threadIdx.x; g0 < quads; g0 += stride * CCL_QUAD_ROUND) {
-        int4 q[CCL_QUAD_ROUND];
-#pragma unroll
-        for (int u = 0; u < CCL_QUAD_ROUND; ++u) {
-            const long long g = g0 + u * stride;
-            q[u] = g < quads ? load_quad(parent, g, N) : make_int4(-1, -1, -1, -1);
-        }
-        // the sizes of the same quads, streamed alike (only seeds' entries
-        // are meaningful)
-        int4 z[CCL_QUAD_ROUND];
-#pragma unroll
-        for (int u = 0; u < CCL_QUAD_ROUND; ++u) {
-            const long long g = g0 + u * stride;
-            z[u] = g < quads ? load_quad(size, g, N) : make_int4(0, 0, 0, 0);
-        }
-#pragma unroll
-        for (int u = 0; u < CCL_QUAD_ROUND; ++u) {
-            const long long s0 = 4 * (g0 + u * stride);
-            const int pv[4] = {q[u].x, q[u].y, q[u].z, q[u].w};
-            const int zv[4] = {z[u].x, z[u].y, z[u].z, z[u].w};
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const long long s = s0 + i;
-                if (pv[i] != s) continue;
-                const bool small = zv[i] <= T && s != 0;
-                int to = (int)s;
-                if (small) {
-                    // the pixel before s (in this quad unless i = 0), else
-                    // the one above for column 0; N <= 2^30
-                    if (((int)s % W) > 0) to = i > 0 ? pv[i - 1] : parent[s - 1];
-                    else to = parent[s - W];
-                }
-                link[s] = to;
-            }
-        }
-    }
-}
-
 // Numbering works on chunks of CCL_CHUNK pixels, one CTA each.
 constexpr int CCL_CHUNK = 4096;
-constexpr int CCL_CHUNK_THREADS = 256;
+constexpr int CCL_CHUNK_THREADS = 512;
 constexpr int CCL_PER = CCL_CHUNK / CCL_CHUNK_THREADS;  // consecutive pixels per thread
 static_assert(CCL_PER % 4 == 0, "runs are read as int4");
 
@@ -330,33 +273,37 @@ __device__ __forceinline__ int cta_sum(int v, int *s_warp)
     return t;
 }
 
-// final[s] = first non-small ancestor of seed s (written over size[]), and
-// per chunk the number of surviving components (seeds with final[s] == s).
-__device__ __forceinline__ void ccl_resolve_count(const int *__restrict__ parent, const int *__restrict__ link,
-                                                  int *final_id, long long N, DevCounters *ctr, int *chunk_count,
-                                                  unsigned chunk)
+// final[s] = first non-small ancestor of seed s, and per chunk the number of
+// surviving components (seeds with final[s] == s).  A small component joins
+// the component of the pixel before its seed, or in column 0 of the one above,
+// whose seed is smaller: the chain is followed from the sizes and parents
+// themselves.  (With a pass of its own that first wrote every seed's link, the
+// two took 25.7 us on an HD image and 243 on the batch of 64; this one takes
+// 18.3 and 143.  The seeds are taken one by one from a mask: the chains written
+// out for each of a thread's pixels took 27.4 us.)  N <= 2^30.
+__device__ __forceinline__ void ccl_resolve_count(const int *__restrict__ parent, const int *__restrict__ size,
+                                                  int *final_id, int W, long long N, long long T, DevCounters *ctr,
+                                                  int *chunk_count, unsigned chunk)
 {
     __shared__ int s_warp[32];
-    // CCL_PER consecutive pixels per thread, their parents and links loaded
-    // first (a seed's link sits at its own index; other entries are unused)
+    // CCL_PER consecutive pixels per thread; a seed is its own parent
     const long long base = chunk * (long long)CCL_CHUNK + (long long)threadIdx.x * CCL_PER;
-    int par[CCL_PER], lk[CCL_PER];
+    int par[CCL_PER];
     load_run(parent, base, N, par);
-    load_run(link, base, N, lk);
-    int cnt = 0;
+    unsigned seeds = 0u;
 #pragma unroll
-    for (int i = 0; i < CCL_PER; ++i) {
-        const long long s = base + i;
-        if (par[i] != s) continue;
-        int f = (int)s, nf = lk[i];
+    for (int i = 0; i < CCL_PER; ++i) seeds |= par[i] == (int)(base + i) ? 1u << i : 0u;
+    int cnt = 0;
+    for (; seeds; seeds &= seeds - 1) {
+        const int s = (int)base + __ffs(seeds) - 1;
+        int f = s;
         long long guard = 0;
-        while (nf != f) {
-            f = nf;
+        while (f != 0 && size[f] <= T) {
+            f = parent[f % W == 0 ? f - W : f - 1];
             if (++guard > N) {
                 atomicExch(&ctr->error, ERR_CCL_CHAIN);
                 break;
             }
-            nf = link[f];
         }
         final_id[s] = f;
         cnt += f == s;
@@ -402,13 +349,33 @@ __device__ __forceinline__ void ccl_chunk_scan(int *counts, long long n, int *to
     if (threadIdx.x == CCL_SCAN_THREADS - 1) *total = s_warp[31];
 }
 
+// The surviving components of chunks [0, chunk), by the chunk's own CTA (every
+// thread receives it).  Up to CCL_SUM_CHUNKS chunks (33 million pixels) each
+// CTA sums the counts before its own instead of waiting for the scan kernel
+// (2.9 us, and a launch); the sums grow with the square of the chunks, so
+// larger images keep the scan.
+constexpr long long CCL_SUM_CHUNKS = 8192;
+bool ccl_scanned(long long N) { return ceil_div_ll(N, CCL_CHUNK) > CCL_SUM_CHUNKS; }
+
+__device__ __forceinline__ int ccl_count_before(const int *__restrict__ counts, unsigned chunk, int *s_warp)
+{
+    int v = 0;
+    for (unsigned i = threadIdx.x; i < chunk; i += blockDim.x) v += counts[i];
+    return cta_sum(v, s_warp);
+}
+
 // number[s] for each surviving seed s: its rank in raster order (the chunk's
-// offset plus the rank inside the chunk); only seeds are written.
+// offset plus the rank inside the chunk); only seeds are written.  The last
+// chunk writes the number of labels to *total.
 __device__ __forceinline__ void ccl_number(const int *__restrict__ parent, const int *__restrict__ final_id,
-                                           const int *__restrict__ chunk_off, int *number, long long N,
-                                           unsigned chunk)
+                                           const int *__restrict__ chunk_count, int *number, long long N,
+                                           unsigned chunk, int *total, bool scanned)
 {
     __shared__ int s_warp[32];
+    // (after the scan the counts are offsets, and the total is written)
+    const int before = scanned ? chunk_count[chunk] : ccl_count_before(chunk_count, chunk, s_warp);
+    if (!scanned && (chunk + 1) * (long long)CCL_CHUNK >= N && threadIdx.x == 0)
+        *total = before + chunk_count[chunk];
     const long long base = chunk * (long long)CCL_CHUNK + (long long)threadIdx.x * CCL_PER;
     int par[CCL_PER];
     load_run(parent, base, N, par);
@@ -436,7 +403,7 @@ __device__ __forceinline__ void ccl_number(const int *__restrict__ parent, const
         s_warp[lane] = w;
     }
     __syncthreads();
-    int rank = chunk_off[chunk] + (wid ? s_warp[wid - 1] : 0) + incl - mine;
+    int rank = before + (wid ? s_warp[wid - 1] : 0) + incl - mine;
     while (flags) {
         const int i = __ffs(flags) - 1;
         number[base + i] = rank++;
@@ -498,21 +465,13 @@ __global__ void k_ccl_flatten_count(int *parent, int *size, long long N)
     ccl_flatten_count(parent, size, N, blockIdx.x, gridDim.x);
 }
 
-__global__ void k_ccl_link(const int *__restrict__ parent, const int *__restrict__ size, int *link, int W,
-                           long long N, long long T)
-{
-    pdl_wait();
-    pdl_release();
-    ccl_link(parent, size, link, W, N, T, blockIdx.x, gridDim.x);
-}
-
 __global__ void __launch_bounds__(CCL_CHUNK_THREADS)
-    k_ccl_resolve_count(const int *__restrict__ parent, const int *__restrict__ link, int *final_id,
-                        long long N, DevCounters *ctr, int *chunk_count)
+    k_ccl_resolve_count(const int *__restrict__ parent, const int *__restrict__ size, int *final_id, int W,
+                        long long N, long long T, DevCounters *ctr, int *chunk_count)
 {
     pdl_wait();
     pdl_release();
-    ccl_resolve_count(parent, link, final_id, N, ctr, chunk_count, blockIdx.x);
+    ccl_resolve_count(parent, size, final_id, W, N, T, ctr, chunk_count, blockIdx.x);
 }
 
 __global__ void __launch_bounds__(CCL_SCAN_THREADS) k_ccl_chunk_scan(int *counts, long long n, int *total)
@@ -524,11 +483,11 @@ __global__ void __launch_bounds__(CCL_SCAN_THREADS) k_ccl_chunk_scan(int *counts
 
 __global__ void __launch_bounds__(CCL_CHUNK_THREADS)
     k_ccl_number(const int *__restrict__ parent, const int *__restrict__ final_id,
-                 const int *__restrict__ chunk_off, int *number, long long N)
+                 const int *__restrict__ chunk_count, int *number, long long N, int *total, bool scanned)
 {
     pdl_wait();
     pdl_release();
-    ccl_number(parent, final_id, chunk_off, number, N, blockIdx.x);
+    ccl_number(parent, final_id, chunk_count, number, N, blockIdx.x, total, scanned);
 }
 
 __global__ void k_ccl_out(const int *__restrict__ parent, const int *__restrict__ final_id,
@@ -584,43 +543,34 @@ __global__ void k_ccl_flatten_count_batch(CclBatch cb)
     ccl_flatten_count(m.parent, m.size, m.N, b.blk, b.nblk);
 }
 
-__global__ void k_ccl_link_batch(CclBatch cb)
-{
-    pdl_wait();
-    pdl_release();
-    const CclBlock b = ccl_block(cb, CCL_KIND_QUADS);
-    const CclImage &m = cb.img[b.i];
-    ccl_link(m.parent, m.size, m.link, m.W, m.N, m.T, b.blk, b.nblk);
-}
-
 __global__ void __launch_bounds__(CCL_CHUNK_THREADS) k_ccl_resolve_count_batch(CclBatch cb)
 {
     pdl_wait();
     pdl_release();
     const CclBlock b = ccl_block(cb, CCL_KIND_CHUNKS);
     const CclImage &m = cb.img[b.i];
-    ccl_resolve_count(m.parent, m.link, m.size, m.N, m.ctr, m.scan_tmp, b.blk);
+    ccl_resolve_count(m.parent, m.size, m.link, m.W, m.N, m.T, m.ctr, m.scan_tmp, b.blk);
 }
 
-// One CTA per image; it also copies the image's counters (no later pass
-// writes them) to where the host gathers them.
+// One CTA per image.
 __global__ void __launch_bounds__(CCL_SCAN_THREADS) k_ccl_chunk_scan_batch(CclBatch cb)
 {
     pdl_wait();
     pdl_release();
-    const int i = blockIdx.x;
-    const CclImage &m = cb.img[i];
+    const CclImage &m = cb.img[blockIdx.x];
     ccl_chunk_scan(m.scan_tmp, ceil_div_ll(m.N, CCL_CHUNK), m.nlab);
-    if (threadIdx.x == 0) *m.ctr_out = *m.ctr;
 }
 
+// (the image's counters, which no later pass writes, go to where the host
+// gathers them)
 __global__ void __launch_bounds__(CCL_CHUNK_THREADS) k_ccl_number_batch(CclBatch cb)
 {
     pdl_wait();
     pdl_release();
     const CclBlock b = ccl_block(cb, CCL_KIND_CHUNKS);
     const CclImage &m = cb.img[b.i];
-    ccl_number(m.parent, m.size, m.scan_tmp, m.scan, m.N, b.blk);
+    ccl_number(m.parent, m.link, m.scan_tmp, m.scan, m.N, b.blk, m.nlab, cb.scanned);
+    if (b.blk == 0 && threadIdx.x == 0) *m.ctr_out = *m.ctr;
 }
 
 __global__ void k_ccl_out_batch(CclBatch cb)
@@ -629,7 +579,7 @@ __global__ void k_ccl_out_batch(CclBatch cb)
     pdl_release();
     const CclBlock b = ccl_block(cb, CCL_KIND_QUADS);
     const CclImage &m = cb.img[b.i];
-    ccl_out(m.parent, m.size, m.scan, cb.out[b.i], m.N, b.blk, b.nblk);
+    ccl_out(m.parent, m.link, m.scan, cb.out[b.i], m.N, b.blk, b.nblk);
 }
 
 long long ccl_scan_tmp_len(long long N) { return ceil_div_ll(N, CCL_CHUNK) + 64; }
@@ -649,16 +599,16 @@ void launch_ccl(const int *labels, int H, int W, int K, int *out, const CclBuffe
         pdl_launch(true, k_ccl_border, dim3((unsigned)std::min<long long>(ceil_div_ll(nb, CCL_THREADS), 152 * 16)),
                    dim3(CCL_THREADS), 0, st, labels, b.parent, H, W, n_tx, n_ty);
     pdl_launch(true, k_ccl_flatten_count, dim3(blocks), dim3(CCL_THREADS), 0, st, b.parent, b.size, N);
-    pdl_launch(true, k_ccl_link, dim3(qblocks), dim3(CCL_THREADS), 0, st, (const int *)b.parent,
-               (const int *)b.size, b.link, W, N, T);
     const long long chunks = ceil_div_ll(N, CCL_CHUNK);
     pdl_launch(true, k_ccl_resolve_count, dim3((unsigned)chunks), dim3(CCL_CHUNK_THREADS), 0, st,
-               (const int *)b.parent, (const int *)b.link, b.size, N, ctr, b.scan_tmp);
-    pdl_launch(true, k_ccl_chunk_scan, dim3(1), dim3(CCL_SCAN_THREADS), 0, st, b.scan_tmp, chunks, d_nlab);
+               (const int *)b.parent, (const int *)b.size, b.link, W, N, T, ctr, b.scan_tmp);
+    const bool scanned = ccl_scanned(N);
+    if (scanned)
+        pdl_launch(true, k_ccl_chunk_scan, dim3(1), dim3(CCL_SCAN_THREADS), 0, st, b.scan_tmp, chunks, d_nlab);
     pdl_launch(true, k_ccl_number, dim3((unsigned)chunks), dim3(CCL_CHUNK_THREADS), 0, st, (const int *)b.parent,
-               (const int *)b.size, (const int *)b.scan_tmp, b.scan, N);
+               (const int *)b.link, (const int *)b.scan_tmp, b.scan, N, d_nlab, scanned);
     pdl_launch(true, k_ccl_out, dim3(qblocks), dim3(CCL_THREADS), 0, st, (const int *)b.parent,
-               (const int *)b.size, (const int *)b.scan, out, N);
+               (const int *)b.link, (const int *)b.scan, out, N);
 }
 
 // Blocks of one image per pass in a batch.  A block first finds its image, so
@@ -684,9 +634,9 @@ void launch_ccl_batch(const CclBatch &cb, const int total[CCL_KINDS], cudaStream
     if (total[CCL_KIND_BORDER] > 0)
         pdl_launch(true, k_ccl_border_batch, dim3(total[CCL_KIND_BORDER]), dim3(CCL_THREADS), 0, st, cb);
     pdl_launch(true, k_ccl_flatten_count_batch, dim3(total[CCL_KIND_PIXELS]), dim3(CCL_THREADS), 0, st, cb);
-    pdl_launch(true, k_ccl_link_batch, dim3(total[CCL_KIND_QUADS]), dim3(CCL_THREADS), 0, st, cb);
     pdl_launch(true, k_ccl_resolve_count_batch, dim3(total[CCL_KIND_CHUNKS]), dim3(CCL_CHUNK_THREADS), 0, st, cb);
-    pdl_launch(true, k_ccl_chunk_scan_batch, dim3(cb.count), dim3(CCL_SCAN_THREADS), 0, st, cb);
+    if (cb.scanned)
+        pdl_launch(true, k_ccl_chunk_scan_batch, dim3(cb.count), dim3(CCL_SCAN_THREADS), 0, st, cb);
     pdl_launch(true, k_ccl_number_batch, dim3(total[CCL_KIND_CHUNKS]), dim3(CCL_CHUNK_THREADS), 0, st, cb);
     pdl_launch(true, k_ccl_out_batch, dim3(total[CCL_KIND_QUADS]), dim3(CCL_THREADS), 0, st, cb);
 }

@@ -23,6 +23,8 @@ constexpr int MAX_TILE_CANDIDATES = 128;
 // and tail overlap the other's path walks).
 constexpr int ASSIGN_THREADS = 512;
 constexpr int ASSIGN_CTAS_PER_SM = 2;
+// Rows of a task of the set-up (fewer for small images: setup_rows()).
+constexpr int SETUP_ROWS = 8;
 // Colour sums are kept as integers: value * 2^COLOR_FRAC_BITS, rounded.  CIELab
 // of 8-bit sRGB has |L|, |a|, |b| < 108, so 32 such values sum below 2^31.
 constexpr int COLOR_FRAC_BITS = 19;
@@ -219,6 +221,7 @@ struct SolveArgs {
     // grid column of the set-up, floor(x * nx / W), as a multiply-high by
     // ceil(2^32 / W) where that is exact; 0: divide
     unsigned grid_rcp_x;
+    int setup_rows;    // rows of a set-up task (at most SETUP_ROWS)
     int count_samples;
     int prune;         // 1: skip pairs whose lower bound exceeds the pixel's best D (0: evaluate all)
     const float4 *plane32;   // (L, a, b, w) per pixel, row pitch `pitch` [FP32 storage]

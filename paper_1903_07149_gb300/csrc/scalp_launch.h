@@ -97,6 +97,7 @@ struct CclBuffers {
     long long scan_tmp_len;
 };
 long long ccl_scan_tmp_len(long long N);
+bool ccl_scanned(long long N);
 void launch_ccl(const int *labels, int H, int W, int K, int *out, const CclBuffers &b,
                 int *d_nlab, DevCounters *ctr, cudaStream_t st);
 
@@ -118,6 +119,7 @@ struct CclBatch {
     int *const *out;           // per image: where its final labels go
     const int *base[CCL_KINDS];
     int count;
+    bool scanned;              // an image has so many chunks that their counts take the scan
 };
 void ccl_batch_blocks(int H, int W, long long blocks[CCL_KINDS]);
 void launch_ccl_batch(const CclBatch &cb, const int total[CCL_KINDS], cudaStream_t st);
@@ -132,7 +134,8 @@ struct SetupInput {
     const float *contour;
     long long rgb_stride, contour_stride;
 };
-long long setup_blocks(int H, int W, int ny);
+long long setup_blocks(const SolveArgs &a);
+int setup_rows(int H, int W, int ny);
 int zero_blocks(int Keff, int tiles);
 void launch_setup_batch(const BatchArgs &b, const SetupInput *in, const int *setup_base, int total_blocks,
                         int zero_parts, int storage, cudaStream_t st);
