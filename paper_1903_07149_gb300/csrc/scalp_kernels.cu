@@ -115,10 +115,7 @@ __device__ __forceinline__ void setup_task(const SolveArgs &a, const float *lin,
     static_assert((long long)SETUP_ROWS * 108 * (1LL << COLOR_FRAC_BITS) < (1LL << 31), "lane colour sums");
     int sL = 0, sa = 0, sb = 0;
     if (valid) {
-#pragma unroll 4
-        for (int y = y0; y < y1; ++y) {
-            const float3 c3 = srgb_to_lab(lin, rgb + y * rgb_stride + 3 * (long long)x);
-            const float c = contour ? contour[y * contour_stride + x] : 0.0f;
+        const auto store = [&](int y, float3 c3, float c) {
             const float w = -expm1f(-(c * c) * inv_s2);  // 1 - exp(-C^2/sigma^2), Eq. 2
             const long long q = (long long)y * a.pitch + x;
             float4 v;
@@ -137,6 +134,17 @@ __device__ __forceinline__ void setup_task(const SolveArgs &a, const float *lin,
             sL += __float2int_rn(v.x * scale);
             sa += __float2int_rn(v.y * scale);
             sb += __float2int_rn(v.z * scale);
+        };
+        // two rows at a time (an odd last one with itself)
+#pragma unroll 2
+        for (int y = y0; y < y1; y += 2) {
+            const int z = min(y + 1, y1 - 1);
+            const float cy0 = contour ? contour[y * contour_stride + x] : 0.0f;
+            const float cy1 = contour ? contour[z * contour_stride + x] : 0.0f;
+            float3 l0, l1;
+            srgb_to_lab2(lin, rgb + y * rgb_stride + 3 * (long long)x, rgb + z * rgb_stride + 3 * (long long)x, l0, l1);
+            store(y, l0, cy0);
+            if (z != y) store(z, l1, cy1);
         }
     }
     if (wait_sums) pdl_wait();
@@ -278,13 +286,19 @@ __global__ void __launch_bounds__(PRIOR_THREADS)
     if (tid == 0) s_max = 0u;
     __syncthreads();
     const int x0 = blockIdx.x * PRIOR_TX, y0 = blockIdx.y * PRIOR_TY;
-    const auto convert = [&](int hx, int hy) {
+    const auto at = [&](int hx, int hy) {
         const int x = min(max(x0 - 1 + hx, 0), W - 1), y = min(max(y0 - 1 + hy, 0), H - 1);
-        const float3 lab = srgb_to_lab(lin, rgb + y * rgb_stride + 3 * (long long)x);
-        s_lab[hy][hx] = make_float4(lab.x, lab.y, lab.z, 0.0f);
+        return rgb + y * rgb_stride + 3 * (long long)x;
     };
-    for (int hy = warp; hy < PRIOR_TY + 2; hy += WARPS) convert(lane, hy);
-    if (tid < 2 * (PRIOR_TY + 2)) convert(PRIOR_TX + (tid & 1), tid >> 1);
+    const auto convert = [&](int hx0, int hy0, int hx1, int hy1) {  // two places
+        float3 a, b;
+        srgb_to_lab2(lin, at(hx0, hy0), at(hx1, hy1), a, b);
+        s_lab[hy0][hx0] = make_float4(a.x, a.y, a.z, 0.0f);
+        s_lab[hy1][hx1] = make_float4(b.x, b.y, b.z, 0.0f);
+    };
+    static_assert((PRIOR_TY + 2) % 2 == 0, "rows in pairs");
+    for (int hy = 2 * warp; hy < PRIOR_TY + 2; hy += 2 * WARPS) convert(lane, hy, lane, hy + 1);
+    if (tid < PRIOR_TY + 2) convert(PRIOR_TX, tid, PRIOR_TX + 1, tid);
     __syncthreads();
     const int x = x0 + lane;
     float gm = 0.0f;

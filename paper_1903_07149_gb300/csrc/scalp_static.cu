@@ -130,10 +130,13 @@ __global__ void __launch_bounds__(SUM_THREADS)
                 px[u][1] = q[1];
                 px[u][2] = q[2];
             }
+            static_assert(SUM_BATCH % 2 == 0, "rows are converted in pairs");
+            float3 c[SUM_BATCH];
+#pragma unroll
+            for (int u = 0; u < SUM_BATCH; u += 2) srgb_to_lab2(lin, px[u], px[u + 1], c[u], c[u + 1]);
 #pragma unroll
             for (int u = 0; u < SUM_BATCH; ++u) {
                 if (yb + u >= y1) break;
-                const float3 c = srgb_to_lab(lin, px[u]);
                 const int k = label[u] < n_labels ? label[u] : -1;
                 if (k != run) {
                     if (run >= 0) hand_over();
@@ -142,9 +145,9 @@ __global__ void __launch_bounds__(SUM_THREADS)
                 }
                 n += 1;
                 sy += yb + u - y0;
-                sL += __float2int_rn(c.x * scale);
-                sa += __float2int_rn(c.y * scale);
-                sb += __float2int_rn(c.z * scale);
+                sL += __float2int_rn(c[u].x * scale);
+                sa += __float2int_rn(c[u].y * scale);
+                sb += __float2int_rn(c[u].z * scale);
             }
         }
         if (run >= 0) hand_over();
