@@ -486,6 +486,11 @@ int scalp_boundary_map(const int32_t *const *labels, int32_t count, int32_t H, i
 typedef struct {
     double br, asa, ue, co;
 } scalp_quality;
+/* n_labels and n_gt of two device maps of `pixels` int32 labels (their largest
+ * values plus one), in one pass over both.  workspace: 8 bytes on the device.
+ * Synchronises `stream`. */
+int scalp_label_counts(const int32_t *labels, const int32_t *gt, int64_t pixels, int32_t counts[2],
+                       void *workspace, size_t workspace_bytes, void *stream);
 size_t scalp_quality_workspace_bytes(int32_t H, int32_t W, int32_t n_labels, int32_t n_gt);
 int scalp_quality_metrics(const int32_t *labels, int32_t n_labels, const int32_t *gt, int32_t n_gt,
                           int32_t H, int32_t W, double eps, void *workspace, size_t workspace_bytes,

@@ -10,6 +10,7 @@
 // a decomposition iff one of its 4-neighbours carries another label; the map
 // is the fraction of the decompositions in which it is one.
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -389,6 +390,68 @@ size_t quality_layout(int n_labels, int n_gt, QualityWs *w, unsigned char *base)
 
 }  // namespace
 
+namespace {
+
+// The largest value of two maps of n pixels, raised into best[0] and best[1].
+__global__ void __launch_bounds__(512) k_map_maxima(const int *__restrict__ m0, const int *__restrict__ m1, long long n,
+                                                    int *best)
+{
+    __shared__ int s_best[2];
+    if (threadIdx.x < 2) s_best[threadIdx.x] = INT_MIN;
+    __syncthreads();
+    int b0 = INT_MIN, b1 = INT_MIN;
+    const bool vec = ((reinterpret_cast<uintptr_t>(m0) | reinterpret_cast<uintptr_t>(m1)) & 15) == 0;
+    const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x, step = (long long)gridDim.x * blockDim.x;
+    const long long quads = vec ? n / 4 : 0;
+    for (long long i = t; i < quads; i += step) {
+        const int4 a = reinterpret_cast<const int4 *>(m0)[i], c = reinterpret_cast<const int4 *>(m1)[i];
+        b0 = max(b0, max(max(a.x, a.y), max(a.z, a.w)));
+        b1 = max(b1, max(max(c.x, c.y), max(c.z, c.w)));
+    }
+    for (long long i = 4 * quads + t; i < n; i += step) {
+        b0 = max(b0, m0[i]);
+        b1 = max(b1, m1[i]);
+    }
+    b0 = __reduce_max_sync(0xffffffffu, b0);
+    b1 = __reduce_max_sync(0xffffffffu, b1);
+    if ((threadIdx.x & 31) == 0) {
+        atomicMax(&s_best[0], b0);
+        atomicMax(&s_best[1], b1);
+    }
+    __syncthreads();
+    if (threadIdx.x < 2) atomicMax(&best[threadIdx.x], s_best[threadIdx.x]);
+}
+
+}  // namespace
+
+// The label counts of a decomposition and a ground truth, one pass over both
+// and one read-back (two library reductions and a stack before).
+extern "C" int scalp_label_counts(const int32_t *labels, const int32_t *gt, int64_t pixels, int32_t counts[2],
+                                  void *workspace, size_t workspace_bytes, void *stream)
+{
+    if (!labels || !gt || !counts) return metrics_fail(SCALP_E_ARG, "labels, gt and counts are required");
+    if (pixels < 1) return metrics_fail(SCALP_E_ARG, "need at least one pixel");
+    if (!workspace || workspace_bytes < 8 || reinterpret_cast<uintptr_t>(workspace) % 4)
+        return metrics_fail(SCALP_E_NOMEM, "8 bytes of device workspace needed");
+    cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+    int *best = static_cast<int *>(workspace);
+    cudaError_t e = cudaMemsetAsync(best, 0x80, 8, st);  // below every label
+    if (e == cudaSuccess) {
+        const long long blocks = std::min<long long>((pixels + 4 * 512 - 1) / (4 * 512), 152 * 4);
+        k_map_maxima<<<(unsigned)blocks, 512, 0, st>>>(labels, gt, pixels, best);
+        e = cudaGetLastError();
+    }
+    int local[2];
+    int *h = reinterpret_cast<int *>(scalp::pinned_status_buffer());
+    if (!h) h = local;
+    if (e == cudaSuccess) e = cudaMemcpyAsync(h, best, 8, cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) return metrics_fail(SCALP_E_CUDA, "label counts: %s", cudaGetErrorString(e));
+    counts[0] = h[0] + 1;
+    counts[1] = h[1] + 1;
+    return SCALP_OK;
+}
+
 extern "C" size_t scalp_quality_workspace_bytes(int32_t H, int32_t W, int32_t n_labels, int32_t n_gt)
 {
     if (H < 1 || W < 1 || n_labels < 1 || n_gt < 1) return 0;
@@ -427,8 +490,11 @@ extern "C" int scalp_quality_metrics(const int32_t *labels, int32_t n_labels, co
         pdl_launch(true, k_quality_total, dim3(1), dim3(1024), 0, st, n_labels, N, w);
         e = cudaGetLastError();
     }
-    double r[4];
-    if (e == cudaSuccess) e = cudaMemcpyAsync(r, w.result, sizeof r, cudaMemcpyDeviceToHost, st);
+    double local[4];
+    static_assert(sizeof(DevCounters) >= sizeof local, "the pinned buffer holds the four metrics");
+    double *r = reinterpret_cast<double *>(scalp::pinned_status_buffer());
+    if (!r) r = local;
+    if (e == cudaSuccess) e = cudaMemcpyAsync(r, w.result, sizeof local, cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return metrics_fail(SCALP_E_CUDA, "quality metrics: %s", cudaGetErrorString(e));
     out->br = r[0];

@@ -99,7 +99,7 @@ EXPORTS = (
     "scalp_server_reserve_bytes", "scalp_server_create", "scalp_server_submit", "scalp_server_step",
     "scalp_server_poll", "scalp_server_stats", "scalp_server_destroy", "scalp_boundary_map",
     "scalp_server_set_step_budget",
-    "scalp_quality_workspace_bytes", "scalp_quality_metrics",
+    "scalp_label_counts", "scalp_quality_workspace_bytes", "scalp_quality_metrics",
     "scalp_gradient_prior_workspace_bytes", "scalp_gradient_prior",
     "scalp_voxel_workspace_bytes", "scalp_voxel_init", "scalp_voxel_iterate", "scalp_voxel_labels",
     "scalp_voxel_get_info", "scalp_voxel_get_state", "scalp_voxel_set_state",
@@ -176,6 +176,7 @@ def load(path: str = LIB_PATH) -> ctypes.CDLL:
             "scalp_server_inject_status": (ctypes.c_int, [P, ctypes.c_uint64, I32, I32]),
             "scalp_server_destroy": (None, [P]),
             "scalp_boundary_map": (ctypes.c_int, [P, I32, I32, I32, P, P]),
+            "scalp_label_counts": (ctypes.c_int, [P, P, I64, ctypes.POINTER(I32), P, ctypes.c_size_t, P]),
             "scalp_quality_workspace_bytes": (ctypes.c_size_t, [I32, I32, I32, I32]),
             "scalp_gradient_prior_workspace_bytes": (ctypes.c_size_t, [I32, I32, I32, I32]),
             "scalp_voxel_workspace_bytes": (ctypes.c_size_t, [I32, I32, I32, I32, ctypes.POINTER(scalp_params)]),
@@ -843,15 +844,22 @@ def quality_metrics(labels, gt, eps: float = 2.0, stream=None):
 
     stream = stream if stream is not None else torch.cuda.current_stream()
     H, W = int(labels.shape[0]), int(labels.shape[1])
-    # one read-back for both label counts
-    n_labels, n_gt = (int(v) + 1 for v in torch.stack((labels.max(), gt.max())).tolist())
+    lab = labels.contiguous()
+    g = gt.contiguous()
+    if lab.dtype == g.dtype == torch.int32 and lab.numel() == g.numel() > 0:
+        # both counts in one pass, on the stream that the maps are ready on
+        ws = torch.empty(8, dtype=torch.uint8, device="cuda")
+        n = (ctypes.c_int32 * 2)()
+        _check(load().scalp_label_counts(lab.data_ptr(), g.data_ptr(), lab.numel(), n, ws.data_ptr(), 8,
+                                         torch.cuda.current_stream().cuda_stream))
+        n_labels, n_gt = n[0], n[1]
+    else:
+        n_labels, n_gt = int(lab.max().item()) + 1, int(g.max().item()) + 1
     nbytes = scalp_quality_workspace_bytes(H, W, n_labels, n_gt)
     if nbytes == 0:
         raise ScalpError(SCALP_E_ARG, "invalid sizes for the quality metrics")
     ws = torch.empty(nbytes, dtype=torch.uint8, device="cuda")
     q = scalp_quality()
-    lab = labels.contiguous()
-    g = gt.contiguous()
     _check(load().scalp_quality_metrics(ctypes.c_void_p(lab.data_ptr()), n_labels,
                                         ctypes.c_void_p(g.data_ptr()), n_gt, H, W, float(eps),
                                         ctypes.c_void_p(ws.data_ptr()), nbytes, ctypes.byref(q),

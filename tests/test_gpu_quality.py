@@ -91,6 +91,10 @@ def test_quality_shapes_and_radii(S, H, W, eps):
     lab = np.where(rng.random((H, W)) < 0.03, rng.integers(0, 12, (H, W)), lab).astype(np.int32)
     gt = np.kron(rng.integers(0, 3, (H // 29 + 1, W // 41 + 1)), np.ones((29, 41), int))[:H, :W].astype(np.int32)
     got = S.quality_metrics(torch.from_numpy(lab).cuda(), torch.from_numpy(gt).cuda(), eps=eps)
+    # the same maps 4 bytes off a 16-byte boundary (the counts' vector loads)
+    a, b = (torch.from_numpy(np.concatenate([[m.max() + 5], m.ravel()]).astype(np.int32)).cuda()[1:].view(H, W)
+            for m in (lab, gt))
+    assert S.quality_metrics(a, b, eps=eps) == got
     ref = _reference(lab, gt, eps)
     assert got["br"] == ref["br"] and got["asa"] == ref["asa"] and got["ue"] == ref["ue"], (got, ref)
     assert got["co"] == pytest.approx(ref["co"], rel=1e-12)
