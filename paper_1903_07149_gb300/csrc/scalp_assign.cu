@@ -115,7 +115,12 @@ __global__ void __launch_bounds__(THREADS, 1024 / THREADS) k_assign(SolveArgs a)
     pdl_wait();
     pdl_release();
     extern __shared__ __align__(16) unsigned char smem[];
-    assign_tile<T, false, COUNT, THREADS, SIDE>(a, blockIdx.x, smem);
+    // a grid of the image's tiles, or (more rows of them than a grid can have)
+    // one row of all
+    const int tile = (int)(blockIdx.y * gridDim.x + blockIdx.x);
+    const bool flat = gridDim.x != (unsigned)a.n_tx;
+    assign_tile<T, false, COUNT, THREADS, SIDE>(a, tile, flat ? tile % a.n_tx : (int)blockIdx.x,
+                                                flat ? tile / a.n_tx : (int)blockIdx.y, smem);
 }
 
 // All tiles of all images of a batch in one launch: block g is tile
@@ -138,7 +143,8 @@ __global__ void __launch_bounds__(ASSIGN_THREADS, ASSIGN_CTAS_PER_SM) k_assign_b
     if (threadIdx.x < sizeof(SolveArgs) / 4)
         reinterpret_cast<int *>(&a)[threadIdx.x] = reinterpret_cast<const int *>(&b.args[i])[threadIdx.x];
     __syncthreads();
-    assign_tile<T, true, COUNT>(a, g - b.tile_base[i], smem);
+    const int tile = g - b.tile_base[i];
+    assign_tile<T, true, COUNT>(a, tile, tile % a.n_tx, tile / a.n_tx, smem);
 }
 
 template <typename T, bool COUNT>
@@ -146,7 +152,7 @@ static void launch_assign_as(const SolveArgs &a, size_t smem_bytes, cudaStream_t
 {
     const int tiles = a.n_tx * a.n_ty;
     const auto launch = [&](auto kernel, int threads) {
-        pdl_launch(pdl, kernel, dim3(tiles), dim3(threads), smem_bytes, st, a);
+        pdl_launch(pdl, kernel, a.n_ty <= 65535 ? dim3(a.n_tx, a.n_ty) : dim3(tiles), dim3(threads), smem_bytes, st, a);
     };
     if (1 << a.tile_shift == TILE_SIDE_SMALL)
         launch(k_assign<T, COUNT, ASSIGN_SMALL_THREADS, TILE_SIDE_SMALL>, ASSIGN_SMALL_THREADS);

@@ -207,13 +207,13 @@ __device__ __forceinline__ int warp_scan_maps(const int *area, const int4 *box, 
 // One tile of one image (the body shared by the single-image and the batched
 // kernels), SIDE x SIDE pixels by THREADS threads.  The pixels of a candidate's
 // window that lie in the tile form a rectangle; each warp owns one or two
-// blocks of 8 x 4 pixels of the tile.
+// blocks of 8 x 4 pixels of the tile (column tx, row ty of the image's tiles).
 // PREFETCH_TILE: the tile's plane rows are first asked into L2 (for batches,
 // whose planes outgrow L2; an image whose plane stays in L2 only pays for it).
 // COUNT: the work is counted when a.count_samples asks for it (the counting
 // code costs the walks and the bound even when it is off).
 template <typename T, bool PREFETCH_TILE = false, bool COUNT = true, int THREADS = ASSIGN_THREADS, int SIDE = TILE_SIDE>
-__device__ __forceinline__ void assign_tile(const SolveArgs &a, int tile, unsigned char *smem)
+__device__ __forceinline__ void assign_tile(const SolveArgs &a, int tile, int tx, int ty, unsigned char *smem)
 {
     constexpr int PIX_PER_THREAD = SIDE * SIDE / THREADS;
     constexpr int WARPS = THREADS / 32;
@@ -221,7 +221,6 @@ __device__ __forceinline__ void assign_tile(const SolveArgs &a, int tile, unsign
     constexpr int BUILD_UNROLL = 4;  // samples per lane in flight
     const T *__restrict__ plane = reinterpret_cast<const T *>(
         sizeof(T) == 16 ? (const void *)a.plane32 : (const void *)a.plane16);
-    const int tx = tile % a.n_tx, ty = tile / a.n_tx;
     const int x0 = tx * SIDE, y0 = ty * SIDE;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 

@@ -178,7 +178,9 @@ __device__ __forceinline__ void phase_assign(const BatchArgs &b, const int *orde
     for (int g = s_tile[0]; g < total_tiles; g = s_tile[slot]) {
         if (threadIdx.x == 0) s_tile[slot ^ 1] = (int)atomicAdd(queue, 1u);
         const int j = batch_find(order_base, b.count, g);
-        assign_tile<T>(b.args[order[j]], g - order_base[j], smem);
+        const SolveArgs &a = b.args[order[j]];
+        const int tile = g - order_base[j];
+        assign_tile<T>(a, tile, tile % a.n_tx, tile / a.n_tx, smem);
         __syncthreads();  // the tile's shared memory is reused; the next index is visible
         slot ^= 1;
     }

@@ -549,20 +549,19 @@ __device__ __forceinline__ int vpath_sums(const float4 *__restrict__ plane, int 
                                           int py, int pt, int ex, int ey, int et, float cL, float ca,
                                           float cb, float &sum_dc, float &sum_w)
 {
-    const bool p_first = px < ex || (px == ex && (py < ey || (py == ey && pt <= et)));
-    const int ax = p_first ? px : ex, ay = p_first ? py : ey, at = p_first ? pt : et;
-    const int dx = (p_first ? ex : px) - ax, dy = (p_first ? ey : py) - ay, dt = (p_first ? et : pt) - at;
+    const int dx = ex - px, dy = ey - py, dt = et - pt;
+    const int first = dx ? dx : dy ? dy : dt;  // below zero: the endpoint is the smaller end
     const int adx = abs(dx), ady = abs(dy), adt = abs(dt);
-    // strides (elements) of the three axes with their signs; the major axis
-    // is the first largest |delta|.  A volume holds at most 2^30 voxels, so
-    // offsets and strides are 32-bit.
+    // strides (elements) of the three axes with their signs along the walk (x
+    // never falls); the major axis is the first largest |delta|.  A volume
+    // holds at most 2^30 voxels, so offsets and strides are 32-bit.
     const int hw = (int)HW;
-    const int sxs = dx < 0 ? -1 : 1, sys = dy < 0 ? -W : W, sts = dt < 0 ? -hw : hw;
+    const int sxs = 1, sys = (dy ^ first) < 0 ? -W : W, sts = (dt ^ first) < 0 ? -hw : hw;
     int ns, d1, d2, smaj, s1, s2;
     if (adx >= ady && adx >= adt) { ns = adx; smaj = sxs; d1 = ady; s1 = sys; d2 = adt; s2 = sts; }
     else if (ady >= adt) { ns = ady; smaj = sys; d1 = adx; s1 = sxs; d2 = adt; s2 = sts; }
     else { ns = adt; smaj = sts; d1 = adx; s1 = sxs; d2 = ady; s2 = sys; }
-    int q = at * hw + ay * W + ax;
+    int q = first < 0 ? et * hw + ey * W + ex : pt * hw + py * W + px;
     float dc = 0.f, w = 0.f;
     if (ns <= FIXED_STEP_MAX_NS) {
         // the fixed-point rule in closed form per minor axis: sample i lies at
