@@ -135,13 +135,13 @@ class Clocks:
 # Kernels per step: reload = set-up (with the grid clusters' sums), update,
 # projection, candidate lists;
 # each iteration = assignment (with the sums), update, projection, candidate
-# lists.  The lists are one kernel up to 12,287 tiles, else a scan and a fill.
+# lists.  The lists are one kernel up to 12,032 tiles, else a scan and a fill.
 FALLBACK_HBM_GBS = 6800.0
 
 
 def list_launches(H: int, W: int) -> int:
     tiles = -(-H // 32) * -(-W // 32)
-    return 1 if tiles <= 12287 else 2
+    return 1 if tiles <= 12032 else 2
 
 
 def reload_launches(H: int, W: int) -> int:

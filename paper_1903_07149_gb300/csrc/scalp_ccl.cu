@@ -13,7 +13,10 @@
 //      component takes the identity of its first non-small ancestor (or the
 //      component of pixel 0).
 //   4. The surviving components are numbered 0.. in raster order of seeds
-//      (per 4096-pixel chunk: a count, a scan of the counts, the ranks).
+//      (per 4096-pixel chunk: a count, then the ranks after the sum of the
+//      previous chunks' counts).
+// Six launches: local, border, flatten, resolve, number, out; bound on small
+// images by their latency chains, on large ones by the local unions.
 #include <algorithm>
 #include <cstdint>
 

@@ -552,7 +552,9 @@ __global__ void __launch_bounds__(SCAN1_THREADS) k_scan_tiles_batch(BatchArgs b)
 // (LISTS_MAX_TILES bounds them), CTA 0 publishes the offsets, and the CTAs
 // fill the slots grid-stride with offsets from their own copy.
 constexpr int LISTS_THREADS = 256;
-constexpr int LISTS_MAX_TILES = 12287;  // (n + 1) ints of shared memory <= 48 KB
+// (n + 1) ints of dynamic shared memory beside at most 1020 bytes of the
+// projection's static arrays: 48 KB in all, what a launch gets unasked
+constexpr int LISTS_MAX_TILES = 12032;
 
 // The scan and fill by CTA blk of nblk (blockDim.x threads); s_off holds
 // n + 1 ints of dynamic shared memory.

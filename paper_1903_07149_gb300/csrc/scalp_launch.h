@@ -92,7 +92,7 @@ void launch_debug_paths(const int *pairs, int M, int *out_xy, int stride_xy, int
 
 // Connectivity enforcement; returns the number of labels through *d_nlab.
 struct CclBuffers {
-    int *parent, *size, *link, *scan;
+    int *parent, *size, *link, *scan;  // link: at each seed, the seed of the component that takes it
     int *scan_tmp;     // block sums for the multi-level scan
     long long scan_tmp_len;
 };

@@ -476,7 +476,9 @@ __global__ void __launch_bounds__(VPROJ_THREADS) k_vproject(VoxArgs a, int whole
 // the projection.
 // ---------------------------------------------------------------------------
 constexpr int VSCAN_THREADS = 1024;
-constexpr int VLISTS_MAX_TILES = 12287;  // (n + 1) ints of shared memory <= 48 KB
+// (n + 1) ints of dynamic shared memory beside at most 1020 bytes of the
+// projection's static arrays: 48 KB in all, what a launch gets unasked
+constexpr int VLISTS_MAX_TILES = 12032;
 
 __device__ __forceinline__ void vfill_slot(const VoxArgs &a, const int *tile_off, long long i)
 {
