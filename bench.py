@@ -132,10 +132,11 @@ class Clocks:
                 "samples": len(rows)}
 
 
-# Kernels per step: reload = set-up (with the grid clusters' sums), update,
-# projection, candidate lists;
-# each iteration = assignment (with the sums), update, projection, candidate
-# lists.  The lists are one kernel up to 12,032 tiles, else a scan and a fill.
+# Kernels per step: reload = zeroing, set-up (with the grid clusters' sums),
+# update, projection, candidate lists; each iteration = assignment (with the
+# sums), update, projection and candidate lists.  The lists are one kernel up to
+# 12,032 tiles, in an iteration together with the projection; else a scan and a
+# fill.
 FALLBACK_HBM_GBS = 6800.0
 
 
@@ -145,11 +146,11 @@ def list_launches(H: int, W: int) -> int:
 
 
 def reload_launches(H: int, W: int) -> int:
-    return 3 + list_launches(H, W)
+    return 4 + list_launches(H, W)
 
 
 def iter_launches(H: int, W: int) -> int:
-    return 3 + list_launches(H, W)
+    return 3 if list_launches(H, W) == 1 else 5
 
 
 def rank_max(x: float, device: str = "cuda") -> float:
