@@ -328,7 +328,9 @@ void scalp_batch_destroy(scalp_batch *b);
  * out_stride floats (0 means W), host or device memory (out_on_device).  The
  * work runs on `stream`; with host output the call synchronises it.  The
  * workspace (device memory, 256-byte aligned, owned by the caller) must hold
- * scalp_gradient_prior_workspace_bytes(...) bytes; it stages host data.
+ * scalp_gradient_prior_workspace_bytes(...) bytes; it stages host data.  With
+ * 4 bytes more per 32 x 32 pixels (tiles, the last ones partial) the call skips
+ * clearing its running maximum; the results are the same.
  * Errors: SCALP_E_ARG for NULL pointers or bad sizes and strides,
  * SCALP_E_NOMEM for a small workspace, SCALP_E_CUDA for a failed CUDA call.
  * The same prior is used inside scalp_init when params->prior is

@@ -270,7 +270,10 @@ int stage_inputs(scalp_ctx *c, const scalp_image *img, const scalp_contour *con,
     if (c->p.prior == SCALP_PRIOR_GRADIENT) {
         // the prior computed from the image, into the contour staging area
         float *d_c = reinterpret_cast<float *>(c->ws + c->L.contour);
-        launch_gradient_prior(rgb, rs, c->H, c->W, c->a.lut, d_c, c->W, &c->a.ctr->prior_max, c->st);
+        // (the orphans' list is not in use before the first assignment)
+        launch_gradient_prior(rgb, rs, c->H, c->W, c->a.lut, d_c, c->W, &c->a.ctr->prior_max,
+                              prior_parts(c->H, c->W) ? reinterpret_cast<unsigned *>(c->a.orphan_list) : nullptr,
+                              c->st);
         rc = launch_check(c, "gradient prior");
         if (rc) return rc;
         cp = d_c;
@@ -916,7 +919,10 @@ int scalp_gradient_prior(const scalp_image *image, float *out, int64_t out_strid
     float *d_out = out_on_device ? out : reinterpret_cast<float *>(ws + o_out);
     const long long d_stride = out_on_device ? out_stride : W;
     if (e == cudaSuccess) {
-        launch_gradient_prior(rgb, rs, H, W, lut, d_out, d_stride, gmax, st);
+        // room beyond the staging takes a maximum per CTA instead of the cleared word
+        const size_t parts = prior_parts(H, W);
+        unsigned *p = parts && workspace_bytes >= need + 4 * parts ? reinterpret_cast<unsigned *>(ws + need) : nullptr;
+        launch_gradient_prior(rgb, rs, H, W, lut, d_out, d_stride, gmax, p, st);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess && !out_on_device) {

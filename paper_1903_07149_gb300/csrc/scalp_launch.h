@@ -45,9 +45,11 @@ void launch_setup(const SolveArgs &a, const uint8_t *rgb, long long rgb_stride,
 cudaError_t srgb_table(const float **table, cudaStream_t st);
 // Contour prior from the image (CIELab gradient magnitude / its maximum) into
 // out (H rows of out_stride floats); lut = the transfer-function table, gmax
-// one word of scratch.  rgb and out are device pointers.
+// one word of scratch, parts = prior_parts() words of scratch (0: not this
+// size) or NULL.  rgb and out are device pointers.
 void launch_gradient_prior(const uint8_t *rgb, long long rgb_stride, int H, int W, const float *lut,
-                           float *out, long long out_stride, unsigned *gmax, cudaStream_t st);
+                           float *out, long long out_stride, unsigned *gmax, unsigned *parts, cudaStream_t st);
+size_t prior_parts(int H, int W);
 // Cluster update (Algorithm 1) from a.acc when from_acc (queueing projections,
 // Eq. 4), then windows, the cluster records and the tile counts.  The tile
 // counts and list cursors must be zero on entry.

@@ -829,6 +829,7 @@ def gradient_prior(rgb, out=None, stream=None):
     nbytes = L.scalp_gradient_prior_workspace_bytes(H, W, 1, 1)
     if nbytes == 0:
         raise ScalpError(SCALP_E_ARG, "invalid sizes")
+    nbytes += 4 * (-(-H // 32) * -(-W // 32))  # a maximum per tile: no clearing
     ws = torch.empty(nbytes, dtype=torch.uint8, device=rgb.device)
     img = scalp_image(H, W, rgb.data_ptr(), 0, 1)
     _check(L.scalp_gradient_prior(ctypes.byref(img), out.data_ptr(), out.stride(0), 1,

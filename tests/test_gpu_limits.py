@@ -85,6 +85,29 @@ def test_prior_output_alignment(S, H, W, offset, pad):
     assert np.all(got == -1.0)
 
 
+# one maximum per tile of 32 x 32 up to 8,192 tiles and where the workspace has
+# the room, else a cleared word: the same bits (2,041 and 257 words a CTA and
+# less than one each; one tile over the limit)
+@pytest.mark.parametrize("H,W", [(1, 1), (65, 130), (512, 514), (1080, 1921), (2048, 4096), (2048, 4097)])
+def test_prior_maximum_forms(S, H, W):
+    import ctypes
+
+    import torch
+
+    gen = torch.Generator(device="cuda").manual_seed(W)
+    rgb = torch.randint(0, 256, (H, W, 3), generator=gen, dtype=torch.uint8, device="cuda")
+    a = S.gradient_prior(rgb)
+    L = S.load()
+    nbytes = L.scalp_gradient_prior_workspace_bytes(H, W, 1, 1)
+    ws = torch.empty(nbytes, dtype=torch.uint8, device="cuda")
+    b = torch.empty((H, W), device="cuda")
+    img = S.scalp_image(H, W, rgb.data_ptr(), 0, 1)
+    rc = L.scalp_gradient_prior(ctypes.byref(img), b.data_ptr(), W, 1, torch.cuda.current_stream().cuda_stream,
+                                ws.data_ptr(), nbytes)
+    assert rc == S.SCALP_OK and torch.equal(a, b)
+    assert float(a.max()) == (1.0 if H * W > 1 else 0.0)
+
+
 # the same limit in two dimensions, against a batch of one (lists of their own):
 # 128 x 94, 191 x 63, 1117 x 11 (12,287, which once did not launch) tiles
 @pytest.mark.parametrize("H,W", [(4096, 3008), (6112, 2016), (352, 35744)])
