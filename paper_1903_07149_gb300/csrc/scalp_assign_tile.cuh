@@ -8,6 +8,7 @@
 #include <climits>
 
 #include "scalp_internal.cuh"
+#include "scalp_offsets.h"
 
 namespace scalp {
 
@@ -218,7 +219,7 @@ __device__ __forceinline__ void assign_tile(const SolveArgs &a, int tile, int tx
     constexpr int PIX_PER_THREAD = SIDE * SIDE / THREADS;
     constexpr int WARPS = THREADS / 32;
     constexpr int QUEUE = assign_queues(SIDE) / WARPS;  // pairs a warp's queue holds
-    constexpr int BUILD_UNROLL = 4;  // samples per lane in flight
+    constexpr int BUILD_UNROLL = STRIP_ROWS;  // samples per lane in flight
     const T *__restrict__ plane = reinterpret_cast<const T *>(
         sizeof(T) == 16 ? (const void *)a.plane32 : (const void *)a.plane16);
     const int x0 = tx * SIDE, y0 = ty * SIDE;
@@ -426,26 +427,21 @@ __device__ __forceinline__ void assign_tile(const SolveArgs &a, int tile, int tx
             const float4 ck = col[c];
             const int bw = b.w & 0xffff, bh = (int)((unsigned)b.w >> 16);
             const int cx = (g - cfirst[c]) * BUILD_STRIP + lcol;
-            // the box's first pixel; offsets within the box fit 32 bits: a
-            // box of at most map_cap pairs has row < min(H, map_cap / 4) and
-            // the plane pitch is at most W + 3, so row * pitch + column < 2^31
+            // the box's first pixel
             const T *__restrict__ pbox = plane + (long long)b.y * a.pitch + b.x;
-            const int cc = min(cx, bw - 1), last = (bh - 1) * a.pitch + cc, step = 4 * a.pitch;
-            int off = lrow * a.pitch + cc;
-            // (entries of columns past the box are not stored: limit < off)
-            const int limit = cx < bw ? last : -1;
+            StripPlaces at = strip_places(lrow, bh, a.pitch, bw, cx);
             float2 *m = maps + (mfirst[c] + lrow * b.z + cx);
             const int mstep = 4 * b.z;
             for (int r = 0; r < bh; r += 4 * BUILD_UNROLL) {
                 T v[BUILD_UNROLL];  // raw samples: all loads issue before any use
 #pragma unroll
-                for (int u = 0; u < BUILD_UNROLL; ++u) v[u] = __ldg(pbox + min(off + u * step, last));
+                for (int u = 0; u < BUILD_UNROLL; ++u) v[u] = __ldg(pbox + min(at.off + u * at.step, at.last));
 #pragma unroll
                 for (int u = 0; u < BUILD_UNROLL; ++u) {
                     const float4 q = sample_value(v[u]);
                     const float2 pair = make_float2(colour_dist(q, ck.x, ck.y, ck.z), q.w);
-                    if (off <= limit) *m = pair;
-                    off += step;
+                    if (at.off < (u == 0 ? at.end : at.more)) *m = pair;
+                    at.off += at.step;
                     m += mstep;
                 }
             }
