@@ -516,7 +516,13 @@ __global__ void __launch_bounds__(PROJ_THREADS) k_project(SolveArgs a, int whole
 // PROJ_CTAS_PER_IMAGE CTAs per image, each cluster searched by a whole CTA.
 constexpr int PROJ_CTAS_PER_IMAGE = 16;
 constexpr int PROJ_LIST_MIN_IMAGES = 32;
-constexpr int PROJ_LIST_MAX_IMAGES = 3071;  // (4 * count + 2) ints <= 48 KB
+// (4 * count + 2) ints of dynamic shared memory beside at most 1 KB of the
+// projection's static arrays: 48 KB in all, what a launch gets unasked
+constexpr int PROJ_STATIC_SMEM = 1024;
+constexpr int PROJ_LIST_MAX_IMAGES = ((48 * 1024 - PROJ_STATIC_SMEM) / 4 - 2) / 4;
+static_assert(PROJ_LIST_MAX_IMAGES == 3007, "as tested");
+static_assert(PROJ_THREADS / 32 * (sizeof(ProjBest) + sizeof(int)) + 32 * sizeof(int) <= PROJ_STATIC_SMEM,
+              "project_cta()'s arrays and the scan's");
 
 __global__ void __launch_bounds__(PROJ_THREADS) k_project_batch_images(BatchArgs b, int whole_image)
 {
