@@ -423,7 +423,9 @@ __device__ __forceinline__ void project_scan(const SolveArgs &a, int k, long lon
     const RowDiv div(w, area);
     if (div.fast && small) {
         const unsigned end = (unsigned)area;  // (area * w < 2^32)
-        const int *__restrict__ corner = a.labels + (long long)ylo * a.W + xlo;
+        // (not __restrict__: the persistent kernel writes the labels between its
+        // barriers, so no load of theirs may take the read-only path)
+        const int *corner = a.labels + (long long)ylo * a.W + xlo;
         for (unsigned base = (unsigned)t; base < end; base += (unsigned)(threads * BATCH)) {
             unsigned match = 0u;
             int lab[BATCH];
