@@ -8,7 +8,6 @@
 #include <climits>
 
 #include "scalp_internal.cuh"
-#include "scalp_offsets.h"
 
 namespace scalp {
 

@@ -7,6 +7,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "scalp_offsets.h"
+
 namespace scalp {
 
 // Assignment tile: a CTA labels TILE_SIDE x TILE_SIDE pixels, or for a single
@@ -190,25 +192,6 @@ __device__ __forceinline__ void cta_scan(const int *in, int *out, int n, int thr
     if (threadIdx.x == 0) out[n] = s_warp[31];
     __syncthreads();
 }
-
-// Row of index i in rows of w pixels: i / w by a 32-bit reciprocal
-// (rcp = ceil(2^32 / w), exact while i * w < 2^32; the caller checks), else by
-// a 64-bit division.
-struct RowDiv {
-    long long w;
-    unsigned rcp;
-    bool fast;
-    __device__ __forceinline__ RowDiv(long long w_, long long area) : w(w_)
-    {
-        fast = w_ > 1 && (unsigned long long)area * (unsigned long long)w_ < (1ULL << 32);
-        rcp = fast ? (unsigned)((0x100000000ULL + w_ - 1) / w_) : 0u;
-    }
-    __device__ __forceinline__ long long row(long long i) const
-    {
-        if (w == 1) return i;
-        return fast ? (long long)__umulhi((unsigned)i, rcp) : i / w;
-    }
-};
 
 // The start of an exact window search, floor(s/n - r) - 1 and ceil(s/n + r)
 // + 1 for a coordinate in [0, lim): the searches then move inward with the

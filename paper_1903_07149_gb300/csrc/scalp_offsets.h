@@ -45,4 +45,25 @@ SCALP_HD StripPlaces strip_places(int lrow, int rows, int pitch, int width, int 
     return s;
 }
 
+// Division of i < 2^30 by d >= 1 through rcp = ceil(2^32 / d): i * rcp / 2^32
+// exceeds i / d by less than i / 2^32 < 1/4, so its floor is the quotient or
+// one more, and then the remainder is negative.  For all i <= end with end * d
+// < 2^32 (and d > 1) the excess is below 1 / d and the floor is the quotient:
+// EXACT leaves the correction out.
+struct Divisor {
+    unsigned d, rcp;
+
+    SCALP_HD explicit Divisor(unsigned d_) : d(d_), rcp(d_ > 1u ? 0xffffffffu / d_ + 1u : 0u) {}
+    SCALP_HD bool exact(unsigned end) const { return d > 1u && (unsigned long long)end * d < (1ull << 32); }
+    template <bool EXACT>
+    SCALP_HD void split(unsigned i, int &quotient, int &remainder) const
+    {
+        const unsigned q = EXACT || rcp ? (unsigned)((unsigned long long)i * rcp >> 32) : i;
+        const int r = (int)(i - q * d);
+        const bool over = !EXACT && r < 0;
+        quotient = (int)q - (over ? 1 : 0);
+        remainder = over ? r + (int)d : r;
+    }
+};
+
 }  // namespace scalp

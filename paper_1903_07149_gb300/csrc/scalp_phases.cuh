@@ -408,54 +408,54 @@ __device__ __forceinline__ bool proj_small(const SolveArgs &a, long long n)
     return 2.0 * (n * bound) * (n * bound) < 4.0e18;
 }
 
-// All pixels of columns xlo .. xlo + w - 1 from row ylo, `area` of them, for
-// cluster k by `threads` threads, of which this is thread t.  Where the rows
-// come from an exact 32-bit reciprocal (RowDiv) and 64 bits hold the squared
-// distances, BATCH label loads are issued before any is compared; the matches,
-// seldom more than a few, are then taken one by one.  (The kernels are short
-// and their code is cold on every launch: distances written out for each load
-// of the batch cost more in instruction fetches than they saved.)
-template <int BATCH>
-__device__ __forceinline__ void project_scan(const SolveArgs &a, int k, long long n, long long sx, long long sy,
-                                             bool small, int xlo, int ylo, int w, long long area, int t, int threads,
-                                             ProjBest &b)
+// The `end` pixels of rows of div.d pixels from (xlo, ylo) for cluster k by
+// `threads` threads, of which this is thread t.  BATCH label loads are issued
+// before any is compared; the matches, seldom more than a few, are then taken
+// one by one.  (The kernels are short and their code is cold on every launch:
+// distances written out for each load of the batch cost more in instruction
+// fetches than they saved.)
+template <int BATCH, bool EXACT>
+__device__ __forceinline__ void project_scan_rows(const SolveArgs &a, int k, long long n, long long sx, long long sy,
+                                                  bool small, int xlo, int ylo, Divisor div, unsigned end, int t,
+                                                  int threads, ProjBest &b)
 {
-    const RowDiv div(w, area);
-    if (div.fast && small) {
-        const unsigned end = (unsigned)area;  // (area * w < 2^32)
-        // (not __restrict__: the persistent kernel writes the labels between its
-        // barriers, so no load of theirs may take the read-only path)
-        const int *corner = a.labels + (long long)ylo * a.W + xlo;
-        for (unsigned base = (unsigned)t; base < end; base += (unsigned)(threads * BATCH)) {
-            unsigned match = 0u;
-            int lab[BATCH];
+    // (not __restrict__: the persistent kernel writes the labels between its
+    // barriers, so no load of theirs may take the read-only path)
+    const int *corner = a.labels + (long long)ylo * a.W + xlo;
+    for (unsigned base = (unsigned)t; base < end; base += (unsigned)(threads * BATCH)) {
+        unsigned match = 0u;
+        int lab[BATCH], row, col;
 #pragma unroll
-            for (int u = 0; u < BATCH; ++u) {
-                // (past the end: the last pixel, which changes nothing)
-                const unsigned i = min(base + (unsigned)(u * threads), end - 1u);
-                const int row = (int)__umulhi(i, div.rcp);
-                lab[u] = corner[row * a.W + (int)(i - (unsigned)(row * w))];
-            }
-#pragma unroll
-            for (int u = 0; u < BATCH; ++u) match |= lab[u] == k ? 1u << u : 0u;
-            for (; match; match &= match - 1) {
-                const unsigned i = min(base + (unsigned)((__ffs(match) - 1) * threads), end - 1u);
-                const int row = (int)__umulhi(i, div.rcp), x = xlo + (int)(i - (unsigned)(row * w)), y = ylo + row;
-                const ProjBest c = proj_candidate((long long)y * a.W + x, x, y, n, sx, sy, true);
-                if (proj_less(c, b)) b = c;
-            }
+        for (int u = 0; u < BATCH; ++u) {
+            // (past the end: the last pixel, which changes nothing)
+            div.split<EXACT>(min(base + (unsigned)(u * threads), end - 1u), row, col);
+            lab[u] = corner[row * a.W + col];
         }
-    } else {
-#pragma unroll 1
-        for (long long i = t; i < area; i += threads) {
-            const long long row = div.row(i);
-            const int x = xlo + (int)(i - row * w), y = ylo + (int)row;
-            const long long p = (long long)y * a.W + x;
-            if (a.labels[p] != k) continue;
-            const ProjBest c = proj_candidate(p, x, y, n, sx, sy, small);
+#pragma unroll
+        for (int u = 0; u < BATCH; ++u) match |= lab[u] == k ? 1u << u : 0u;
+        for (; match; match &= match - 1) {
+            div.split<EXACT>(min(base + (unsigned)((__ffs(match) - 1) * threads), end - 1u), row, col);
+            const int x = xlo + col, y = ylo + row;
+            const ProjBest c = proj_candidate((long long)y * a.W + x, x, y, n, sx, sy, EXACT || small);
             if (proj_less(c, b)) b = c;
         }
     }
+}
+
+// The w x h pixels from (xlo, ylo).  Windows below 1,626 x 1,626 divide
+// exactly and their clusters have 64-bit squared distances; larger ones and
+// those of large clusters take the general form, with as many loads in flight
+// (one at a time, solves of 2160 x 3840 with 12 clusters took 34.8 ms per two
+// iterations against 31.4).
+template <int BATCH>
+__device__ __forceinline__ void project_scan(const SolveArgs &a, int k, long long n, long long sx, long long sy,
+                                             bool small, int xlo, int ylo, int w, int h, int t, int threads,
+                                             ProjBest &b)
+{
+    const Divisor div((unsigned)max(w, 1));
+    const unsigned end = (unsigned)(max(w, 0) * max(h, 0));  // (within the image: at most 2^30)
+    if (small && div.exact(end)) project_scan_rows<BATCH, true>(a, k, n, sx, sy, small, xlo, ylo, div, end, t, threads, b);
+    else project_scan_rows<BATCH, false>(a, k, n, sx, sy, small, xlo, ylo, div, end, t, threads, b);
 }
 
 // Eq. 4 for queued cluster j of one image by one warp: the same argmin, with
@@ -469,8 +469,7 @@ __device__ __forceinline__ void project_warp(const SolveArgs &a, int j)
     const bool small = proj_small(a, n);
     ProjBest b = {~0ull, ~0ull, LLONG_MAX};
     if (!small || !project_near(a, k, n, sx, sy, w4, b)) {
-        const int w = w4.y - w4.x + 1;
-        project_scan<4>(a, k, n, sx, sy, small, w4.x, w4.z, w, (long long)w * (w4.w - w4.z + 1), lane, 32, b);
+        project_scan<4>(a, k, n, sx, sy, small, w4.x, w4.z, w4.y - w4.x + 1, w4.w - w4.z + 1, lane, 32, b);
     }
     project_orphans(a, k, n, sx, sy, small, lane, 32, b);
     proj_shfl_min(b);
@@ -522,11 +521,10 @@ __device__ __forceinline__ void project_cta(const SolveArgs &a, int whole_image,
                 const int4 w4 = a.prev_win[k];
                 xlo = w4.x; xhi = w4.y; ylo = w4.z; yhi = w4.w;
             }
-            const int w = xhi - xlo + 1;
-            const long long area = (long long)w * (yhi - ylo + 1);
             const bool small = proj_small(a, n);
             ProjBest b = {~0ull, ~0ull, LLONG_MAX};
-            project_scan<PROJ_BATCH>(a, k, n, sx, sy, small, xlo, ylo, w, area, tid, PROJ_THREADS, b);
+            project_scan<PROJ_BATCH>(a, k, n, sx, sy, small, xlo, ylo, xhi - xlo + 1, yhi - ylo + 1, tid, PROJ_THREADS,
+                                     b);
             if (!whole_image) project_orphans(a, k, n, sx, sy, small, tid, PROJ_THREADS, b);
             proj_shfl_min(b);
             if (lane == 0) s_best[warp] = b;

@@ -357,54 +357,55 @@ __device__ __forceinline__ void vshfl_min(VBest &b)
     }
 }
 
-// The voxels of one box for cluster k, thread t of `threads`: eight label loads
-// before any is compared where the box's rows and frames come from exact 32-bit
-// reciprocals and 64 bits hold the squared distances; the matches one by one
-// (compact code: it is cold on every launch).
-__device__ __forceinline__ void vproject_scan(const VoxArgs &a, int k, long long n, long long sx, long long sy,
-                                              long long st, bool small, int xlo, int ylo, int tlo, long long w,
-                                              long long h, long long vol, int t, int threads, VBest &b)
+// The `end` voxels of rows of div_w.d and frames of div_h.d rows from (xlo, ylo,
+// tlo) for cluster k, thread t of `threads`: eight label loads before any is
+// compared, then the matches one by one (compact code: it is cold on every
+// launch).
+template <bool EXACT>
+__device__ __forceinline__ void vproject_scan_rows(const VoxArgs &a, int k, long long n, long long sx, long long sy,
+                                                   long long st, bool small, int xlo, int ylo, int tlo, Divisor div_w,
+                                                   Divisor div_h, unsigned end, int t, int threads, VBest &b)
 {
     constexpr int VB = 8;
-    // voxel i of the box: row i / w, frame row / h
-    const RowDiv div_w(w, vol), div_h(h, w > 0 ? vol / w : 0);
-    if (div_w.fast && (div_h.fast || h == 1) && small) {
-        const unsigned end = (unsigned)vol;  // (vol * w < 2^32)
-        const auto place = [&](unsigned i, int &x, int &y, int &z) {
-            const unsigned row = __umulhi(i, div_w.rcp), fr = h == 1 ? row : __umulhi(row, div_h.rcp);
-            x = xlo + (int)(i - row * (unsigned)w);
-            y = ylo + (int)(row - fr * (unsigned)h);
-            z = tlo + (int)fr;
-        };
-        for (unsigned base = (unsigned)t; base < end; base += (unsigned)(threads * VB)) {
-            unsigned match = 0u;
-            int lab[VB];
+    const auto place = [&](unsigned i, int &x, int &y, int &z) {
+        int row;
+        div_w.split<EXACT>(min(i, end - 1u), row, x);  // (past the end: the last voxel, which changes nothing)
+        div_h.split<EXACT>((unsigned)row, z, y);
+        x += xlo;
+        y += ylo;
+        z += tlo;
+    };
+    for (unsigned base = (unsigned)t; base < end; base += (unsigned)(threads * VB)) {
+        unsigned match = 0u;
+        int lab[VB], x, y, z;
 #pragma unroll
-            for (int u = 0; u < VB; ++u) {  // (past the end: the last voxel, which changes nothing)
-                int x, y, z;
-                place(min(base + (unsigned)(u * threads), end - 1u), x, y, z);
-                lab[u] = a.labels[((long long)z * a.H + y) * a.W + x];
-            }
-#pragma unroll
-            for (int u = 0; u < VB; ++u) match |= lab[u] == k ? 1u << u : 0u;
-            for (; match; match &= match - 1) {
-                int x, y, z;
-                place(min(base + (unsigned)((__ffs(match) - 1) * threads), end - 1u), x, y, z);
-                const VBest c = vcandidate(((long long)z * a.H + y) * a.W + x, x, y, z, n, sx, sy, st, true);
-                if (vless(c, b)) b = c;
-            }
+        for (int u = 0; u < VB; ++u) {
+            place(base + (unsigned)(u * threads), x, y, z);
+            lab[u] = a.labels[((long long)z * a.H + y) * a.W + x];
         }
-    } else {
-#pragma unroll 1
-        for (long long i = t; i < vol; i += threads) {
-            const long long row = div_w.row(i), fr = div_h.row(row);
-            const int x = xlo + (int)(i - row * w), y = ylo + (int)(row - fr * h), z = tlo + (int)fr;
-            const long long p = ((long long)z * a.H + y) * a.W + x;
-            if (a.labels[p] != k) continue;
-            const VBest c = vcandidate(p, x, y, z, n, sx, sy, st, small);
+#pragma unroll
+        for (int u = 0; u < VB; ++u) match |= lab[u] == k ? 1u << u : 0u;
+        for (; match; match &= match - 1) {
+            place(base + (unsigned)((__ffs(match) - 1) * threads), x, y, z);
+            const VBest c =
+                vcandidate(((long long)z * a.H + y) * a.W + x, x, y, z, n, sx, sy, st, EXACT || small);
             if (vless(c, b)) b = c;
         }
     }
+}
+
+// The w x h x d voxels from (xlo, ylo, tlo); the two forms as in 2-D.
+__device__ __forceinline__ void vproject_scan(const VoxArgs &a, int k, long long n, long long sx, long long sy,
+                                              long long st, bool small, int xlo, int ylo, int tlo, int w, int h,
+                                              int d, int t, int threads, VBest &b)
+{
+    const Divisor div_w((unsigned)max(w, 1)), div_h((unsigned)max(h, 1));
+    const unsigned rows = (unsigned)(max(h, 0) * max(d, 0));
+    const unsigned end = (unsigned)max(w, 0) * rows;  // (within the volume: at most 2^30)
+    if (small && div_w.exact(end) && div_h.exact(rows))
+        vproject_scan_rows<true>(a, k, n, sx, sy, st, small, xlo, ylo, tlo, div_w, div_h, end, t, threads, b);
+    else
+        vproject_scan_rows<false>(a, k, n, sx, sy, st, small, xlo, ylo, tlo, div_w, div_h, end, t, threads, b);
 }
 
 // Queue entries j0, j0 + stride, ...: one CTA per queued cluster.
@@ -422,13 +423,12 @@ __device__ __forceinline__ void vproject_cta(const VoxArgs &a, int whole, int j0
             const int *pw = a.prev_win + 6 * (long long)k;
             xlo = pw[0]; xhi = pw[1]; ylo = pw[2]; yhi = pw[3]; tlo = pw[4]; thi = pw[5];
         }
-        const long long w = xhi - xlo + 1, h = yhi - ylo + 1;
-        const long long vol = max(0LL, w) * max(0LL, h) * max(0LL, (long long)(thi - tlo + 1));
         // 64-bit squared distances when 3 (n * largest dimension)^2 < 2^62
         const double bound = (double)max(a.W, max(a.H, a.T));
         const bool small = 3.0 * ((double)n * bound) * ((double)n * bound) < 4.0e18;
         VBest b = {~0ull, ~0ull, LLONG_MAX};
-        vproject_scan(a, k, n, sx, sy, st, small, xlo, ylo, tlo, w, h, vol, tid, VPROJ_THREADS, b);
+        vproject_scan(a, k, n, sx, sy, st, small, xlo, ylo, tlo, xhi - xlo + 1, yhi - ylo + 1, thi - tlo + 1, tid,
+                      VPROJ_THREADS, b);
         for (int i = tid; i < n_orphans; i += VPROJ_THREADS) {
             const int p = a.orphan_list[i];
             if (a.labels[p] != k) continue;

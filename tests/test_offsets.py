@@ -1,11 +1,13 @@
-"""Places on the plane that the distance maps' build reads, at the limits of
-the accepted sizes (H * W <= 2^30): few rows and a pitch of up to 2^30.  A warp
-covers rows past the box's last one; the places formed for them stay inside the
-box.  The header that the kernels include is compiled for the host."""
+"""Index arithmetic of the kernels at the limits of the accepted sizes (H * W <=
+2^30), from the header that they include, compiled for the host.  Places on the
+plane that the distance maps' build reads: a warp covers rows past the box's
+last one; the places formed for them stay inside the box.  Rows and columns of
+the projections' windows: the divisions by a reciprocal are exact."""
 import ctypes
 import os
 import subprocess
 
+import numpy as np
 import pytest
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
@@ -21,6 +23,12 @@ def lib(tmp_path_factory):
                    'extern "C" void places(int lrow, int rows, int pitch, int width, int col, unsigned *o)\n'
                    "{ const scalp::StripPlaces s = scalp::strip_places(lrow, rows, pitch, width, col);\n"
                    "  o[0] = s.off; o[1] = s.step; o[2] = s.last; o[3] = s.end; o[4] = s.more; }\n")
+    src.write_text(src.read_text() +
+                   'extern "C" int exact(unsigned d, unsigned end) { return scalp::Divisor(d).exact(end); }\n'
+                   'extern "C" void split(unsigned d, int ex, const unsigned *i, int n, int *q, int *r)\n'
+                   "{ const scalp::Divisor v(d);\n"
+                   "  for (int j = 0; j < n; ++j) {\n"
+                   "    if (ex) v.split<true>(i[j], q[j], r[j]); else v.split<false>(i[j], q[j], r[j]); } }\n")
     subprocess.run(["g++", "-O1", "-shared", "-fPIC", "-o", str(so), str(src)], check=True)
     return ctypes.CDLL(str(so))
 
@@ -54,6 +62,29 @@ def test_places_stay_in_the_box(lib, H):
                         place += step
                     assert place < 1 << 32
                     assert stored == ({row: row * pitch + c for row in range(lrow, rows, 4)} if col < width else {})
+
+
+def test_divisions_are_exact(lib):
+    rng = np.random.default_rng(11)
+    widths = list(range(1, 70)) + [481, 1080, 1625, 1626, 1920, 3840, 4096, 32767, 32768, 32769, 65535, 65536, 65537,
+                                   LIMIT // 3, LIMIT // 2, LIMIT - 1, LIMIT]
+    widths += [int(2 ** v) for v in rng.uniform(6, 30, 300)]
+    forms = set()
+    for d in widths:
+        for end in (d, min(LIMIT, 1625 * d), min(LIMIT, max(1, ((1 << 32) - 1) // d)), LIMIT // d * d):
+            ex = lib.exact(d, ctypes.c_uint(end))
+            assert bool(ex) == (d > 1 and end * d < 1 << 32)
+            q0 = rng.integers(0, max(1, end // d), 40)
+            i = np.concatenate([np.arange(0, min(end, 20)), rng.integers(0, end, 60), end - 1 - np.arange(min(end, 20)),
+                                q0 * d, q0 * d + d - 1, np.maximum(q0 * d - 1, 0)]).astype(np.int64)
+            i = np.ascontiguousarray(i[i < end], np.uint32)
+            for form in {0, ex}:
+                q, r = np.empty(i.size, np.int32), np.empty(i.size, np.int32)
+                lib.split(d, form, ctypes.c_void_p(i.ctypes.data), i.size, ctypes.c_void_p(q.ctypes.data),
+                          ctypes.c_void_p(r.ctypes.data))
+                assert np.array_equal(q, i // d) and np.array_equal(r, i % d), (d, end, form)
+                forms.add(form)
+    assert forms == {0, 1}
 
 
 # Thin images whose pitch times the rows of a warp's batch leaves 32 bits
