@@ -564,7 +564,7 @@ __global__ void __launch_bounds__(PROJ_THREADS) k_project_batch(BatchArgs b, int
         for (int i = threadIdx.x; i < count; i += blockDim.x) {
             const SolveArgs &a = b.args[i];
             const float side = 2.0f * (float)a.r + 1.0f;  // window side
-            const bool cta = whole_image || a.ctr->proj_orphans > PROJ_WARP_ORPHANS || side * side > PROJ_WARP_MAX_AREA;
+            const bool cta = whole_image || !proj_by_warp(a) || side * side > PROJ_WARP_MAX_AREA;
             s_nw[i] = cta ? 0 : s_nc[i];
             s_nc[i] = cta ? s_nc[i] : 0;
         }

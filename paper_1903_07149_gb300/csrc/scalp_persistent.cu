@@ -138,7 +138,7 @@ __device__ __noinline__ void phase_project(const BatchArgs &b, unsigned char *sm
     int *s_cnt = reinterpret_cast<int *>(smem);  // per image: queue length, 0 with many orphans
     int *s_pref = s_cnt + count;                 // count + 1: its prefix
     for (int i = threadIdx.x; i < count; i += blockDim.x)
-        s_cnt[i] = b.args[i].ctr->proj_orphans > PROJ_WARP_ORPHANS ? 0 : b.args[i].ctr->nproj;
+        s_cnt[i] = proj_by_warp(b.args[i]) ? b.args[i].ctr->nproj : 0;
     __syncthreads();
     cta_scan(s_cnt, s_pref, count, ASSIGN_THREADS, s_warp);
     const int total = s_pref[count];
@@ -149,7 +149,7 @@ __device__ __noinline__ void phase_project(const BatchArgs &b, unsigned char *sm
     }
     // images with many orphans: image by image, entry j on CTA (j mod G)
     for (int i = 0; i < count; ++i) {
-        if (s_cnt[i] != 0 || b.args[i].ctr->proj_orphans <= PROJ_WARP_ORPHANS) continue;
+        if (s_cnt[i] != 0 || proj_by_warp(b.args[i])) continue;
         const int nproj = b.args[i].ctr->nproj;
         for (int j = blockIdx.x; j < nproj; j += G) project_by_cta(b.args[i], j);
     }

@@ -325,8 +325,19 @@ static_assert(offsetof(ClusterDev, xk) == 12 && offsetof(ClusterDev, yk) == 16 &
 // assignment lists those (there are seldom more than a few, but one was
 // enough to make every search take the whole image: 0.8 ms more per HD solve
 // for such inputs, 3.7 ms for the 32 x 240 x 320 video), and the searches go
-// through the window and the list.  Larger lists are left to whole CTAs.
-constexpr int PROJ_WARP_ORPHANS = 1024;
+// through the window and the list.  One warp alone is long about many: lists
+// of more than N / 128 pixels, or 1,024, are left to whole CTAs, and above N / 4
+// the image's rows in order are quicker than the list's scattered places.  One
+// iteration of 1080 x 1920 with 2000 clusters and 3, 12, 25 and 90% of the
+// columns in no window: 560, 1068, 1620, 1545 us; warps first, whatever the
+// list, and never the whole image: 1615, 3915, 8516, 23648; the whole image
+// from N / 16: 560, 1584, 1620, 1545; from N / 2: 560, 1073, 1830, 1545.
+constexpr int PROJ_WARP_ORPHANS = 1024, PROJ_WARP_SHIFT = 7, PROJ_LIST_SHIFT = 2;
+__device__ __forceinline__ bool proj_by_warp(const SolveArgs &a)
+{
+    const int orphans = a.ctr->proj_orphans;
+    return orphans <= PROJ_WARP_ORPHANS && orphans <= a.N >> PROJ_WARP_SHIFT;
+}
 
 // The listed orphans' candidates for cluster k; thread t of `threads`.
 __device__ __forceinline__ void project_orphans(const SolveArgs &a, int k, long long n, long long sx, long long sy,
@@ -477,8 +488,8 @@ __device__ __forceinline__ void project_warp(const SolveArgs &a, int j)
 }
 
 // Queued projections over the window and the orphans (with whole_image, at
-// set-up, the whole image).  Queue entries j0, j0 + stride, ... of one image.
-// Each warp first looks near the endpoint of one (as many at a time as the CTA
+// set-up, or very many orphans the whole image).  Queue entries j0, j0 + stride,
+// ... of one image.  Each warp first looks near the endpoint of one (as many at a time as the CTA
 // has warps), and only what it cannot settle there the whole CTA searches,
 // cluster by cluster.  Per launch, against a CTA per cluster over its whole
 // window: HD 10.7 -> 9.5 us, UHD 20.6 -> 13.1.
@@ -489,7 +500,8 @@ __device__ __forceinline__ void project_cta(const SolveArgs &a, int whole_image,
     __shared__ int s_left[WARPS];  // per warp: the cluster left to the CTA, or -1
     const int nproj = a.ctr->nproj;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const bool look = !whole_image;
+    const bool look = !whole_image && proj_by_warp(a);
+    const bool whole = whole_image || a.ctr->proj_orphans > a.N >> PROJ_LIST_SHIFT;
     for (long long first = j0; first < nproj; first += (long long)stride * WARPS) {
         if (look) {
             const long long j = first + (long long)stride * warp;
@@ -517,7 +529,7 @@ __device__ __forceinline__ void project_cta(const SolveArgs &a, int whole_image,
             if (k < 0) continue;
             const long long n = a.st_n[k], sx = a.st_sx[k], sy = a.st_sy[k];
             int xlo = 0, xhi = a.W - 1, ylo = 0, yhi = a.H - 1;
-            if (!whole_image) {
+            if (!whole) {
                 const int4 w4 = a.prev_win[k];
                 xlo = w4.x; xhi = w4.y; ylo = w4.z; yhi = w4.w;
             }
@@ -525,7 +537,7 @@ __device__ __forceinline__ void project_cta(const SolveArgs &a, int whole_image,
             ProjBest b = {~0ull, ~0ull, LLONG_MAX};
             project_scan<PROJ_BATCH>(a, k, n, sx, sy, small, xlo, ylo, xhi - xlo + 1, yhi - ylo + 1, tid, PROJ_THREADS,
                                      b);
-            if (!whole_image) project_orphans(a, k, n, sx, sy, small, tid, PROJ_THREADS, b);
+            if (!whole) project_orphans(a, k, n, sx, sy, small, tid, PROJ_THREADS, b);
             proj_shfl_min(b);
             if (lane == 0) s_best[warp] = b;
             __syncthreads();

@@ -408,11 +408,18 @@ __device__ __forceinline__ void vproject_scan(const VoxArgs &a, int k, long long
         vproject_scan_rows<false>(a, k, n, sx, sy, st, small, xlo, ylo, tlo, div_w, div_h, end, t, threads, b);
 }
 
-// Queue entries j0, j0 + stride, ...: one CTA per queued cluster.
+// Queue entries j0, j0 + stride, ...: one CTA per queued cluster.  A list of more
+// than half the voxels is slower than the volume in order (32 x 240 x 320 with
+// 2000 clusters, an iteration with 25, 50 and 90% of the columns in no window:
+// 3.19, 4.96 and 5.33 ms; by the list 3.30, 6.51 and 11.31; the volume from
+// a quarter on 4.51, 4.99 and 5.34).
+constexpr int VPROJ_LIST_SHIFT = 1;
+
 __device__ __forceinline__ void vproject_cta(const VoxArgs &a, int whole, int j0, int stride)
 {
     __shared__ VBest s_best[VPROJ_THREADS / 32];
     const int nproj = a.ctr->nproj;
+    whole |= a.ctr->proj_orphans > a.N >> VPROJ_LIST_SHIFT;
     const int n_orphans = whole ? 0 : a.ctr->proj_orphans;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     for (int j = j0; j < nproj; j += stride) {
