@@ -198,14 +198,6 @@ void launch_assign_batch(const BatchArgs &b, int storage, bool count, int total_
     }
 }
 
-// Whether the pruning bound's error estimate holds (scalp_assign_tile.cuh):
-// coordinates exact in FP32, and lam and m^2/r^2 far enough from both ends of
-// the FP32 range that no product under- or overflows where D would not.
-bool bound_valid(int H, int W, float lam, float ms2)
-{
-    return std::max(H, W) <= (1 << 24) && ms2 >= 1e-12f && ms2 <= 1e12f && (lam == 0.0f || lam >= 1e-12f);
-}
-
 // The limit is a property of the kernel, shared by every context on the
 // device: it is always set to the largest map buffer, which covers any launch.
 static cudaError_t configure(const void *f, int side)

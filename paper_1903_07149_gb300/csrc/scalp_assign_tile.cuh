@@ -142,11 +142,15 @@ __device__ __forceinline__ int find_slot(const int *cid, int cnt, int k)
 // as |f . g| <= P + K, so P' + K' + f . g stays below q - 98 u (P + K); the
 // computed D is above q - 20 u (P + K) (at most ten roundings).  A pair whose
 // bound exceeds the pixel's pass-1 D raised by 2^-20 (bound_threshold()
-// subtracts P') therefore has a larger D: it can neither win nor tie.  The
-// host turns the pruning off where these estimates do not hold (bound_valid()
-// in scalp_assign.cu: products that could leave the FP32 range, coordinates
-// above 2^24).  BOUND_SCALE and bound_threshold() are in scalp_internal.cuh
-// (the supervoxels use them too).
+// subtracts P') therefore has a larger D: it can neither win nor tie.
+// That holds for every accepted weight, and for sides up to 2^24, whose places
+// FP32 holds exactly (the host turns the pruning off above):
+//   * Products below the normal range err by 2^-150 each, at most twenty of
+//     them, times places and samples below 2^7: D is raised by 2^-100 as well.
+//   * P or D above 1e30 prunes nothing.  K then overflows only where q does not
+//     stay below 1e30 (|f . g| <= 2 sqrt(P K)), and a NaN prunes nothing.
+// BOUND_SCALE and bound_threshold() are in scalp_internal.cuh (the supervoxels
+// use them too).
 
 __device__ __forceinline__ unsigned long long pack_best(float D, int slot)
 {
@@ -530,16 +534,17 @@ __device__ __forceinline__ void assign_tile(const SolveArgs &a, int tile, int tx
         for (bool more = true; more;) {
             // the pixels' side of the bound
             float fL[PIX_PER_THREAD], fa[PIX_PER_THREAD], fb[PIX_PER_THREAD], thr[PIX_PER_THREAD];
-            const float X = (float)(px - x0), Y = (float)(py - y0);
+            const float X = (float)(px - x0);
+            float Y[PIX_PER_THREAD];
             {
                 T own[PIX_PER_THREAD];
                 load_own(own);
 #pragma unroll
                 for (int j = 0; j < PIX_PER_THREAD; ++j) {
                     const float4 v = sample_value(own[j]);
-                    const float Yj = Y + (float)(j * ROW_STEP);
+                    Y[j] = (float)(py - y0 + j * ROW_STEP);
                     thr[j] = a.prune ? bound_threshold(dprev[j], fmaf(a.lam, fmaf(v.x, v.x, fmaf(v.y, v.y, v.z * v.z)),
-                                                                      a.ms2 * fmaf(X, X, Yj * Yj)))
+                                                                      a.ms2 * fmaf(X, X, Y[j] * Y[j])))
                                      : __int_as_float(0x7fffffff);
                     fL[j] = -2.0f * a.lam * v.x;
                     fa[j] = -2.0f * a.lam * v.y;
@@ -576,7 +581,7 @@ __device__ __forceinline__ void assign_tile(const SolveArgs &a, int tile, int tx
                     // (a pixel of the rectangle lies in the image)
                     const bool in = inx && ((unsigned)r0.y & (1u << (py - y0 + j * ROW_STEP))) && slot[j] != c;
                     const float bound = fmaf(fL[j], ck.x, fmaf(fa[j], ck.y, fmaf(fb[j], ck.z,
-                                             fmaf(Y + (float)(j * ROW_STEP), __int_as_float(r0.w), base))));
+                                             fmaf(Y[j], __int_as_float(r0.w), base))));
                     const bool loses = bound > thr[j];
                     if (COUNT && in && loses) {
                         // a pair that cannot win is not walked (counted as the method's work)

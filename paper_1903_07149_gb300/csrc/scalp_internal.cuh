@@ -625,10 +625,12 @@ __device__ __forceinline__ float scalp_distance(float dcp, float sum_dc, float s
 constexpr float BOUND_SCALE = 1.0f - 1.0f / 131072.0f;
 
 // What f . g + K' must exceed for the pair to lose; NaN (no pair loses) for a
-// pixel without a pass-1 D, or with one near the end of the FP32 range.
+// pixel without a pass-1 D, or where D or P is near the end of the FP32 range.
+constexpr float BOUND_SLACK = 0x1p-100f;
 __device__ __forceinline__ float bound_threshold(float D, float P)
 {
-    return D < 1e30f ? fmaf(D, 1.0f + 1.0f / 1048576.0f, -BOUND_SCALE * P) : __int_as_float(0x7fffffff);
+    return D < 1e30f && P < 1e30f ? fmaf(D + BOUND_SLACK, 1.0f + 1.0f / 1048576.0f, -BOUND_SCALE * P)
+                                  : __int_as_float(0x7fffffff);
 }
 
 // ---------------------------------------------------------------------------

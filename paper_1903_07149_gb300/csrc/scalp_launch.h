@@ -78,8 +78,6 @@ void launch_batch_update(const BatchArgs &b, int total_clusters, int total_fill,
 // pairs per CTA; smem_bytes = assign_smem_bytes(a.map_cap, tile side).
 void launch_assign(const SolveArgs &a, int storage, size_t smem_bytes, cudaStream_t st, bool pdl = false);
 size_t assign_smem_bytes(int map_cap, int side);
-// Whether the assignment may prune with these sizes and weights.
-bool bound_valid(int H, int W, float lam, float ms2);
 // Distance-map pairs of an assignment CTA for a grid of `tiles` tiles.
 int assign_map_capacity(int device, int side, int tiles);
 // Whether a single image is cut into TILE_SIDE_SMALL tiles.

@@ -62,7 +62,6 @@ struct VoxArgs {
     int tpw_x, tpw_y, tpw_t;  // bound on the tiles one window spans, per axis
     long long tile_cap;
     int count_samples;
-    int prune;                // 1: skip pairs whose lower bound exceeds the voxel's pass-1 D
     const float4 *plane;      // (L, a, b, w) per voxel
     int *labels;
     long long *st_n, *st_sx, *st_sy, *st_st;
@@ -790,9 +789,8 @@ __global__ void __launch_bounds__(VTILE) k_vassign(VoxArgs a)
             float fL, fa, fb, thr;
             {
                 const float4 v = valid ? __ldg(a.plane + p) : make_float4(0.f, 0.f, 0.f, 0.f);
-                thr = a.prune ? bound_threshold(dprev, fmaf(a.lam, fmaf(v.x, v.x, fmaf(v.y, v.y, v.z * v.z)),
-                                                            a.ms2 * fmaf(X, X, fmaf(Y, Y, Z * Z))))
-                              : __int_as_float(0x7fffffff);
+                thr = bound_threshold(dprev, fmaf(a.lam, fmaf(v.x, v.x, fmaf(v.y, v.y, v.z * v.z)),
+                                                  a.ms2 * fmaf(X, X, fmaf(Y, Y, Z * Z))));
                 fL = -2.0f * a.lam * v.x;
                 fa = -2.0f * a.lam * v.y;
                 fb = -2.0f * a.lam * v.z;
@@ -1125,7 +1123,6 @@ int scalp_voxel_init(scalp_vctx **out, const scalp_volume *vol, int32_t K, float
     a.lam = params->lambda;
     a.gamma = (float)c->gamma;
     a.ms2 = (float)((double)m * (double)m / (c->r * c->r));
-    a.prune = bound_valid(c->H, c->W, a.lam, a.ms2) ? 1 : 0;
     a.n_tx = L.n_tx; a.n_ty = L.n_ty; a.n_tt = L.n_tt;
     a.tpw_x = L.tpw_x; a.tpw_y = L.tpw_y; a.tpw_t = L.tpw_t;
     a.tile_cap = L.tile_cap;
