@@ -97,8 +97,8 @@ struct QualityWs {
 };
 
 // The offsets at distance < eps, as half-widths: row offset dy takes the
-// columns within half[|dy|] (-1: none).  Up to QUALITY_RADIUS rows, the larger
-// radii test the distance itself.
+// columns within half[|dy|] (-1: none).  Up to QUALITY_RADIUS rows; for larger
+// radii k_quality_far tests the distance itself.
 constexpr int QUALITY_RADIUS = 15;
 struct Disk {
     int r;
@@ -122,10 +122,9 @@ struct Disk {
 // shuffles and ballots.
 constexpr int QUALITY_ROWS = 16, QUALITY_THREADS = 256, QUALITY_SLOTS = 256, QUALITY_PROBES = 8;
 
-template <bool FAR>
 __global__ void __launch_bounds__(QUALITY_THREADS)
-    k_quality_pixels(const int *__restrict__ lab, const int *__restrict__ gt, int n_gt, int H, int W, double eps,
-                     Disk disk, QualityWs w)
+    k_quality_pixels(const int *__restrict__ lab, const int *__restrict__ gt, int n_gt, int H, int W, Disk disk,
+                     QualityWs w)
 {
     constexpr int WARPS = QUALITY_THREADS / 32;
     __shared__ unsigned long long s_mask[WARPS][QUALITY_ROWS + 2 * QUALITY_RADIUS];
@@ -169,7 +168,7 @@ __global__ void __launch_bounds__(QUALITY_THREADS)
         // the warp's (superpixels) and of the two next to it (segments).
         // Places outside the image move to its edge, where a neighbour then
         // equals the pixel itself.
-        const int r = FAR ? 0 : disk.r, rows = y1 - y0 + 2 * r;
+        const int r = disk.r, rows = y1 - y0 + 2 * r;
         const bool valid = x < W, halo_valid = lane < 16 ? x >= 16 : x + 16 < W;
         const int xc = min(x, W - 1), xh = lane < 16 ? max(x - 16, 0) : min(x + 16, W - 1);
         const int xg = lane == 0 ? max(x - 1, 0) : lane == 31 ? min(x + 1, W - 1) : xc;
@@ -188,44 +187,23 @@ __global__ void __launch_bounds__(QUALITY_THREADS)
             if (lane == 0) l = h_lo;
             if (lane == 31) rt = h_hi;
             const int e4 = (l != at.c) + (rt != at.c) + (up.c != at.c) + (down.c != at.c);
-            if (!FAR) {
-                int hl = __shfl_up_sync(FULL, at.h, 1), hr = __shfl_down_sync(FULL, at.h, 1);
-                const int c_lo = __shfl_sync(FULL, at.c, 0), c_hi = __shfl_sync(FULL, at.c, 31);
-                if (lane == 16) hl = c_hi;
-                if (lane == 15) hr = c_lo;
-                // (bits 0 and 63 lack a neighbour; no disk reaches them)
-                const unsigned mc = __ballot_sync(FULL, in && valid && e4);
-                const unsigned mh = __ballot_sync(FULL, in && halo_valid && (hl != at.h || hr != at.h || up.h != at.h ||
-                                                                             down.h != at.h));
-                if (lane == 0)
-                    s_mask[warp][i] = (mh & 0xffffu) | (unsigned long long)mc << 16 | (unsigned long long)(mh >> 16) << 48;
-            }
+            int hl = __shfl_up_sync(FULL, at.h, 1), hr = __shfl_down_sync(FULL, at.h, 1);
+            const int c_lo = __shfl_sync(FULL, at.c, 0), c_hi = __shfl_sync(FULL, at.c, 31);
+            if (lane == 16) hl = c_hi;
+            if (lane == 15) hr = c_lo;
+            // (bits 0 and 63 lack a neighbour; no disk reaches them)
+            const unsigned mc = __ballot_sync(FULL, in && valid && e4);
+            const unsigned mh = __ballot_sync(FULL, in && halo_valid && (hl != at.h || hr != at.h || up.h != at.h ||
+                                                                         down.h != at.h));
+            if (lane == 0)
+                s_mask[warp][i] = (mh & 0xffffu) | (unsigned long long)mc << 16 | (unsigned long long)(mh >> 16) << 48;
             if (i < r || i >= rows - r) return;
             int gl = __shfl_up_sync(FULL, at.g, 1), gr = __shfl_down_sync(FULL, at.g, 1);
             if (lane == 0) gl = at.e;
             if (lane == 31) gr = at.e;
             const bool bnd_gt = valid && (gl != at.g || gr != at.g || up.g != at.g || down.g != at.g);
-            if (FAR) {
-                const auto far_at = [&](int qx, int qy) {
-                    return lab[(long long)min(max(qy, 0), H - 1) * W + min(max(qx, 0), W - 1)];
-                };
-                bool found = false;
-                if (bnd_gt)
-                    for (int dy = -disk.r; dy <= disk.r && !found; ++dy)
-                        for (int dx = -disk.r; dx <= disk.r && !found; ++dx) {
-                            const int qx = x + dx, qy = y + dy;
-                            if (qx < 0 || qy < 0 || qx >= W || qy >= H) continue;
-                            if (sqrt((double)dx * dx + (double)dy * dy) >= eps) continue;
-                            const int c = far_at(qx, qy);
-                            found = far_at(qx - 1, qy) != c || far_at(qx + 1, qy) != c || far_at(qx, qy - 1) != c ||
-                                    far_at(qx, qy + 1) != c;
-                        }
-                n_bnd += bnd_gt;
-                n_hit += found;
-            } else {
-                const unsigned G = __ballot_sync(FULL, bnd_gt);
-                if (lane == 0) s_gt[warp][i - r] = G;
-            }
+            const unsigned G = __ballot_sync(FULL, bnd_gt);
+            if (lane == 0) s_gt[warp][i - r] = G;
             const int e = e4 + (x == 0) + (x == W - 1) + (y == 0) + (y == H - 1);
             const int key = valid ? at.c * n_gt + at.g : -1;  // (n_labels * n_gt <= 2^28)
             if (key != run_key) {
@@ -255,24 +233,22 @@ __global__ void __launch_bounds__(QUALITY_THREADS)
 #pragma unroll
             for (int u = 0; u < B; ++u) now[u + 2] = next[u];
         }
-        if (!FAR) {
-            __syncwarp();
-            if (lane < y1 - y0) {
-                // row y0 + lane: the dilated boundary against the segments'
-                unsigned long long d = 0;
-                for (int dy = -r; dy <= r; ++dy) {
-                    const int h = disk.half[abs(dy)];
-                    if (h < 0) continue;
-                    const unsigned long long m = s_mask[warp][lane + r + dy];
-                    d |= m;
-                    for (int t = 1; t <= h; ++t) d |= m << t | m >> t;
-                }
-                const unsigned G = s_gt[warp][lane];
-                n_bnd = __popc(G);
-                n_hit = __popc(G & (unsigned)(d >> 16));
+        __syncwarp();
+        if (lane < y1 - y0) {
+            // row y0 + lane: the dilated boundary against the segments'
+            unsigned long long d = 0;
+            for (int dy = -r; dy <= r; ++dy) {
+                const int h = disk.half[abs(dy)];
+                if (h < 0) continue;
+                const unsigned long long m = s_mask[warp][lane + r + dy];
+                d |= m;
+                for (int t = 1; t <= h; ++t) d |= m << t | m >> t;
             }
-            __syncwarp();
+            const unsigned G = s_gt[warp][lane];
+            n_bnd = __popc(G);
+            n_hit = __popc(G & (unsigned)(d >> 16));
         }
+        __syncwarp();
     }
     // what is left, one hand-over per pair of the warp
     for (unsigned pending = __ballot_sync(FULL, run_key >= 0); pending;) {
@@ -298,6 +274,43 @@ __global__ void __launch_bounds__(QUALITY_THREADS)
     }
     if (threadIdx.x < 2 && s_count[threadIdx.x])
         atomicAdd(&w.counts[threadIdx.x], (unsigned long long)s_count[threadIdx.x]);
+}
+
+// Radii above QUALITY_RADIUS: the ground-truth boundary pixels found, a pixel per
+// thread, each searching its own disk row by row until it meets a boundary.
+// Bound by the search's loads.  (The warps of k_quality_pixels took their rows
+// one after the other, a search a lane, with a square root per offset: a call on
+// 1080 x 1920 at eps = 20 3.43 ms against 0.24; 321 x 481 with 4 superpixels at
+// eps = 40 63.5 against 1.43, and 9.4 a pixel per thread with the square roots.)
+__global__ void __launch_bounds__(256)
+    k_quality_far(const int *__restrict__ lab, const int *__restrict__ gt, int H, int W, int r, long long d2_max,
+                  QualityWs w)
+{
+    const long long N = (long long)H * W;
+    const auto boundary = [&](const int *__restrict__ l, int x, int y) {
+        const long long p = (long long)y * W + x;
+        const int c = l[p];
+        return (x > 0 && l[p - 1] != c) || (x < W - 1 && l[p + 1] != c) || (y > 0 && l[p - W] != c) ||
+               (y < H - 1 && l[p + W] != c);
+    };
+    unsigned hits = 0;
+    for (long long p = blockIdx.x * (long long)blockDim.x + threadIdx.x; p < N; p += (long long)gridDim.x * blockDim.x) {
+        const int y = (int)((unsigned)p / (unsigned)W), x = (int)p - y * W;  // N <= 2^30
+        if (!boundary(gt, x, y)) continue;
+        bool found = false;
+        for (int dy = max(-r, -y); dy <= min(r, H - 1 - y) && !found; ++dy) {
+            const long long left = d2_max - (long long)dy * dy;
+            if (left < 0) continue;
+            long long h = (long long)sqrt((double)left);  // (the disk's half-width here, exactly)
+            while (h * h > left) --h;
+            while ((h + 1) * (h + 1) <= left) ++h;
+            const int last = (int)min(h, (long long)(W - 1 - x));
+            for (int dx = -(int)min(h, (long long)x); dx <= last && !found; ++dx) found = boundary(lab, x + dx, y + dy);
+        }
+        hits += found;
+    }
+    hits = __reduce_add_sync(0xffffffffu, hits);
+    if ((threadIdx.x & 31) == 0 && hits) atomicAdd(&w.counts[1], (unsigned long long)hits);
 }
 
 // One warp per superpixel: its row of overlaps gives its size (their sum), the
@@ -475,17 +488,31 @@ extern "C" int scalp_quality_metrics(const int32_t *labels, int32_t n_labels, co
     cudaError_t e = cudaMemsetAsync(workspace, 0, need, st);
     const long long N = (long long)H * W;
     if (e == cudaSuccess) {
+        const int r = (int)std::min(std::ceil(eps), (double)std::max(H, W));
+        const bool far = r > QUALITY_RADIUS;
         Disk disk{};
-        disk.r = (int)std::min(std::ceil(eps), (double)std::max(H, W));
-        const bool far = disk.r > QUALITY_RADIUS;
+        disk.r = far ? 0 : r;  // (far: no offset, so that no pixel is found)
         for (int dy = 0; dy <= QUALITY_RADIUS; ++dy) {
             disk.half[dy] = -1;
-            for (int dx = 0; !far && dx <= disk.r && !(std::sqrt((double)(dx * dx + dy * dy)) >= eps); ++dx)
+            for (int dx = 0; !far && dx <= r && !(std::sqrt((double)(dx * dx + dy * dy)) >= eps); ++dx)
                 disk.half[dy] = (signed char)dx;
         }
         const unsigned blocks = (unsigned)((long long)((W + 63) / 64) * ((H + 63) / 64));
-        if (far) k_quality_pixels<true><<<blocks, QUALITY_THREADS, 0, st>>>(labels, gt, n_gt, H, W, eps, disk, w);
-        else k_quality_pixels<false><<<blocks, QUALITY_THREADS, 0, st>>>(labels, gt, n_gt, H, W, eps, disk, w);
+        k_quality_pixels<<<blocks, QUALITY_THREADS, 0, st>>>(labels, gt, n_gt, H, W, disk, w);
+        // the largest squared distance below eps (square roots are monotone)
+        long long d2_max = 2LL * r * r;
+        if (far && !(std::sqrt((double)d2_max) < eps)) {
+            long long lo = 0;  // (0 < eps)
+            for (long long hi = d2_max; hi - lo > 1;) {
+                const long long mid = lo + (hi - lo) / 2;
+                if (std::sqrt((double)mid) < eps) lo = mid;
+                else hi = mid;
+            }
+            d2_max = lo;
+        }
+        if (far)
+            k_quality_far<<<(unsigned)std::min<long long>((N + 255) / 256, 152 * 16), 256, 0, st>>>(labels, gt, H, W, r,
+                                                                                                    d2_max, w);
         pdl_launch(true, k_quality_rows, dim3((unsigned)((n_labels + 7) / 8)), dim3(256), 0, st, n_labels, n_gt, w);
         pdl_launch(true, k_quality_total, dim3(1), dim3(1024), 0, st, n_labels, N, w);
         e = cudaGetLastError();
