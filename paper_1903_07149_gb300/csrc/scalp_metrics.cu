@@ -381,7 +381,6 @@ size_t quality_layout(int n_labels, int n_gt, QualityWs *w, unsigned char *base)
         return base ? base + off : nullptr;
     };
     unsigned char *ov = take((size_t)n_labels * n_gt * sizeof(int));
-    unsigned char *area = take((size_t)n_labels * 8);
     unsigned char *perim = take((size_t)n_labels * 8);
     unsigned char *best = take((size_t)n_labels * 8);
     unsigned char *ue = take((size_t)n_labels * 8);
@@ -390,7 +389,6 @@ size_t quality_layout(int n_labels, int n_gt, QualityWs *w, unsigned char *base)
     unsigned char *result = take(4 * 8);
     if (w) {
         w->ov = reinterpret_cast<int *>(ov);
-        (void)area;  // (the sizes are the overlaps' sums)
         w->perim = reinterpret_cast<unsigned long long *>(perim);
         w->best = reinterpret_cast<long long *>(best);
         w->ue = reinterpret_cast<long long *>(ue);
