@@ -347,8 +347,11 @@ __global__ void __launch_bounds__(PRIOR_THREADS)
     else atomicMax(gmax, s_max);
 }
 
-// PRIOR_QUADS times four pixels of a row per thread; each four as one 16-byte
-// word where the rows start on 16 bytes (VEC).  PARTS: the maximum is that of
+// 4 * PRIOR_QUADS pixels per thread, each four of a row as one 16-byte word
+// where the rows start on 16 bytes (VEC; an output without gaps is one row), else
+// one by one, neighbours by neighbouring lanes (2160 x 3839 without gaps, a call
+// 89.1 -> 64.7 us, 1079 x 1919 29.7 -> 21.5; rows 3,841 apart 89.0 -> 69.8: a thread
+// took four neighbours in turn before).  PARTS: the maximum is that of
 // the gradient's n_parts CTAs, reduced here by every CTA while its pixels'
 // loads are in flight; otherwise it is gmax[0].  The reduction replaces clearing
 // and raising one word (a launch of its own before the gradient pass): 1080 x
@@ -365,17 +368,19 @@ __global__ void __launch_bounds__(PRIOR_THREADS)
 {
     __shared__ unsigned s_max[PRIOR_THREADS / 32];
     pdl_wait();  // every magnitude and the final maximum
-    const unsigned quads = (unsigned)(W + 3) / 4, total = quads * (unsigned)H;  // at most 2^30
-    float4 v[PRIOR_QUADS];
-    float *at[PRIOR_QUADS];
-    int left[PRIOR_QUADS];  // pixels from here to the row's end; 0: none here
+    constexpr int PIECES = VEC ? PRIOR_QUADS : 4 * PRIOR_QUADS, WIDTH = VEC ? 4 : 1;
+    const unsigned pieces = (unsigned)(W + WIDTH - 1) / WIDTH, total = pieces * (unsigned)H;  // at most 2^30
+    float4 v[PIECES];
+    float *at[PIECES];
+    int left[PIECES];  // pixels from here to the row's end; 0: none here
 #pragma unroll
-    for (int u = 0; u < PRIOR_QUADS; ++u) {
-        const unsigned i = (blockIdx.x * (unsigned)PRIOR_QUADS + u) * PRIOR_THREADS + threadIdx.x;
-        const unsigned y = i / quads, x = (i - y * quads) * 4;
+    for (int u = 0; u < PIECES; ++u) {
+        const unsigned i = (blockIdx.x * (unsigned)PIECES + u) * PRIOR_THREADS + threadIdx.x;
+        const unsigned y = i / pieces, x = (i - y * pieces) * WIDTH;
         left[u] = i < total ? W - (int)x : 0;
         at[u] = out + y * out_stride + x;
         if (VEC && left[u] >= 4) v[u] = *reinterpret_cast<const float4 *>(at[u]);
+        if (!VEC && left[u] > 0) v[u].x = *at[u];
     }
     unsigned bits;
     if (PARTS) {
@@ -392,11 +397,14 @@ __global__ void __launch_bounds__(PRIOR_THREADS)
     const float m = __uint_as_float(bits);
     const auto scaled = [&](float g) { return m > 0.0f ? g / m : 0.0f; };
 #pragma unroll
-    for (int u = 0; u < PRIOR_QUADS; ++u) {
-        if (VEC && left[u] >= 4)
+    for (int u = 0; u < PIECES; ++u) {
+        if (!VEC) {
+            if (left[u] > 0) *at[u] = scaled(v[u].x);
+        } else if (left[u] >= 4) {
             *reinterpret_cast<float4 *>(at[u]) = make_float4(scaled(v[u].x), scaled(v[u].y), scaled(v[u].z), scaled(v[u].w));
-        else
-            for (int k = 0; k < min(left[u], 4); ++k) at[u][k] = scaled(at[u][k]);
+        } else {
+            for (int k = 0; k < left[u]; ++k) at[u][k] = scaled(at[u][k]);
+        }
     }
 }
 
@@ -418,11 +426,16 @@ void launch_gradient_prior(const uint8_t *rgb, long long rgb_stride, int H, int 
     const dim3 grid((unsigned)ceil_div_ll(W, PRIOR_TX), (unsigned)ceil_div_ll(H, PRIOR_TY));
     pdl_launch(false, k_prior_gradient, grid, dim3(PRIOR_THREADS), 0, st, rgb, rgb_stride, H, W, lut,
                out, out_stride, gmax, parts ? 1 : 0);
-    const bool vec = reinterpret_cast<uintptr_t>(out) % 16 == 0 && out_stride % 4 == 0;
+    if (out_stride == W) {  // (H * W <= 2^30)
+        W *= H;
+        H = 1;
+        out_stride = W;
+    }
+    const bool vec = reinterpret_cast<uintptr_t>(out) % 16 == 0 && (H == 1 || out_stride % 4 == 0);
     const auto normalise = vec ? (parts ? k_prior_normalise<true, true> : k_prior_normalise<true, false>)
                                : (parts ? k_prior_normalise<false, true> : k_prior_normalise<false, false>);
-    pdl_launch(true, normalise,
-               dim3((unsigned)ceil_div_ll((long long)((W + 3) / 4) * H, PRIOR_QUADS * PRIOR_THREADS)),
+    const long long pieces = (vec ? (W + 3LL) / 4 : W) * H, per_cta = PRIOR_QUADS * PRIOR_THREADS * (vec ? 1 : 4);
+    pdl_launch(true, normalise, dim3((unsigned)ceil_div_ll(pieces, per_cta)),
                dim3(PRIOR_THREADS), 0, st, out, out_stride, H, W, (const unsigned *)gmax,
                (int)(grid.x * grid.y));
 }
