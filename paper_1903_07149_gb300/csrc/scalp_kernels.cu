@@ -358,9 +358,12 @@ __global__ void __launch_bounds__(PRIOR_THREADS)
 // 1920, calls in a row 22.4 -> 20.8 us on the device, their issue by the host
 // 21 -> 18.5.
 constexpr int PRIOR_QUADS = 2;
-// (2,040 words a CTA on 1080 x 1920; beyond this many the reading costs more
-// than the cleared word)
-constexpr long long PRIOR_PARTS_MAX = 8192;
+// Every CTA reads all of them, so beyond some 2,600 tiles one cleared word is the
+// better form.  Calls in a row on the device, a word per tile against one: 176
+// tiles 8.3 and 10.3 us, 920 14.4 and 14.4, 2,040 21.7 and 22.4, 2,752 26.7 and
+// 26.7, 3,600 32.9 and 31.8, 8,160 (2160 x 3840) 64.4 and 59.5, 9,375 74.0 and
+// 67.7.
+constexpr long long PRIOR_PARTS_MAX = 2560;
 
 template <bool VEC, bool PARTS>
 __global__ void __launch_bounds__(PRIOR_THREADS)

@@ -37,3 +37,27 @@ def test_rows_and_gaps(H, W):
     S.gradient_prior(rgb, out=flat[1:1 + H * W].view(H, W))
     assert np.array_equal(flat[1:1 + H * W].view(H, W).cpu().numpy(), want)
     assert float(flat[0]) == -1.0 and bool((flat[1 + H * W:] == -1.0).all())
+
+
+# up to 2,560 tiles of 32 x 32 take a maximum each where the workspace has the
+# room (2,550, 2,560 and 2,600 here): the bits of the one cleared word
+@pytest.mark.parametrize("H,W", [(1600, 1632), (1280, 2048), (1280, 2049)])
+def test_maximum_per_tile(H, W):
+    import ctypes
+
+    import torch
+
+    scalp_build.build()
+    from paper_1903_07149_gb300 import scalp as S
+
+    gen = torch.Generator(device="cuda").manual_seed(W)
+    rgb = torch.randint(0, 256, (H, W, 3), generator=gen, dtype=torch.uint8, device="cuda")
+    a = S.gradient_prior(rgb)
+    L = S.load()
+    nbytes = L.scalp_gradient_prior_workspace_bytes(H, W, 1, 1)
+    ws = torch.empty(nbytes, dtype=torch.uint8, device="cuda")
+    b = torch.empty((H, W), device="cuda")
+    img = S.scalp_image(H, W, rgb.data_ptr(), 0, 1)
+    rc = L.scalp_gradient_prior(ctypes.byref(img), b.data_ptr(), W, 1, torch.cuda.current_stream().cuda_stream,
+                                ws.data_ptr(), nbytes)
+    assert rc == S.SCALP_OK and torch.equal(a, b) and float(a.max()) == 1.0
