@@ -134,9 +134,13 @@ __device__ __forceinline__ ProjBest proj_candidate(long long p, int x, int y, lo
 // divisions and four window searches come one after the other (8.4 and 8.6
 // us a launch for 60 and 2000 clusters, 5.4 and 6.5 on eight lanes).  Above
 // it the chip is full and the extra warps only cost (120,000 clusters of a
-// batch: 39.6 us on one thread each, 84.6 on eight lanes).
+// batch: 39.6 us on one thread each, 84.6 on eight lanes).  An iteration of
+// 1080 x 1920 by lanes and by threads: 2,040 clusters 100.1 and 101.0 us, 11,972
+// 101.3 and 103.0, 16,055 106.8 and 108.8, 24,012 114.2 and 114.2, 32,026 121.4
+// and 118.8, 64,030 162.0 and 156.4; of two images half as high 24,012 129.3 and
+// 132.0, 32,026 139.3 and 138.3.
 // ---------------------------------------------------------------------------
-constexpr int UPDATE_LANES = 8, UPDATE_LANES_MAX = 32768;
+constexpr int UPDATE_LANES = 8, UPDATE_LANES_MAX = 24576;
 
 // One thread per cluster.
 __device__ __forceinline__ void update_cluster(const SolveArgs &a, int k, int from_acc)
