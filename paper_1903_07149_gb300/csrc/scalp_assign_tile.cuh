@@ -240,7 +240,7 @@ __device__ __forceinline__ void assign_tile(const SolveArgs &a, int tile, int tx
     };
 
     const int off = a.tile_off[tile];
-    // the list capacity is a proven bound; the clamp only guards memory if the
+    // the list capacity is a proven bound; the held_lamp only guards memory if the
     // device-side overflow check (reported as an error) ever fired
     const int cnt = (int)max(0LL, min((long long)a.tile_off[tile + 1], a.tile_cap) - off);
     const bool fast = cnt <= MAX_TILE_CANDIDATES;
@@ -333,7 +333,7 @@ __device__ __forceinline__ void assign_tile(const SolveArgs &a, int tile, int tx
             size = min(bw, 0xffff) | (min(bh, 0xffff) << 16);
         }
         box[rank] = make_int4(bx0, by0, pitch, size);
-        // a box larger than the whole buffer never fits: clamp it so that the
+        // a box larger than the whole buffer never fits: held_lamp it so that the
         // prefix sums stay small
         area[rank] = map_cap > 0 ? (int)min(n, (long long)map_cap + 1) : 0;
     };
@@ -616,25 +616,36 @@ __device__ __forceinline__ void assign_tile(const SolveArgs &a, int tile, int tx
             }
         }
     } else {
-        // per-pixel path: every candidate straight from the global list
+        // per-pixel path: every candidate straight from the global list.  The
+        // pointers in registers: from the batch's shared memory in each round,
+        // 40 small images with step 3 took 8.88 ms per five iterations, 8.43
+        // so.  FP16 planes hold the weights as well (or the hot path above is
+        // allocated worse: 12 served images 7.21 ms, 7.05 so); with FP32 it is
+        // the other way round (batch of 64 28.6 ms, 28.1 so).
+        const int *list = a.tile_list + off;
+        const ClusterDev *cdev = a.cdev;
+        constexpr bool HOLD = sizeof(T) == 8;
+        const int held_pitch = a.pitch;
+        const float held_lam = a.lam, held_gamma = a.gamma, held_ms2 = a.ms2;
 #pragma unroll 1
         for (int j = 0; j < PIX_PER_THREAD; ++j) {
             int px, py;
             my_pixel(j, px, py);
             if (px >= a.W || py >= a.H) continue;
-            const float4 own = fetch_sample<T>(plane + (long long)py * a.pitch + px);
+            const float4 own = fetch_sample<T>(plane + (long long)py * (HOLD ? held_pitch : a.pitch) + px);
             float bestD = FLT_MAX;
             for (int i = 0; i < cnt; ++i) {
-                const int k = a.tile_list[off + i];
-                const ClusterDev cd = a.cdev[k];
+                const int k = list[i];
+                const ClusterDev cd = cdev[k];
                 if (px < cd.xlo || px > cd.xhi || py < cd.ylo || py > cd.yhi) continue;
                 const PathSetup s = path_setup(px, py, cd.ex, cd.ey);
                 float sdc, sw;
-                const int len = path_sums<T>(plane, a.pitch, 0, 0, s, cd.L, cd.a, cd.b, sdc, sw);
+                const int len = path_sums<T>(plane, HOLD ? held_pitch : a.pitch, 0, 0, s, cd.L, cd.a, cd.b, sdc, sw);
                 const float dcp = colour_dist(own, cd.L, cd.a, cd.b);
                 const float ddx = (float)px - cd.xk, ddy = (float)py - cd.yk;
                 const float ds = fmaf(ddx, ddx, ddy * ddy);
-                const float D = scalp_distance(dcp, sdc, sw, len, a.lam, a.gamma, a.ms2, ds);
+                const float D = scalp_distance(dcp, sdc, sw, len, HOLD ? held_lam : a.lam,
+                                               HOLD ? held_gamma : a.gamma, HOLD ? held_ms2 : a.ms2, ds);
                 if (D < bestD || (D == bestD && k < bestk[j])) {
                     bestD = D;
                     bestk[j] = k;
