@@ -1310,7 +1310,7 @@ int scalp_batch_init(scalp_batch **out, int32_t count, const scalp_image *images
         p.workspace_bytes = scalp_workspace_bytes(Hs[i], Ws[i], K[i], params);
         off += (p.workspace_bytes + ALIGN - 1) & ~(ALIGN - 1);
         scalp_ctx *c = nullptr;
-        const int rc = init_ctx(&c, &images[i], contours ? &contours[i] : nullptr, K[i], m[i], &p, true, false);
+        const int rc = init_ctx(&c, &images[i], contours ? &contours[i] : nullptr, K[i], m[i], &p, true, count == 1);
         if (rc != SCALP_OK) {
             char msg[512];
             snprintf(msg, sizeof msg, "image %d: %s", i, g_last_error.c_str());
@@ -1403,8 +1403,9 @@ int scalp_batch_init(scalp_batch **out, int32_t count, const scalp_image *images
         return batch_fail(SCALP_E_CUDA, "batch set-up: %s", cudaGetErrorString(e));
     }
     // the set-up of all images as the flat launches of a reload (image by
-    // image, five launches each, it took 350 us for 12 images of 321 x 481)
-    int rc = scalp_batch_reload(b, images, contours);
+    // image, five launches each, it took 350 us for 12 images of 321 x 481);
+    // a single image's own launches have been made
+    int rc = count == 1 ? SCALP_OK : scalp_batch_reload(b, images, contours);
     if (rc == SCALP_OK) {
         // the host vectors copied above go out of scope, and host inputs are released
         e = cudaStreamSynchronize(b->st);
