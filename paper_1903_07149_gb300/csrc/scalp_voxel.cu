@@ -62,6 +62,7 @@ struct VoxArgs {
     int tpw_x, tpw_y, tpw_t;  // bound on the tiles one window spans, per axis
     long long tile_cap;
     int count_samples;
+    int thin_w, thin_h, thin_d;  // voxels of a tile along each axis, where the volume is thinner than it
     const float4 *plane;      // (L, a, b, w) per voxel
     int *labels;
     long long *st_n, *st_sx, *st_sy, *st_st;
@@ -117,7 +118,7 @@ __device__ __forceinline__ int vwindow_end(long long n, long long s, long long N
 
 // ---------------------------------------------------------------------------
 // Integer sums of (1, x, y, t, L, a, b) per label; colour fixed point
-// 2^COLOR_FRAC_BITS.  A warp's 32 voxels share a frame and lie within 32
+// 2^COLOR_FRAC_BITS.  A warp's 32 voxels lie in one tile, or share a frame and lie within 32
 // columns and 2 rows of a base, so the three offsets pack into one 32-bit
 // warp sum (10 bits each).
 // ---------------------------------------------------------------------------
@@ -669,6 +670,20 @@ __device__ __forceinline__ int vfind_slot(const int *ids, int cnt, int k)
 //   s_rec = (box, K bits, g_x bits, g_y bits), s_col = (c, g_t)
 // with the box as one bit per column (0-15), row (16-23) and frame (24-27) of
 // the tile.
+//
+// THIN: a volume of fewer than sixteen columns, or of one row, fills the lanes
+// of that layout poorly (and most warps not at all).  The tile's voxels (a.thin_w
+// x a.thin_h x a.thin_d, x fastest) are packed into the first warps' lanes then,
+// the CTA has no more warps than it can use, and up to half a tile's voxels the
+// warps form groups: every group takes the voxels, group g checks the slots = g
+// modulo the number of groups against the first group's pass-1 D's, and they
+// meet in the voxels' best D.  Six iterations, packed and in the layout above:
+// 300 x 700 x 1 with 40 clusters 427 and 1688 us, x 7 1.61 and 2.02 ms (with 300
+// clusters), 300 x 300 x 9 684 and 962 us, x 15 1032 and 1139; 2000 x 1 x 600
+// 1.30 and 4.95 ms; a line of 60,000 347-814 and 799-2501 us.  Few frames or a
+// few rows fill the layout's warps one by one and stay with it (2 x 400 x 600
+// 413 us).
+template <bool THIN>
 __global__ void __launch_bounds__(VTILE) k_vassign(VoxArgs a)
 {
     static_assert(VTX == 16 && VTY == 8 && VTT == 4, "a box is 16 + 8 + 4 bits, a warp 16 x 2 voxels");
@@ -686,9 +701,21 @@ __global__ void __launch_bounds__(VTILE) k_vassign(VoxArgs a)
     const int tx = tile % a.n_tx, ty = (tile / a.n_tx) % a.n_ty, tt = tile / (a.n_tx * a.n_ty);
     const int x0 = tx * VTX, y0 = ty * VTY, t0 = tt * VTT;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int lx = tid % VTX, ly = (tid / VTX) % VTY, lt = tid / (VTX * VTY);
+    const int blocks = THIN ? (a.thin_w * a.thin_h * a.thin_d + 31) >> 5 : VTILE / 32;  // of 32 voxels
+    const int groups = THIN ? (int)(blockDim.x >> 5) / blocks : 1, group = THIN ? warp / blocks : 0;
+    const int base = THIN ? warp % blocks * 32 : warp * 32;  // of the warp's voxels in the tile
+    // place in the tile of its voxel v
+    const auto place = [&](int v, int &vx, int &vy, int &vt) {
+        const int row = THIN ? v / a.thin_w : v / VTX;
+        vx = THIN ? v - row * a.thin_w : v % VTX;
+        vt = THIN ? row / a.thin_h : row / VTY;
+        vy = THIN ? row - vt * a.thin_h : row % VTY;
+    };
+    int lx, ly, lt;
+    place(base + lane, lx, ly, lt);
     const int x = x0 + lx, y = y0 + ly, t = t0 + lt;
-    const bool valid = x < a.W && y < a.H && t < a.T;
+    const bool inside = x < a.W && y < a.H && t < a.T && (!THIN || (lt < a.thin_d && group < groups));
+    const bool valid = inside && group == 0;  // (the voxel's own thread)
     const int off = a.tile_off[tile];
     const int cnt = (int)max(0LL, min((long long)a.tile_off[tile + 1], a.tile_cap) - off);
     const bool fast = cnt <= VCAND;
@@ -754,11 +781,17 @@ __global__ void __launch_bounds__(VTILE) k_vassign(VoxArgs a)
         const int wy = y0 + (ly & ~1);  // the warp's first row
         const auto evaluate = [&](int v, int c, int &len) {
             const VoxCluster &cd = cand[c];
-            const int qx = x0 + (v & 15), qy = wy + (v >> 4);
-            const float dcp = colour_dist(__ldg(a.plane + ((long long)t * a.H + qy) * a.W + qx), cd.L, cd.a, cd.b);
+            int qx = x0 + (v & 15), qy = wy + (v >> 4), qt = t;
+            if (THIN) {
+                place(base + v, qx, qy, qt);
+                qx += x0;
+                qy += y0;
+                qt += t0;
+            }
+            const float dcp = colour_dist(__ldg(a.plane + ((long long)qt * a.H + qy) * a.W + qx), cd.L, cd.a, cd.b);
             float sdc, sw;
-            len = vpath_sums(a.plane, a.W, a.HW, qx, qy, t, cd.ex, cd.ey, cd.et, cd.L, cd.a, cd.b, sdc, sw);
-            const float ddx = (float)qx - cd.xk, ddy = (float)qy - cd.yk, ddt = (float)t - cd.tk;
+            len = vpath_sums(a.plane, a.W, a.HW, qx, qy, qt, cd.ex, cd.ey, cd.et, cd.L, cd.a, cd.b, sdc, sw);
+            const float ddx = (float)qx - cd.xk, ddy = (float)qy - cd.yk, ddt = (float)qt - cd.tk;
             return scalp_distance(dcp, sdc, sw, len, a.lam, a.gamma, a.ms2, fmaf(ddx, ddx, fmaf(ddy, ddy, ddt * ddt)));
         };
         const auto count_pair = [&](int len) {
@@ -766,7 +799,8 @@ __global__ void __launch_bounds__(VTILE) k_vassign(VoxArgs a)
             my_pairs += 1;
         };
         // pass 1: the previous label, when the voxel is in its box
-        const unsigned bits = 1u << lx | 1u << (16 + ly) | 1u << (24 + lt);
+        // (a lane without a voxel has no bits, and is in no box)
+        const unsigned bits = THIN && !inside ? 0u : 1u << lx | 1u << (16 + ly) | 1u << (24 + lt);
         int slot = prev >= 0 ? vfind_slot(s_sorted, cnt, prev) : -1;
         if (slot >= 0 && ((unsigned)s_rec[slot].x & bits) != bits) slot = -1;
         float dprev = __int_as_float(0x7fffffff);  // NaN: none
@@ -777,18 +811,29 @@ __global__ void __launch_bounds__(VTILE) k_vassign(VoxArgs a)
             mine = vpack_best(dprev, slot);
             count_pair(len);
         }
-        s_best[tid] = mine;
-        __syncwarp();
+        if (group == 0) s_best[base + lane] = mine;
+        if (THIN) {
+            __syncthreads();
+            if (group > 0 && inside) {  // (the first group's pass 1; ~0: a NaN, and no slot)
+                mine = s_best[base + lane];
+                dprev = __uint_as_float((unsigned)(mine >> 32));
+                slot = (int)(unsigned)mine;
+            }
+            __syncthreads();  // the D's before any group lowers them
+        } else {
+            __syncwarp();
+        }
         // pass 2: the other candidates
         uint16_t *wq = s_queue[warp];
         const unsigned warp_rows = 3u << (16 + (ly & ~1)), warp_frame = 1u << (24 + lt);
+        const unsigned warp_bits = THIN ? __reduce_or_sync(FULL, bits) : 0u;
         int queued = 0, c0 = -32;  // warp-uniform, as all that follows
         unsigned any = 0u;         // candidates c0 + bit that meet the warp's voxels and are left
         for (bool more = true; more;) {
             const float X = (float)lx, Y = (float)ly, Z = (float)lt;
             float fL, fa, fb, thr;
             {
-                const float4 v = valid ? __ldg(a.plane + p) : make_float4(0.f, 0.f, 0.f, 0.f);
+                const float4 v = inside ? __ldg(a.plane + p) : make_float4(0.f, 0.f, 0.f, 0.f);
                 thr = bound_threshold(dprev, fmaf(a.lam, fmaf(v.x, v.x, fmaf(v.y, v.y, v.z * v.z)),
                                                   a.ms2 * fmaf(X, X, fmaf(Y, Y, Z * Z))));
                 fL = -2.0f * a.lam * v.x;
@@ -802,7 +847,13 @@ __global__ void __launch_bounds__(VTILE) k_vassign(VoxArgs a)
                     more = c0 < cnt;
                     if (!more) break;
                     const unsigned m = c0 + lane < cnt ? (unsigned)s_rec[c0 + lane].x : 0u;
-                    any = __ballot_sync(FULL, (m & warp_rows) && (m & warp_frame));
+                    if (THIN) {
+                        const unsigned meet = m & warp_bits;
+                        any = __ballot_sync(FULL, (meet & 0xffffu) && (meet & 0xff0000u) && (meet & 0xf000000u) &&
+                                                      (c0 + lane) % groups == group);
+                    } else {
+                        any = __ballot_sync(FULL, (m & warp_rows) && (m & warp_frame));
+                    }
                     continue;
                 }
                 const int c = c0 + __ffs(any) - 1;
@@ -810,7 +861,7 @@ __global__ void __launch_bounds__(VTILE) k_vassign(VoxArgs a)
                 const int4 r = s_rec[c];
                 const float4 ck = s_col[c];
                 // (a voxel of the box lies in the volume)
-                const bool in = ((unsigned)r.x & bits) == bits && c != slot;
+                const bool in = ((unsigned)r.x & bits) == bits && c != slot && (!THIN || bits);
                 const float bound =
                     fmaf(fL, ck.x, fmaf(fa, ck.y, fmaf(fb, ck.z, fmaf(X, __int_as_float(r.z),
                                         fmaf(Y, __int_as_float(r.w), fmaf(Z, ck.w, __int_as_float(r.y)))))));
@@ -833,7 +884,7 @@ __global__ void __launch_bounds__(VTILE) k_vassign(VoxArgs a)
                 const int e = wq[done + lane], v = e & 31, c = e >> 5;
                 int len;
                 const float D = evaluate(v, c, len);
-                atomicMin(&s_best[warp * 32 + v], vpack_best(D, c));
+                atomicMin(&s_best[base + v], vpack_best(D, c));
                 count_pair(len);
             }
             if (more) {  // the pairs left over start the next queue
@@ -844,9 +895,10 @@ __global__ void __launch_bounds__(VTILE) k_vassign(VoxArgs a)
                 __syncwarp();
             }
         }
-        __syncwarp();
+        if (THIN) __syncthreads();
+        else __syncwarp();
         if (valid) {
-            const unsigned long long bb = s_best[tid];
+            const unsigned long long bb = s_best[base + lane];
             // slot -> cluster index (the record's pad field holds k)
             if (bb != ~0ull) lab = cand[(int)(bb & 0xffffffffu)].pad;
         }
@@ -883,10 +935,10 @@ __global__ void __launch_bounds__(VTILE) k_vassign(VoxArgs a)
             a.orphan_list[atomicAdd(&a.ctr->orphans, 1)] = (int)p;
         }
     }
-    // a warp = 32 voxels of one frame: 16 columns x 2 rows
+    // a warp = 32 voxels of one frame: 16 columns x 2 rows (THIN: any of the tile)
     const float4 own = valid ? __ldg(a.plane + p) : make_float4(0.f, 0.f, 0.f, 0.f);
-    const int bx = x0, by = y0 + (ly & ~1), bt = t;
-    vaggregate(a, valid, lab, bx, by, bt, lx, ly & 1, 0, own);
+    if (THIN) vaggregate(a, valid, lab, x0, y0, t0, lx, ly, lt, own);
+    else vaggregate(a, valid, lab, x0, y0 + (ly & ~1), t, lx, ly & 1, 0, own);
     if (a.count_samples) {
         for (int o = 16; o > 0; o >>= 1) {
             my_samples += __shfl_down_sync(0xffffffffu, my_samples, o);
@@ -1004,6 +1056,7 @@ struct scalp_vctx {
     unsigned char *ws;
     VLayout L;
     VoxArgs a;
+    int thin_threads;  // of an assignment CTA that packs its tile (0: a voxel per thread)
     int iterations;
     // profiling: an event pair around each assignment launch
     bool profiling = false;
@@ -1126,6 +1179,16 @@ int scalp_voxel_init(scalp_vctx **out, const scalp_volume *vol, int32_t K, float
     a.n_tx = L.n_tx; a.n_ty = L.n_ty; a.n_tt = L.n_tt;
     a.tpw_x = L.tpw_x; a.tpw_y = L.tpw_y; a.tpw_t = L.tpw_t;
     a.tile_cap = L.tile_cap;
+    a.thin_w = std::min(c->W, VTX);
+    a.thin_h = std::min(c->H, VTY);
+    a.thin_d = std::min(c->T, VTT);
+    // a voxel per thread, or two groups of warps up to half a tile; the sorting
+    // of a tile's candidates takes a thread each (VCAND)
+    const int thin = a.thin_w * a.thin_h * a.thin_d, thin_blocks = (thin + 31) / 32;
+    c->thin_threads = a.thin_w == VTX && a.thin_h > 1
+                          ? 0
+                          : std::max(VCAND, thin_blocks * (thin <= VTILE / 2 ? 64 : 32));
+    static_assert(VCAND % 32 == 0, "whole warps");
     a.plane = reinterpret_cast<const float4 *>(c->ws + L.plane);
     a.labels = reinterpret_cast<int *>(c->ws + L.labels);
     a.st_n = reinterpret_cast<long long *>(c->ws + L.st_n);
@@ -1197,7 +1260,8 @@ int scalp_voxel_iterate(scalp_vctx *c, int32_t n)
             }
             cudaEventRecord(c->ev[2 * c->ev_pending], c->st);
         }
-        pdl_launch(!prof, k_vassign, dim3(tiles), dim3(VTILE), 0, c->st, c->a);
+        pdl_launch(!prof, c->thin_threads ? k_vassign<true> : k_vassign<false>, dim3(tiles),
+                   dim3(c->thin_threads ? c->thin_threads : VTILE), 0, c->st, c->a);
         if (prof) cudaEventRecord(c->ev[2 * c->ev_pending++ + 1], c->st);
         venqueue_update(c, 1, 0);
         ++c->iterations;
