@@ -355,7 +355,7 @@ __global__ void __launch_bounds__(PRIOR_THREADS)
 // the gradient's n_parts CTAs, reduced here by every CTA while its pixels'
 // loads are in flight; otherwise it is gmax[0].  The reduction replaces clearing
 // and raising one word (a launch of its own before the gradient pass): 1080 x
-// 1920, calls in a row 22.4 -> 20.8 us on the device, their issue by the host
+// 1920, calls in a row 22.4 -> 21.7 us on the device, their issue by the host
 // 21 -> 18.5.
 constexpr int PRIOR_QUADS = 2;
 // Every CTA reads all of them, so beyond some 2,600 tiles one cleared word is the

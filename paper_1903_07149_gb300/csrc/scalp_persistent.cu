@@ -9,8 +9,9 @@
 //      scalp_assign_tile.cuh), with the update's fused partial sums;
 //   2. update of every cluster of every image, one thread each;
 //   3. the scan of each image's tile counts (one CTA per image) and the
-//      projection (Eq. 4) of each image's queued clusters (one CTA per queued
-//      cluster, spread over the grid);
+//      projection (Eq. 4) of each image's queued clusters (a warp per cluster,
+//      spread over the grid; a CTA per cluster for images with many pixels in
+//      no window);
 //   4. the candidate lists: every (cluster, tile) slot of every image.
 // The phases run the same device bodies in the same order of effects as the
 // per-kernel launches (the sums are integers, so the order in which tiles

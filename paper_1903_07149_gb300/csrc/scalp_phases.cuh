@@ -293,8 +293,8 @@ __device__ __forceinline__ void update_cluster_lanes(const SolveArgs &a, int k, 
     cd.ex = e.x; cd.ey = e.y;
     cd.pad = k;
     if (ok) {
-        // the window's tiles, one per lane in turn (one division for the
-        // lane's first, then steps of UPDATE_LANES)
+        // the window's tiles, one per lane in turn (a window seldom has more
+        // than one or two per lane)
         const int tx0 = cd.xlo >> a.tile_shift, ty0 = cd.ylo >> a.tile_shift;
         const int nx = (cd.xhi >> a.tile_shift) - tx0 + 1, nt = nx * ((cd.yhi >> a.tile_shift) - ty0 + 1);
         for (int t = j; t < nt; t += UPDATE_LANES)

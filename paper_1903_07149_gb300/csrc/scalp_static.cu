@@ -67,8 +67,9 @@ __global__ void k_static_table(StaticScratch *s)
 // memory once; a run that finds no place in the table adds its own.  Sums of
 // the labels of every 32-pixel row segment instead (warp reductions and six
 // atomics per label and row) took 27.8 us on 1080 x 1920 with 2000 labels, the
-// table 22.9 us (both with the inputs in DRAM); the conversion of the pixels is
-// most of what is left.
+// table 22.9 us (both with the inputs in DRAM).  What is left is the latency of
+// the row steps and of the table's additions: converting two pixels at a time
+// with packed instructions changed nothing (23.1).
 constexpr int SUM_ROWS = 8, SUM_THREADS = 256, SUM_SLOTS = 256, SUM_PROBES = 8, SUM_BATCH = 4;
 constexpr int SUM_CTA_ROWS = SUM_THREADS / 64 * SUM_ROWS;
 static_assert(SUM_ROWS * 108LL * (1LL << COLOR_FRAC_BITS) < (1LL << 31), "a run's colour sums");
