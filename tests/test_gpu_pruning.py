@@ -84,10 +84,13 @@ def test_work(S, m, lam, shape):
     for prune in (True, False):
         seg = S.Segmenter(rgb, con, 2000, m=m, lam=lam, prune=prune)
         seg.iterate(2)
-        seg.profile(1)
-        seg.iterate(3)
-        t, launches = seg.profile(0)
-        ms.append(t / launches)
+        best = float("inf")
+        for _ in range(4):
+            seg.profile(1)
+            seg.iterate(3)
+            t, launches = seg.profile(0)
+            best = min(best, t / launches)
+        ms.append(best)
         seg.close()
     assert ms[0] < 0.95 * ms[1], ms
 
